@@ -97,6 +97,7 @@ enum { CCZ4_PREC_FP64 = 0, CCZ4_PREC_MIXED = 1 };
    ACC: RK accumulator. RHS: output of ccz4_rhs. INI: Q_ini of the
    Sommerfeld condition (ghost part only is used). TILE: halo tiles. The
    state-shaped buffers (U, Y0, Y1, ACC, RHS, INI) share one layout.
+   ccz4_rhs and the step calls use TILE and MIX as scratch.
    MIX: [33][n_points] mixed second derivatives written by ccz4_fill_halos
    with the tiles: for g~_xx..g~_zz (slots 0..17), alpha (18..20),
    beta^x..beta^z (21..29) and phi (30..32), three slots each in the order
@@ -231,8 +232,9 @@ ccz4_status ccz4_rk_stage(ccz4_grid *g, const ccz4_params *P, int stage, double 
 /* Input and output buffers (CCZ4_BUF_*) of RK stage s = 0..3. */
 ccz4_status ccz4_stage_buffers(int stage, int *in_buf, int *out_buf);
 
-/* n_steps full RK4 steps on U: for each stage, ccz4_fill_halos of the
-   stage input followed by ccz4_rk_stage. */
+/* n_steps full RK4 steps on U: for each stage what ccz4_fill_halos_for of
+   the stage input followed by ccz4_rk_stage computes, without the tiles in
+   between. */
 ccz4_status ccz4_step(ccz4_grid *g, const ccz4_params *P, double dt, int n_steps, void *stream);
 
 /* n_steps RK4 steps on U, like ccz4_step, replayed from a CUDA graph of one
@@ -542,19 +544,16 @@ ccz4_status ccz4_tracers_step(ccz4_tracers *t, int buf, double dt, void *stream)
 ccz4_status ccz4_tracers_read(ccz4_tracers *t, double *pos, double *values, void *stream);
 ccz4_status ccz4_tracers_free(ccz4_tracers *t);
 
-/* Launch shapes (a tuning choice; results are identical, but for SPLIT in
-   the mixed precision, whose FP32 algebra may round a few intermediate
-   values differently, within 1e-8 of a field's largest value): the flat stage
+/* Launch shapes (a tuning choice; results are identical): the flat algebra
    kernel asks the default number of resident 128-thread blocks per SM
-   (CCZ4_STAGE_SHAPE_DEFAULT: 4 in FP64, 3 in the mixed precision), one
-   more (MORE_BLOCKS, fewer registers per thread) or one fewer
-   (FEWER_BLOCKS, more registers), or, for the mixed precision (FP64 keeps
-   its default), two phases in one launch (SPLIT: every thread first takes
-   all the stencil values of its point into its own shared-memory slots,
-   then evaluates the algebra and the update from them); the halo fill runs 256 threads per
-   patch with 8 independent loads per thread in its gather (DEFAULT), 512
-   threads (WIDE), 16 loads (DEEP) or 128 threads (NARROW). Drops a
-   captured step graph. CCZ4_ERR_INVALID for an unknown shape. */
+   (CCZ4_STAGE_SHAPE_DEFAULT), one more (MORE_BLOCKS, fewer registers per
+   thread) or one fewer (FEWER_BLOCKS, more registers); SPLIT, the stencil
+   values of a point before its algebra, is what every launch does by now
+   and equals the default; the derivative pass and the halo fill run 256
+   threads per patch (DEFAULT), 512 (WIDE) or 128 (NARROW; the pass's shapes
+   exist for 9^3 patches), the fill with 8 independent loads per thread in its
+   gather or 16 (DEEP). Drops a captured step graph. CCZ4_ERR_INVALID for an
+   unknown shape. */
 enum { CCZ4_STAGE_SHAPE_DEFAULT = 0, CCZ4_STAGE_SHAPE_MORE_BLOCKS = 1, CCZ4_STAGE_SHAPE_FEWER_BLOCKS = 2,
        CCZ4_STAGE_SHAPE_SPLIT = 3 };
 enum { CCZ4_FILL_SHAPE_DEFAULT = 0, CCZ4_FILL_SHAPE_WIDE = 1, CCZ4_FILL_SHAPE_DEEP = 2, CCZ4_FILL_SHAPE_NARROW = 3 };

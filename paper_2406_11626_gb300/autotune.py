@@ -5,16 +5,15 @@ The cost of a step depends on
   (p+6)^3 points for p^3 interior ones: 8x at p = 6, 4.6x at p = 9, 3.4x
   at p = 12, 2.6x at p = 17, so small patches move more halo data while
   large ones give the halo fill fewer, larger blocks);
-- the launch of the stage kernel: a flat grid of one thread per point, a
+- the launch of the algebra kernel: a flat grid of one thread per point, a
   persistent launch whose warps take 32-point items from a device queue,
-  or (p = 9) the fill and the stage in one cooperative launch per RK stage;
-- the stage kernel's launch shape: the default number of resident
+  or (p = 9) the derivative pass and the algebra in one cooperative launch
+  per RK stage;
+- the algebra kernel's launch shape: the default number of resident
   128-thread blocks per SM, one more (fewer registers per thread, more
-  warps to hide latency, more register spills), one fewer, or (mixed
-  precision) two phases in one launch, the stencil values of each point
-  parked in shared memory before the algebra runs on them;
-- the halo fill's launch shape: threads per patch block and the number of
-  independent loads per thread in its gather.
+  warps to hide latency, more register spills) or one fewer (shape 3 is the
+  default again);
+- the derivative pass's launch shape: threads per patch block.
 The tuner times one RK4 step (replays of the step captured as a CUDA graph,
 the way a production loop runs it, CUDA events) of each candidate on the
 workload itself and descends one coordinate at a time: first p and the
@@ -41,8 +40,8 @@ DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "ccz4_gb300", "a
 # the patch edges of the paper's patch-size study, plus the largest edge the fill kernel takes
 CANDIDATES = (6, 9, 12, 17, 18)
 LAUNCHES = ("flat", "queue", "fused")
-STAGE_SHAPES = (0, 1, 2, 3)   # default, one resident block more, one fewer, two phases (mixed)
-FILL_SHAPES = (0, 1, 2, 3)    # 256 threads x 8 loads, 512 x 8, 256 x 16, 128 x 8
+STAGE_SHAPES = (0, 1, 2, 3)   # default, one resident block more, one fewer, default
+FILL_SHAPES = (0, 1, 2, 3)    # 256 threads, 512, 256, 128
 WORKLOADS = ("puncture144", "puncture3level", "binary")
 
 

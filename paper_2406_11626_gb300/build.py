@@ -30,7 +30,7 @@ def _nvcc():
 
 
 def _deps(src):
-    return [src] + glob.glob(os.path.join(CSRC, "*.cuh")) + [os.path.join(ROOT, "include", "ccz4.h")]
+    return [src] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + [os.path.join(ROOT, "include", "ccz4.h")]
 
 
 def _compile(src):

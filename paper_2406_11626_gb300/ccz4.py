@@ -305,16 +305,17 @@ class Grid:
         return cls(cfg.p, cfg.np, cfg.ijk(), cfg.origin, cfg.dx, cfg.bc, level=getattr(cfg, "level", None))
 
     def set_launch(self, mode):
-        """'flat' (default) or 'queue' launch of the stage kernel, or 'fused'
-        (9^3 patches): the fill and the stage of each RK stage of step and
-        step_graph in one cooperative launch."""
+        """'flat' (default) or 'queue' launch of the algebra kernel, or 'fused'
+        (9^3 patches): the derivative pass and the algebra of each RK stage of
+        step and step_graph in one cooperative launch."""
         m = {"flat": 0, "queue": 1, "fused": 2}[mode] if isinstance(mode, str) else int(mode)
         _check(lib().ccz4_set_launch(self._h, m))
 
     def set_tuning(self, stage_shape=0, fill_shape=0):
-        """Launch shapes of the flat stage kernel (0 default, 1 one resident
-        block more, 2 one fewer, 3 two phases (mixed precision)) and of the halo fill (0 default, 1 512
-        threads, 2 16 loads per thread, 3 128 threads); results are identical."""
+        """Launch shapes of the flat algebra kernel (0 and 3 default, 1 one
+        resident block more, 2 one fewer) and of the derivative pass and the
+        halo fill (0 default, 1 512 threads, 2 16 loads per thread in the fill,
+        3 128 threads); results are identical."""
         _check(lib().ccz4_set_tuning(self._h, int(stage_shape), int(fill_shape)))
 
     def restrict(self, buf="U", stream=None):

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "ccz4_internal.cuh"
+#include "derive.h"
 #include "mesh_plan.h"
 
 namespace ccz4 {
@@ -25,9 +26,6 @@ void set_error(const char *fmt, ...) {
 }
 
 int constraint_blocks(long long n_points);
-// shared-memory limits of the two-phase stage kernels (rhs_shapes.cu, rhs_mesh_shapes.cu)
-cudaError_t prepare_shaped_uniform();
-cudaError_t prepare_shaped_mesh();
 // constraint norms over the leaf points outside n_centres balls (constraints.cu)
 cudaError_t launch_constraints_excluded(const GridView &g, const double *H, const double *M, int n_centres,
                                         const double *centres, double radius, double *partial, int blocks,
@@ -96,16 +94,36 @@ extern "C" ccz4_status ccz4_set_allocator(ccz4_alloc_fn alloc, ccz4_dealloc_fn d
   return CCZ4_OK;
 }
 
+static size_t der_bytes(const GridView &v) { return sizeof(double) * (size_t)DER_SLOTS * (size_t)v.n_points; }
+
+// A large buffer of a grid from its allocator; NULL with the error message set on failure.
+static double *large_alloc(ccz4_grid *g, size_t bytes) {
+  if (g->alloc) {
+    double *p = (double *)g->alloc(g->alloc_ctx, bytes, nullptr);
+    if (p && ((uintptr_t)p & 255u) == 0) return p;
+    set_error("the allocator returned %s for %zu bytes", p ? "an unaligned pointer" : "NULL", bytes);
+    if (p) g->dealloc(g->alloc_ctx, p, bytes, nullptr);
+    return nullptr;
+  }
+  double *p = nullptr;
+  cudaError_t e = cudaMalloc(&p, bytes);
+  if (e == cudaSuccess) return p;
+  set_error("cudaMalloc of %lld doubles failed: %s", (long long)(bytes / sizeof(double)), cudaGetErrorString(e));
+  cudaGetLastError();
+  return nullptr;
+}
+
+static void large_free(ccz4_grid *g, double *p, size_t bytes) {
+  if (!p) return;
+  if (g->dealloc) g->dealloc(g->alloc_ctx, p, bytes, nullptr);
+  else cudaFree(p);
+}
+
 static void free_all(ccz4_grid *g) {
   if (g->step_exec) cudaGraphExecDestroy(g->step_exec);
   if (g->cap_stream) cudaStreamDestroy(g->cap_stream);
-  for (int b = 0; b < 8; ++b) {
-    if (!g->buf[b]) continue;
-    if (g->dealloc)
-      g->dealloc(g->alloc_ctx, g->buf[b], sizeof(double) * (size_t)g->buf_len[b], nullptr);
-    else
-      cudaFree(g->buf[b]);
-  }
+  for (int b = 0; b < 8; ++b) large_free(g, g->buf[b], sizeof(double) * (size_t)g->buf_len[b]);
+  large_free(g, g->der, der_bytes(g->v));
   cudaFree(g->d_ijk);
   cudaFree(g->d_owner);
   cudaFree(g->d_gcoord);
@@ -285,28 +303,16 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
     g->buf_len[b] = lens[b];
     if (lens[b] == 0) continue;
     const size_t bytes = sizeof(double) * (size_t)lens[b];
-    if (g->alloc) {
-      g->buf[b] = (double *)g->alloc(g->alloc_ctx, bytes, nullptr);
-      if (!g->buf[b] || ((uintptr_t)g->buf[b] & 255u)) {
-        set_error("the allocator returned %s for %zu bytes", g->buf[b] ? "an unaligned pointer" : "NULL", bytes);
-        if (g->buf[b]) {
-          g->dealloc(g->alloc_ctx, g->buf[b], bytes, nullptr);
-          g->buf[b] = nullptr;
-        }
-        free_all(g);
-        return CCZ4_ERR_NOMEM;
-      }
-    } else {
-      cudaError_t e = cudaMalloc(&g->buf[b], bytes);
-      if (e != cudaSuccess) {
-        g->buf[b] = nullptr;
-        set_error("cudaMalloc of %lld doubles failed: %s", lens[b], cudaGetErrorString(e));
-        cudaGetLastError();
-        free_all(g);
-        return CCZ4_ERR_NOMEM;
-      }
+    g->buf[b] = large_alloc(g, bytes);
+    if (!g->buf[b]) {
+      free_all(g);
+      return CCZ4_ERR_NOMEM;
     }
     cudaMemset(g->buf[b], 0, bytes);
+  }
+  if (v.n_points > 0 && !(g->der = large_alloc(g, der_bytes(v)))) {
+    free_all(g);
+    return CCZ4_ERR_NOMEM;
   }
   g->red_blocks = constraint_blocks(v.n_points);
   bool ok = cudaMalloc(&g->d_ijk, sizeof(int) * 3 * (size_t)d->n_patches) == cudaSuccess &&
@@ -350,9 +356,8 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
     }
   }
   prepare_fill_halos(v.p);
+  prepare_derive();
   if (v.p == 9) prepare_fused();
-  if (mesh) prepare_shaped_mesh();
-  else prepare_shaped_uniform();
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     set_error("grid set-up failed: %s", cudaGetErrorString(e));
@@ -551,6 +556,12 @@ static const double *ini_ptr(ccz4_grid *g) {
   return g->buf[CCZ4_BUF_INI] ? g->buf[CCZ4_BUF_INI] : g->buf[CCZ4_BUF_U];
 }
 
+// The derivative pass of a state buffer as the algebra for P needs it.
+static cudaError_t derivatives(ccz4_grid *g, const ccz4_params *P, int buf, cudaStream_t s) {
+  return launch_derive(g->v, g->buf[buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der, all_fields(),
+                       P->precision == CCZ4_PREC_MIXED, false, false, s);
+}
+
 extern "C" ccz4_status ccz4_rhs(ccz4_grid *g, const ccz4_params *P, int in_buf, int out_buf, void *stream) {
   if (check_grid(g) || check_params(P)) return CCZ4_ERR_INVALID;
   if (!state_buffer(in_buf) || !state_buffer(out_buf) || in_buf == out_buf || !g->buf[in_buf] ||
@@ -559,9 +570,8 @@ extern "C" ccz4_status ccz4_rhs(ccz4_grid *g, const ccz4_params *P, int in_buf, 
     return CCZ4_ERR_INVALID;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  CUDA_TRY(launch_fill_halos(g->v, g->buf[in_buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], s,
-                             P->precision == CCZ4_PREC_MIXED));
-  CUDA_TRY(launch_rhs(g->v, *P, g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->buf[in_buf], ini_ptr(g), g->buf[out_buf], s));
+  CUDA_TRY(derivatives(g, P, in_buf, s));
+  CUDA_TRY(launch_rhs(g->v, *P, g->der, g->buf[CCZ4_BUF_MIX], g->buf[in_buf], ini_ptr(g), g->buf[out_buf], s));
   return CCZ4_OK;
 }
 
@@ -575,26 +585,24 @@ static ccz4_status restrict_levels(ccz4_grid *g, double *U, cudaStream_t s) {
   return CCZ4_OK;
 }
 
-// One RK4 stage from the halo'd tiles; stage 3 ends the step (enforcement
-// in the stage kernel, then the restriction on a mesh).
+// One RK4 stage from its derivatives; stage 3 ends the step (enforcement in
+// the algebra kernel, then the restriction on a mesh).
 static ccz4_status stage_kernel(ccz4_grid *g, const ccz4_params *P, int stage, double dt, cudaStream_t s) {
-  double *in = g->buf[kStageIn[stage]];
-  CUDA_TRY(launch_rk_stage(g->v, *P, stage, dt, g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], in, ini_ptr(g), g->buf[CCZ4_BUF_U],
-                           g->buf[CCZ4_BUF_ACC], g->buf[kStageOut[stage]], s));
+  CUDA_TRY(launch_rk_stage(g->v, *P, stage, dt, g->der, g->buf[CCZ4_BUF_MIX], g->buf[kStageIn[stage]], ini_ptr(g),
+                           g->buf[CCZ4_BUF_U], g->buf[CCZ4_BUF_ACC], g->buf[kStageOut[stage]], s));
   if (stage == 3 && g->v.n_levels > 1) return restrict_levels(g, g->buf[kStageOut[stage]], s);
   return CCZ4_OK;
 }
 
-// One RK4 stage of a step: the halo fill and the stage kernel as two
+// One RK4 stage of a step: the derivative pass and the algebra kernel as two
 // launches, or (CCZ4_LAUNCH_FUSED) both in one cooperative launch; the
 // restriction after stage 3 stays a launch of its own.
 static ccz4_status step_stage(ccz4_grid *g, const ccz4_params *P, int stage, double dt, cudaStream_t s) {
   if (!g->fused) {
-    CUDA_TRY(launch_fill_halos(g->v, g->buf[kStageIn[stage]], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], s,
-                               P->precision == CCZ4_PREC_MIXED));
+    CUDA_TRY(derivatives(g, P, kStageIn[stage], s));
     return stage_kernel(g, P, stage, dt, s);
   }
-  CUDA_TRY(launch_fused_stage(g->v, *P, stage, dt, g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX],
+  CUDA_TRY(launch_fused_stage(g->v, *P, stage, dt, g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der,
                               g->buf[kStageIn[stage]], ini_ptr(g), g->buf[CCZ4_BUF_U], g->buf[CCZ4_BUF_ACC],
                               g->buf[kStageOut[stage]], s));
   if (stage == 3 && g->v.n_levels > 1) return restrict_levels(g, g->buf[kStageOut[stage]], s);
@@ -668,6 +676,9 @@ extern "C" ccz4_status ccz4_rk_stage(ccz4_grid *g, const ccz4_params *P, int sta
     set_error("rk_stage: stage must be 0..3 (got %d) and dt finite", stage);
     return CCZ4_ERR_INVALID;
   }
+  // the stage's input as the halo fill left it in the tile buffer
+  CUDA_TRY(launch_derive(g->v, g->buf[kStageIn[stage]], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der,
+                         all_fields(), P->precision == CCZ4_PREC_MIXED, true, false, (cudaStream_t)stream));
   return stage_kernel(g, P, stage, dt, (cudaStream_t)stream);
 }
 
@@ -686,7 +697,7 @@ extern "C" ccz4_status ccz4_step(ccz4_grid *g, const ccz4_params *P, double dt, 
   return CCZ4_OK;
 }
 
-// Captures one RK4 step (four halo fills and four stage launches) into a
+// Captures one RK4 step (four derivative passes and four stage launches) into a
 // CUDA graph on a private stream; kernel arguments, parameters and dt are
 // baked into the graph.
 static ccz4_status capture_step(ccz4_grid *g, const ccz4_params *P, double dt) {

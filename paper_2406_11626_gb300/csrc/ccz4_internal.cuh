@@ -213,6 +213,7 @@ struct ccz4_grid {
   ccz4_dealloc_fn dealloc;
   void *alloc_ctx;
   int fused;                    // CCZ4_LAUNCH_FUSED: one cooperative launch per RK stage (p = 9)
+  double *der;                  // derivative buffer, [DER_SLOTS][n_points] (derive.cuh), from the same allocator
 };
 
 // Kernel launchers (one translation unit each).
@@ -223,14 +224,14 @@ cudaError_t launch_ghost_setup(const GridView &g, GhostGeo *out, cudaStream_t s)
 cudaError_t launch_fill_halos(const GridView &g, const double *src, double *tile, double *mix, cudaStream_t s,
                               bool fp32_weights = false);
 cudaError_t prepare_fill_halos(int p);
-// One cooperative launch per RK stage (rhs_fused.cu): the halo fill of every
-// patch, a grid-wide barrier, the interior points and the Sommerfeld ghost
-// cells; p = 9 only. prepare_fused raises its shared-memory limit (once per
+// One cooperative launch per RK stage (rhs_fused.cu): the derivative pass of
+// every patch, a grid-wide barrier, the interior points and the Sommerfeld
+// ghost cells; p = 9 only. prepare_fused raises its shared-memory limit (once per
 // grid, outside any stream capture).
 cudaError_t prepare_fused();
 cudaError_t launch_fused_stage(const GridView &g, const ccz4_params &P, int stage, double dt, double *tile,
-                               double *mix, const double *in, const double *ini, const double *U, double *acc,
-                               double *out, cudaStream_t s);
+                               double *mix, double *der, const double *in, const double *ini, const double *U,
+                               double *acc, double *out, cudaStream_t s);
 // psi_4 at every interior point from the halo'd tiles: Re into out[0 .. n_points), Im into out[S ..),
 // the tetrad centred at centre (psi4.cu)
 cudaError_t launch_psi4(const GridView &g, const double *tile, const double centre[3], double *out, cudaStream_t s);
@@ -238,10 +239,10 @@ cudaError_t launch_psi4(const GridView &g, const double *tile, const double cent
 constexpr int NMIX = 33;
 // largest patch edge whose halo'd tile of one field fits in the fill kernel's shared memory
 constexpr int MAX_P = 18;
-cudaError_t launch_rhs(const GridView &g, const ccz4_params &P, const double *tile, const double *mix,
+cudaError_t launch_rhs(const GridView &g, const ccz4_params &P, const double *der, const double *mix,
                        const double *in, const double *ini, double *out, cudaStream_t s);
 cudaError_t launch_rk_stage(const GridView &g, const ccz4_params &P, int stage, double dt,
-                            const double *tile, const double *mix, const double *in, const double *ini,
+                            const double *der, const double *mix, const double *in, const double *ini,
                             const double *U, double *acc, double *out, cudaStream_t s);
 cudaError_t launch_enforce(const GridView &g, double *U, cudaStream_t s);
 // restriction of level l onto the n_par parents par[] of level l-1 (children kid[n_par][27])

@@ -1,0 +1,129 @@
+// The derivative pass (derive.cuh): kernels and launches.
+#include "derive.cuh"
+
+namespace ccz4 {
+namespace {
+
+template <int SRC, bool MIXED, bool RAW, int SHAPE, int PF, int NF>
+__global__ void __launch_bounds__(FILL_SHAPE_THREADS[SHAPE], (PF == 9 ? 1024 : 768) / FILL_SHAPE_THREADS[SHAPE])
+    derive_kernel(GridView g, const double *__restrict__ src, double *tile, double *__restrict__ mix,
+                  double *__restrict__ der, LevelScale ls, FieldList fl, bool tile_out) {
+  extern __shared__ double smem[];
+  derive_patch<SRC, MIXED, RAW, FILL_SHAPE_THREADS[SHAPE], PF, NF>(g, src, tile, mix, der, ls, fl, blockIdx.x,
+                                                                   blockIdx.y, gridDim.y, tile_out, smem);
+}
+
+// Field groups per patch. A block's set-up (the source table) is shared by
+// the fields it takes, so a grid of many patches gives each block all fields;
+// a grid of few patches splits them until there are about two waves of
+// blocks (27 patches of 9^3: one block per field).
+int field_groups(const GridView &g, const FieldList &fl) {
+  const int want = 6 * 152;
+  int k = g.n_patches > 0 ? (want + g.n_patches - 1) / g.n_patches : 1;
+  k = k < 1 ? 1 : k;
+  return k < fl.n ? k : fl.n;
+}
+
+template <int SRC, bool MIXED, bool RAW, int SHAPE, int PF, int NF>
+cudaError_t launch_one(const GridView &g, const double *src, double *tile, double *mix, double *der,
+                       const FieldList &fl, bool tile_out, cudaStream_t s) {
+  const dim3 grid(g.n_patches, field_groups(g, fl));
+  derive_kernel<SRC, MIXED, RAW, SHAPE, PF, NF><<<grid, FILL_SHAPE_THREADS[SHAPE], derive_smem_bytes(g.p, RAW), s>>>(
+      g, src, tile, mix, der, level_scale(g), fl, tile_out);
+  return cudaGetLastError();
+}
+
+template <int SRC, bool MIXED, int SHAPE>
+cudaError_t launch_edge(const GridView &g, const double *src, double *tile, double *mix, double *der,
+                        const FieldList &fl, bool tile_out, cudaStream_t s) {
+  if (g.p == 9) return launch_one<SRC, MIXED, false, SHAPE, 9, NV>(g, src, tile, mix, der, fl, tile_out, s);
+  if constexpr (SHAPE == 0) {
+    if (derive_raw(g.p)) return launch_one<SRC, MIXED, true, 0, 0, NV>(g, src, tile, mix, der, fl, tile_out, s);
+    return launch_one<SRC, MIXED, false, 0, 0, NV>(g, src, tile, mix, der, fl, tile_out, s);
+  } else {
+    return launch_edge<SRC, MIXED, 0>(g, src, tile, mix, der, fl, tile_out, s);
+  }
+}
+
+template <int SRC, bool MIXED>
+cudaError_t launch_shape(const GridView &g, const double *src, double *tile, double *mix, double *der,
+                         const FieldList &fl, bool tile_out, cudaStream_t s) {
+  if constexpr (SRC != FROM_TILE) {
+    if (g.fill_shape == 1) return launch_edge<SRC, MIXED, 1>(g, src, tile, mix, der, fl, tile_out, s);
+    if (g.fill_shape == 3) return launch_edge<SRC, MIXED, 3>(g, src, tile, mix, der, fl, tile_out, s);
+  }
+  return launch_edge<SRC, MIXED, 0>(g, src, tile, mix, der, fl, tile_out, s);
+}
+
+template <int SRC, bool MIXED, bool RAW, int SHAPE, int PF, int NF>
+cudaError_t prepare_one(int p) {
+  return cudaFuncSetAttribute(derive_kernel<SRC, MIXED, RAW, SHAPE, PF, NF>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)derive_smem_bytes(p, RAW));
+}
+
+// The largest dynamic shared memory that any grid asks of the general instances.
+int largest_edge(bool raw) {
+  int q = 1;
+  for (int p = 1; p <= MAX_P; ++p)
+    if (derive_raw(p) == raw) q = p;
+  return q;
+}
+
+template <int SRC, bool MIXED>
+cudaError_t prepare_source() {
+  cudaError_t e = prepare_one<SRC, MIXED, false, 0, 9, NV>(9);
+  if (e == cudaSuccess) e = prepare_one<SRC, MIXED, false, 0, 0, NV>(largest_edge(false));
+  if (e == cudaSuccess) e = prepare_one<SRC, MIXED, true, 0, 0, NV>(largest_edge(true));
+  if constexpr (SRC != FROM_TILE) {
+    if (e == cudaSuccess) e = prepare_one<SRC, MIXED, false, 1, 9, NV>(9);
+    if (e == cudaSuccess) e = prepare_one<SRC, MIXED, false, 3, 9, NV>(9);
+  }
+  return e;
+}
+
+}  // namespace
+
+cudaError_t prepare_derive() {
+  cudaError_t e = prepare_source<FROM_LEVEL, false>();
+  if (e == cudaSuccess) e = prepare_source<FROM_LEVEL, true>();
+  if (e == cudaSuccess) e = prepare_source<FROM_MESH, false>();
+  if (e == cudaSuccess) e = prepare_source<FROM_MESH, true>();
+  if (e == cudaSuccess) e = prepare_source<FROM_TILE, false>();
+  if (e == cudaSuccess) e = prepare_source<FROM_TILE, true>();
+  if (e == cudaSuccess) e = prepare_one<FROM_LEVEL, false, false, 0, 9, 58>(9);
+  if (e == cudaSuccess) e = prepare_one<FROM_LEVEL, false, false, 0, 0, 58>(largest_edge(false));
+  if (e == cudaSuccess) e = prepare_one<FROM_LEVEL, false, true, 0, 0, 58>(largest_edge(true));
+  return e;
+}
+
+FieldList all_fields() {
+  FieldList fl;
+  fl.n = 0;
+  for (int pass = 0; pass < 2; ++pass)
+    for (int v = 0; v < NV; ++v)
+      if ((mix_slot(v) >= 0) == (pass == 0)) fl.f[fl.n++] = (unsigned char)v;
+  return fl;
+}
+
+cudaError_t launch_derive(const GridView &g, const double *src, double *tile, double *mix, double *der,
+                          const FieldList &fl, bool mixed, bool from_tile, bool tile_out, cudaStream_t s) {
+  if (g.n_patches == 0 || fl.n == 0) return cudaSuccess;
+  if (from_tile)
+    return mixed ? launch_shape<FROM_TILE, true>(g, src, tile, mix, der, fl, false, s)
+                 : launch_shape<FROM_TILE, false>(g, src, tile, mix, der, fl, false, s);
+  if (g.src)
+    return mixed ? launch_shape<FROM_MESH, true>(g, src, tile, mix, der, fl, false, s)
+                 : launch_shape<FROM_MESH, false>(g, src, tile, mix, der, fl, tile_out, s);
+  return mixed ? launch_shape<FROM_LEVEL, true>(g, src, tile, mix, der, fl, false, s)
+               : launch_shape<FROM_LEVEL, false>(g, src, tile, mix, der, fl, tile_out, s);
+}
+
+cudaError_t launch_derive_fo(const GridView &g, const double *src, double *der, const FieldList &fl, cudaStream_t s) {
+  if (g.n_patches == 0 || fl.n == 0) return cudaSuccess;
+  if (g.p == 9) return launch_one<FROM_LEVEL, false, false, 0, 9, 58>(g, src, nullptr, nullptr, der, fl, false, s);
+  if (derive_raw(g.p))
+    return launch_one<FROM_LEVEL, false, true, 0, 0, 58>(g, src, nullptr, nullptr, der, fl, false, s);
+  return launch_one<FROM_LEVEL, false, false, 0, 0, 58>(g, src, nullptr, nullptr, der, fl, false, s);
+}
+
+}  // namespace ccz4

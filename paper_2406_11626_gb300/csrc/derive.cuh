@@ -1,0 +1,401 @@
+// The derivative pass: everything a right-hand side needs of its neighbours.
+//
+// One block gathers a patch's halo'd tile field by field into shared memory
+// and writes, for each of the patch's points, the unscaled stencil sums of
+// the field: the three first-derivative sums and the Kreiss-Oliger sum, for
+// the fields with second derivatives also the three pure ones, and the mixed
+// second derivatives (as the halo fill forms them). The pointwise algebra
+// (algebra kernels, monitors) then reads each point's values in full lines
+// and touches no neighbour.
+//
+// Why a pass of its own: the FP64 pipe issues 2 operations per clock per SM,
+// and about 45 % of the right-hand side's FP64 operations are stencil sums.
+// Here they run on the integer pipes instead (fixed_stencil.cuh), at the
+// occupancy and the register count of a small kernel; a value is converted
+// once per tile it lands in (4.6 times at a patch edge of 9) and not once for
+// each of the 19 points that read it. The algebra is left with the FP64
+// operations that have to be FP64, needs no tile (nothing is reused through
+// L1) and spills less.
+#pragma once
+
+#include "derive.h"
+#include "fixed_stencil.cuh"
+#include "halo_fill.cuh"
+
+namespace ccz4 {
+
+namespace {
+
+// The word and the exponent under which a tile value waits in shared memory:
+// its mantissa as a signed integer of 57 bits and its biased exponent; the
+// value's own bits where the exponent is FX_TOP or more, 0 for zero (and for
+// subnormal values).
+__device__ __forceinline__ long long fx_word(double u, unsigned &e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(u);
+  e = (unsigned)(b >> 52) & 0x7FFu;
+  const unsigned long long m = ((b << 4) & 0x00FFFFFFFFFFFFF0ull) | 0x0100000000000000ull;
+  const unsigned long long n = (unsigned long long)((long long)b >> 63);
+  return e >= FX_TOP ? (long long)b : e == 0u ? 0 : (long long)((m ^ n) - n);
+}
+__device__ __forceinline__ double fx_value(long long w, unsigned e) {
+  if (e >= FX_TOP) return __longlong_as_double(w);
+  if (e == 0) return 0.0;
+  const unsigned long long n = (unsigned long long)(w >> 63), a = ((unsigned long long)w ^ n) - n;
+  return __longlong_as_double((long long)((n & 0x8000000000000000ull) | ((unsigned long long)e << 52) |
+                                          ((a >> 4) & 0x000FFFFFFFFFFFFFull)));
+}
+__device__ __forceinline__ long long fx_sar(long long x, unsigned s) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));  // all sign bits beyond 63
+  return r;
+}
+
+// v units of 2^(e - 1075 - K) as FP32: the two halves converted and joined in one
+// rounding, then two exact scalings (a result outside the FP32 range becomes
+// zero or infinite, as the FP32 conversions of the mixed precision do).
+template <int K>
+__device__ __forceinline__ float fx_outf(long long v, unsigned e) {
+  const float f = fmaf(__int2float_rn((int)(v >> 32)), 4294967296.0f, __uint2float_rn((unsigned)v));
+  const int s = (int)e - 896;  // FP32 exponent field of 2^(e - 1023)
+  const float sc = s < 1 ? 0.0f : s > 254 ? __uint_as_float(0x7F800000u) : __uint_as_float((unsigned)s << 23);
+  return f == 0.0f ? 0.0f : (f * (K == 4 ? 1.3877787807814457e-17f : 5.5511151231257827e-17f)) * sc;  // 2^-(52 + K)
+}
+template <int K, class O>
+__device__ __forceinline__ O fx_result(long long v, unsigned e) {
+  if constexpr (std::is_same<O, float>::value) return fx_outf<K>(v, e);
+  else return fx_out<K>(v, (e << 21) | FX_LOW);
+}
+
+// The stencil sums of one point whose largest neighbour lies outside [FX_FLOOR, FX_TOP), in FP64.
+template <bool SECOND>
+__device__ __noinline__ void point_sums_fp64(const long long *w, const unsigned *ex, int T, double *out) {
+  const int st[3] = {1, T, T * T};
+  const double c = fx_value(w[0], ex[0]);
+  double s[3] = {0.0, 0.0, 0.0};
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k) {
+    double p[3], m[3];
+    for (int j = 0; j < 3; ++j) {
+      const int o = (j + 1) * st[k];
+      p[j] = fx_value(w[o], ex[o]);
+      m[j] = fx_value(w[-o], ex[-o]);
+      s[j] += p[j] + m[j];
+    }
+    out[k] = fma(8.0, p[0] - m[0], -(p[1] - m[1]));
+    if (SECOND) out[4 + k] = fma(-30.0, c, fma(16.0, p[0] + m[0], -(p[1] + m[1])));
+  }
+  out[3] = fma(-60.0, c, fma(15.0, s[0], fma(-6.0, s[1], s[2])));
+}
+
+// The stencil sums of the point at w, ex: out[0..2] first derivatives, out[3]
+// dissipation, out[4..6] pure second derivatives.
+template <bool SECOND, class O>
+__device__ __forceinline__ void point_sums(const long long *w, const unsigned *ex, int T, O *out) {
+  const int st[3] = {1, T, T * T};
+  const unsigned e0 = ex[0];
+  unsigned ep[3][3], em[3][3], e = e0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      ep[k][j] = ex[(j + 1) * st[k]];
+      em[k][j] = ex[-(j + 1) * st[k]];
+      e = max(e, max(ep[k][j], em[k][j]));
+    }
+  if (e - FX_FLOOR >= FX_TOP - FX_FLOOR && e != 0u) {  // (all zero: the sums below are zero)
+    double d[7];
+    point_sums_fp64<SECOND>(w, ex, T, d);
+#pragma unroll
+    for (int q = 0; q < (SECOND ? 7 : 4); ++q) out[q] = cvt<O>(d[q]);
+    return;
+  }
+  const long long q = fx_sar(w[0], e - e0) >> 2;
+  long long s1 = 0, s2 = 0, s3 = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int s = st[k];
+    const long long p1 = fx_sar(w[s], e - ep[k][0]), m1 = fx_sar(w[-s], e - em[k][0]);
+    const long long p2 = fx_sar(w[2 * s], e - ep[k][1]), m2 = fx_sar(w[-2 * s], e - em[k][1]);
+    const long long t1 = p1 + m1, t2 = p2 + m2;
+    out[k] = fx_result<4, O>((p1 - m1) * 8 - (p2 - m2), e);
+    if (SECOND) out[4 + k] = fx_result<2, O>(((t1 >> 2) - 2 * q) * 16 - (t2 >> 2) + 2 * q, e);
+    s1 += t1;
+    s2 += t2;
+    s3 += fx_sar(w[3 * s], e - ep[k][2]) + fx_sar(w[-3 * s], e - em[k][2]);
+  }
+  out[3] = fx_result<2, O>((((s1 >> 2) - 4 * q) * 5 - 2 * (s2 >> 2)) * 3 + (s3 >> 2), e);
+}
+
+// The same from raw FP64 values, for patch edges whose tile leaves no room for the exponents.
+template <bool SECOND, class O>
+__device__ __forceinline__ void point_sums_raw(const double *t, int T, O *out) {
+  const int st[3] = {1, T, T * T};
+  double p[3][3], m[3][3], d1[3], d2[3], ko;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      p[k][j] = t[(j + 1) * st[k]];
+      m[k][j] = t[-(j + 1) * st[k]];
+    }
+  fx_axes<true, SECOND>(t[0], p, m, d1, d2, ko);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    out[k] = cvt<O>(d1[k]);
+    if (SECOND) out[4 + k] = cvt<O>(d2[k]);
+  }
+  out[3] = cvt<O>(ko);
+}
+
+// Where a patch's tile comes from: gathered through the neighbour lookup of a
+// single level, or through a refined mesh's table, or read from the tile
+// buffer that a halo fill has written.
+enum { FROM_LEVEL = 0, FROM_MESH = 1, FROM_TILE = 2 };
+
+// First sums of the mixed derivatives from the raw FP64 tile; FP32 sums for
+// the fields whose mixed derivatives the mixed precision keeps in FP32.
+__device__ __forceinline__ void mixed_first(double *ext, int e, const double *ts, int c0, int s, bool f32) {
+  const double a = ts[c0 + s] - ts[c0 - s], b = ts[c0 + 2 * s] - ts[c0 - 2 * s];
+  if (f32) reinterpret_cast<float *>(ext)[e] = fmaf(8.0f, cvt<float>(a), -cvt<float>(b));
+  else ext[e] = fma(8.0, a, -b);
+}
+
+// Doubles that the widened region of the mixed derivatives takes, and the
+// place of the exponents with it: a field's mixed derivatives are done before
+// its exponents are written, so the two share their place (unless RAW, which
+// keeps no exponents).
+__host__ __device__ constexpr int derive_ext(int p) {
+  return fill_wide(p) ? (p + 4) * (p + 4) * p : (p + 4) * p * p;
+}
+__host__ __device__ constexpr int derive_shared(int p, bool raw) {
+  const int T3 = (p + 2 * HALO) * (p + 2 * HALO) * (p + 2 * HALO), e = derive_ext(p), x = raw ? 0 : (T3 + 1) / 2;
+  return e > x ? e : x;
+}
+// Shared memory of a block: the tile's words, the shared place above and the
+// source table (not FROM_TILE). 54 KB at a patch edge of 9: four blocks per SM.
+inline size_t derive_smem_bytes(int p, bool raw) {
+  const size_t T = (size_t)p + 2 * HALO, T3 = T * T * T;
+  return T3 * (8 + 4) + 8 * (size_t)derive_shared(p, raw);
+}
+inline bool derive_raw(int p) { return derive_smem_bytes(p, false) > FILL_SMEM_LIMIT; }
+
+// The fields group, group + groups, ... of the list, of patch n, by one block
+// of THREADS threads. NF: fields of the formulation (25, or 58 without second
+// derivatives). tile: the tile buffer; interpolated halo points of a mesh pass
+// through it, tile_out (FP64) has the whole tile written to it, FROM_TILE reads it.
+template <int SRC, bool MIXED, bool RAW, int THREADS, int PF, int NF>
+__device__ __forceinline__ void derive_patch(const GridView &g, const double *__restrict__ src, double *tile,
+                                             double *__restrict__ mix, double *__restrict__ der, const LevelScale &ls,
+                                             const FieldList &fl, int n, int group, int groups, bool tile_out,
+                                             double *smem) {
+  constexpr int BATCH = 8;
+  const int p = PF > 0 ? PF : g.p, T = PF > 0 ? PF + 2 * HALO : g.T;
+  const int T3 = PF > 0 ? T * T * T : (int)g.T3;
+  const int pe = p + 4, next = pe * p * p, p3 = p * p * p;
+  const bool wide = fill_wide(p);
+  double *ts = smem;
+  double *ext = ts + T3;
+  unsigned *ex = reinterpret_cast<unsigned *>(ext);
+  int *idx = reinterpret_cast<int *>(ext + derive_shared(p, RAW));
+  constexpr bool MESH = SRC == FROM_MESH;
+  int e0 = 0, e1 = 0, xb0 = 0, nx = 0, yb0 = 0, ny = 0;
+  if (MESH) {
+    const int *sp = g.src + (long long)n * T3;
+    for (int t = threadIdx.x; t < T3; t += THREADS) idx[t] = __ldg(sp + t);
+    e0 = __ldg(g.ibeg + n);
+    e1 = __ldg(g.ibeg + n + 1);
+    xb0 = __ldg(g.xbeg + n);
+    nx = __ldg(g.xbeg + n + 1) - xb0;
+    yb0 = __ldg(g.ybeg + n);
+    ny = __ldg(g.ybeg + n + 1) - yb0;
+    // a patch without separable tables: one entry per thread, every field of the group
+    for (int e = nx == 0 ? e0 + (int)threadIdx.x : e1; e < e1; e += THREADS) {
+      const InterpEntry *ep = g.interp + e;
+      int c[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) c[k] = __ldg(&ep->src[k]);
+      const int r = __ldg(&ep->r), t = __ldg(&ep->t);
+      for (int j = group; j < fl.n; j += groups)
+        __stcs(tile + ((long long)fl.f[j] * g.n_patches + n) * T3 + t,
+               interp_value(c, r & 3, (r >> 2) & 3, (r >> 4) & 3, src + fl.f[j] * g.S));
+    }
+  } else if (SRC == FROM_LEVEL) {
+    const int bx = __ldg(g.ijk + 3 * n) * p - HALO;
+    const int by = __ldg(g.ijk + 3 * n + 1) * p - HALO;
+    const int bz = __ldg(g.ijk + 3 * n + 2) * p - HALO;
+    for (int t = threadIdx.x; t < T3; t += THREADS) {
+      const int lz = t / (T * T), ly = (t / T) % T, lx = t % T;
+      idx[t] = (int)locate(g, bx + lx, by + ly, bz + lz);
+    }
+  }
+  const double cmix = MESH ? ls.cmix[patch_level(g, n)] : ls.cmix[0];
+  const float cmixf = MESH ? ls.cmixf[patch_level(g, n)] : ls.cmixf[0];
+  const long long pbase = (long long)n * p3, np = g.n_points;
+  // tile offsets of this thread's points (a compile-time edge: the same for every field)
+  constexpr int ROUNDS = PF > 0 ? (PF * PF * PF + THREADS - 1) / THREADS : 1;
+  auto centre_at = [&](int q) {
+    const int x = q % p, y = (q / p) % p, z = q / (p * p);
+    return ((z + HALO) * T + (y + HALO)) * T + (x + HALO);
+  };
+  int at[ROUNDS];
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r) at[r] = PF > 0 ? centre_at(threadIdx.x + r * THREADS) : 0;
+  constexpr int JM = (1 << JOB_BITS) - 1;
+  for (int j = group; j < fl.n; j += groups) {
+    const int v = fl.f[j];
+    const double *sv = src + (long long)v * g.S;
+    double *tv = tile + ((long long)v * g.n_patches + n) * T3;
+    const int slot = NF == NV ? mix_slot(v) : -1;
+    __syncthreads();  // the source table is written; the previous field's readers are done
+    if (MESH && nx > 0) {
+      double *xv = ts, *yv = ts + nx;
+      for (int q = threadIdx.x; q < nx; q += THREADS) {
+        const XJob *J = g.xjob + xb0 + q;
+        const int rx = __ldg(&J->rx);
+        const double q0 = __ldg(sv + __ldg(&J->s0));
+        xv[q] = rx ? lerp3(rx, q0, __ldg(sv + __ldg(&J->s1))) : q0;
+      }
+      __syncthreads();
+      for (int q = threadIdx.x; q < ny; q += THREADS) {
+        const int k = __ldg(g.yjob + yb0 + q);
+        yv[q] = lerp3((k >> (2 * JOB_BITS)) & 3, xv[k & JM], xv[(k >> JOB_BITS) & JM]);
+      }
+      __syncthreads();
+      for (int e = e0 + threadIdx.x; e < e1; e += THREADS) {
+        const int k = __ldg(&g.zjob[e].yab);
+        tv[__ldg(&g.zjob[e].t)] = lerp3((k >> (2 * JOB_BITS)) & 3, yv[k & JM], yv[(k >> JOB_BITS) & JM]);
+      }
+      __syncthreads();
+    }
+    const bool second = slot >= 0;
+    for (int t0 = threadIdx.x; t0 < T3; t0 += BATCH * THREADS) {
+      double val[BATCH];
+#pragma unroll
+      for (int u = 0; u < BATCH; ++u) {
+        const int t = t0 + u * THREADS;
+        val[u] = 0.0;
+        if (t >= T3) continue;
+        if (SRC == FROM_TILE) {
+          val[u] = __ldcs(tv + t);
+        } else {
+          const int s = idx[t];
+          if (s >= 0) val[u] = __ldg(sv + s);
+          else if (MESH && s <= -2) val[u] = __ldcg(tv + t);  // interpolated above (through L2)
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < BATCH; ++u) {
+        const int t = t0 + u * THREADS;
+        if (t >= T3) continue;
+        double w = val[u];
+        if (SRC == FROM_TILE && der_f32(MIXED, v))  // a split pair: its value
+          w = cvt<double>(__int_as_float(__double2loint(w))) + cvt<double>(__int_as_float(__double2hiint(w)));
+        if (SRC != FROM_TILE && tile_out) __stcs(tv + t, w);
+        if (!RAW && (!second || SRC == FROM_TILE)) {
+          unsigned e;
+          reinterpret_cast<long long *>(ts)[t] = fx_word(w, e);
+          ex[t] = e;
+        } else {
+          ts[t] = w;
+        }
+      }
+    }
+    __syncthreads();
+    if (second && SRC != FROM_TILE) {
+      // the mixed derivatives, as the halo fill forms them
+      const bool f32 = MIXED && mix_fslot(slot) >= 0;
+#pragma unroll 1
+      for (int pass = 0; pass < (wide ? 1 : 3); ++pass) {
+        const int si = pass == 0 ? T : T * T;
+        for (int e = threadIdx.x; e < next; e += THREADS) {
+          const int a = e % pe - 2, b = (e / pe) % p, c = e / (pe * p);
+          const int x = pass == 2 ? b : a, y = pass == 2 ? a : b;
+          mixed_first(ext, e, ts, ((c + HALO) * T + (y + HALO)) * T + (x + HALO), si, f32);
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < p3; q += THREADS) {
+          const int x = q % p, y = (q / p) % p, z = q / (p * p);
+          const int a = pass == 2 ? y : x, b = pass == 2 ? x : y;
+          mixed_out(ext, (z * p + b) * pe + (a + 2), 1, cmix, cmixf, f32, mix, np, pbase, slot + pass, q);
+        }
+        __syncthreads();
+      }
+      if (wide) {
+        for (int e = threadIdx.x; e < pe * pe * p; e += THREADS) {
+          const int a = e % pe - 2, b = (e / pe) % pe - 2, c = e / (pe * pe);
+          if ((a < 0 || a >= p) && (b < 0 || b >= p)) continue;
+          mixed_first(ext, e, ts, ((c + HALO) * T + (b + HALO)) * T + (a + HALO), T * T, f32);
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < p3; q += THREADS) {
+          const int x = q % p, y = (q / p) % p, z = q / (p * p);
+          const int e = (z * pe + (y + 2)) * pe + (x + 2);
+          mixed_out(ext, e, 1, cmix, cmixf, f32, mix, np, pbase, slot + 1, q);
+          mixed_out(ext, e, pe, cmix, cmixf, f32, mix, np, pbase, slot + 2, q);
+        }
+      }
+      if (!RAW) {
+        __syncthreads();  // the exponents take the widened region's place
+        for (int t = threadIdx.x; t < T3; t += THREADS) {
+          unsigned e;
+          reinterpret_cast<long long *>(ts)[t] = fx_word(ts[t], e);
+          ex[t] = e;
+        }
+        __syncthreads();
+      }
+    }
+    const bool f32 = der_f32(MIXED, v);
+    double *dd = der + (MIXED ? (v == ALPHA ? 0 : 7) : 4 * v) * np + pbase;
+    double *dp = MIXED ? dd + 4 * np : der + (4 * NF + 3 * (second ? slot / 3 : 0)) * np + pbase;
+    float *fd = reinterpret_cast<float *>(der + DER_D * np) + (long long)(4 * der_f(v)) * np + pbase;
+    float *fp = reinterpret_cast<float *>(der + DER_D * np) + (long long)(DER_F + 3 * der_f2(v)) * np + pbase;
+    auto each = [&](auto is_second, auto zero) {
+      using O = decltype(zero);
+      constexpr bool SECOND = decltype(is_second)::value;
+      auto point = [&](int q, int c0) {
+        O o[7];
+        if constexpr (RAW) point_sums_raw<SECOND, O>(ts + c0, T, o);
+        else point_sums<SECOND, O>(reinterpret_cast<const long long *>(ts) + c0, ex + c0, T, o);
+        O *a, *b;
+        if constexpr (std::is_same<O, float>::value) {
+          a = fd + q;
+          b = fp + q;
+        } else {
+          a = dd + q;
+          b = dp + q;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k * np] = o[k];
+        if (SECOND) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) b[k * np] = o[4 + k];
+        }
+      };
+      if (PF > 0) {
+#pragma unroll 1
+        for (int r = 0, q = threadIdx.x; r < ROUNDS; ++r, q += THREADS) {
+          int c0 = at[0];
+#pragma unroll
+          for (int s = 1; s < ROUNDS; ++s) c0 = r == s ? at[s] : c0;
+          if (q < p3) point(q, c0);
+        }
+      } else {
+        for (int q = threadIdx.x; q < p3; q += THREADS) point(q, centre_at(q));
+      }
+    };
+    if constexpr (NF != NV) {
+      each(std::false_type(), 0.0);
+    } else if constexpr (MIXED) {
+      if (!f32) each(std::true_type(), 0.0);
+      else if (second) each(std::true_type(), 0.0f);
+      else each(std::false_type(), 0.0f);
+    } else {
+      if (second) each(std::true_type(), 0.0);
+      else each(std::false_type(), 0.0);
+    }
+  }
+}
+
+}  // namespace
+
+}  // namespace ccz4

@@ -48,31 +48,27 @@ cudaError_t launch_ghost_setup(const GridView &g, GhostGeo *out, cudaStream_t s)
   return cudaGetLastError();
 }
 
-cudaError_t launch_stage_uniform(const GridView &g, const ccz4_params &P, int stage, const double *tile,
-                                 const double *mix, const double *in, const double *ini, const StageArgs &a,
-                                 cudaStream_t s) {
-  return launch_stage<false>(g, P, stage, tile, mix, in, ini, a, s);
+cudaError_t launch_stage_uniform(const GridView &g, const ccz4_params &P, int stage, const StageBufs &b,
+                                 const StageArgs &a, cudaStream_t s) {
+  return launch_stage<false>(g, P, stage, b, a, s);
 }
 
-static cudaError_t dispatch(const GridView &g, const ccz4_params &P, int stage, const double *tile,
-                            const double *mix, const double *in, const double *ini, const StageArgs &a,
+static cudaError_t dispatch(const GridView &g, const ccz4_params &P, int stage, const StageBufs &b, const StageArgs &a,
                             cudaStream_t s) {
-  if (g.src) return launch_stage_mesh(g, P, stage, tile, mix, in, ini, a, s);
-  return launch_stage_uniform(g, P, stage, tile, mix, in, ini, a, s);
+  if (g.src) return launch_stage_mesh(g, P, stage, b, a, s);
+  return launch_stage_uniform(g, P, stage, b, a, s);
 }
 
-cudaError_t launch_rhs(const GridView &g, const ccz4_params &P, const double *tile, const double *mix,
-                       const double *in, const double *ini, double *out, cudaStream_t s) {
-  StageArgs a{nullptr, nullptr, out, 0.0};
-  return dispatch(g, P, -1, tile, mix, in, ini, a, s);
+cudaError_t launch_rhs(const GridView &g, const ccz4_params &P, const double *der, const double *mix, const double *in,
+                       const double *ini, double *out, cudaStream_t s) {
+  return dispatch(g, P, -1, StageBufs{der, mix, in, ini}, StageArgs{nullptr, nullptr, out, 0.0}, s);
 }
 
-cudaError_t launch_rk_stage(const GridView &g, const ccz4_params &P, int stage, double dt,
-                            const double *tile, const double *mix, const double *in, const double *ini,
-                            const double *U, double *acc, double *out, cudaStream_t s) {
+cudaError_t launch_rk_stage(const GridView &g, const ccz4_params &P, int stage, double dt, const double *der,
+                            const double *mix, const double *in, const double *ini, const double *U, double *acc,
+                            double *out, cudaStream_t s) {
   if (stage < 0 || stage > 3) return cudaErrorInvalidValue;
-  StageArgs a{U, acc, out, dt};
-  return dispatch(g, P, stage, tile, mix, in, ini, a, s);
+  return dispatch(g, P, stage, StageBufs{der, mix, in, ini}, StageArgs{U, acc, out, dt}, s);
 }
 
 }  // namespace ccz4

@@ -1,19 +1,17 @@
 // One launch per RK stage (CCZ4_LAUNCH_FUSED): a cooperative kernel whose
-// blocks first fill the halo'd tiles of all patches (one patch per block at
-// a time, the fill of halo.cu), wait for one another at a grid-wide barrier,
-// then evolve the interior points (32-point items per warp, strided over the
-// grid) and the Sommerfeld ghost cells. This is the paper's enclave
+// blocks first take the derivatives of all patches (one patch per block at
+// a time, the pass of derive.cuh), wait for one another at a grid-wide barrier,
+// then evolve the Sommerfeld ghost cells and the interior points (items of 32
+// per warp, strided over the grid). This is the paper's enclave
 // batching taken to a whole stage: every patch of every level in one task.
-// Compiled for 9^3 patches (the stage kernel's instance for that edge) and
+// Compiled for 9^3 patches (the derivative pass's instance for that edge) and
 // the RK stages; the restriction after a step stays its own launch.
 //
-// The mixed derivatives are written by the fill phase of the same launch, so
-// they are read back with coherent loads (not the read-only path); the tiles
-// already are (streaming loads), and the grid barrier orders them.
-#define CCZ4_MIX_LOAD __ldcg
+// The derivatives are written by the first phase of the same launch, so they
+// are read back with coherent loads through L2; the grid barrier orders them.
+#define CCZ4_DER_LOAD __ldcg
 #include <cooperative_groups.h>
 
-#include "halo_fill.cuh"
 #include "stage_kernels.cuh"
 
 namespace ccz4 {
@@ -24,27 +22,29 @@ constexpr int FUSED_PF = 9;
 
 template <int MODE, class R, bool MESH>
 __global__ void __launch_bounds__(FUSED_THREADS, (StageBlocks<R, 0>::value))
-    fused_stage_kernel(GridView g, Phys<R> P, LevelCoef<R> LC, LevelScale ls, ccz4_params Pg,
-                       const double *__restrict__ in, const double *__restrict__ ini, double *tile, double *mix,
-                       StageArgs a) {
+    fused_stage_kernel(GridView g, Phys<R> P, LevelCoef<R> LC, LevelScale ls, ccz4_params Pg, FieldList fl,
+                       double *tile, double *mix, double *der, const double *__restrict__ in,
+                       const double *__restrict__ ini, StageArgs a) {
   extern __shared__ double smem[];
-  constexpr bool F32W = std::is_same<R, float>::value;
   for (int n = blockIdx.x; n < g.n_patches; n += gridDim.x) {
-    fill_patch<MESH, F32W, FUSED_THREADS, 8, FUSED_PF>(g, in, tile, mix, ls, n, smem);
+    derive_patch<MESH ? FROM_MESH : FROM_LEVEL, std::is_same<R, float>::value, false, FUSED_THREADS, FUSED_PF, NV>(
+        g, in, tile, mix, der, ls, fl, n, 0, 1, false, smem);
     __syncthreads();  // the next patch's source table overwrites this one's shared memory
   }
   cooperative_groups::this_grid().sync();
+  const StageBufs b{der, mix, in, ini};
   const int lane = threadIdx.x & 31;
-  const long long warps = (long long)gridDim.x * (FUSED_THREADS / 32);
-  for (long long item = (long long)blockIdx.x * (FUSED_THREADS / 32) + threadIdx.x / 32; item * 32 < g.n_points;
+  const long long warps = (long long)gridDim.x * (FUSED_THREADS / 32), gi = (g.n_ghost + 31) / 32;
+  for (long long item = (long long)blockIdx.x * (FUSED_THREADS / 32) + threadIdx.x / 32; (item - gi) * 32 < g.n_points;
        item += warps) {
-    const long long i = item * 32 + lane;
-    if (i < g.n_points) stage_point<MODE, R, MESH, FUSED_PF>(g, P, LC, tile, mix, a, i);
+    if (item < gi) {
+      const long long id = item * 32 + lane;
+      if (id < g.n_ghost) ghost_cell<MODE>(g, Pg, b, a, id);
+    } else {
+      const long long i = (item - gi) * 32 + lane;
+      if (i < g.n_points) stage_point<MODE, R, MESH>(g, P, LC, b, a, i);
+    }
   }
-  const long long total = g.n_ghost * NV;
-  for (long long q = (long long)blockIdx.x * FUSED_THREADS + threadIdx.x; q < total;
-       q += (long long)gridDim.x * FUSED_THREADS)
-    ghost_point<MODE>(g, Pg, in, ini, a, q % g.n_ghost, (int)(q / g.n_ghost));
 }
 
 template <int MODE, class R, bool MESH>
@@ -69,28 +69,24 @@ const void *fused_any(int mode, bool mixed, bool mesh) {
 }
 
 template <int MODE, class R, bool MESH>
-cudaError_t launch_fused_as(const GridView &g, const ccz4_params &P, double *tile, double *mix, const double *in,
-                            const double *ini, const StageArgs &a, cudaStream_t s) {
+cudaError_t launch_fused_as(const GridView &g, const ccz4_params &P, double *tile, double *mix, double *der,
+                            const double *in, const double *ini, const StageArgs &a, cudaStream_t s) {
   const void *fn = fused_fn<MODE, R, MESH>();
-  const size_t smem = fill_smem_bytes(FUSED_PF);
+  const size_t smem = derive_smem_bytes(FUSED_PF, false);
   int dev = 0, sms = 0, occ = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, FUSED_THREADS, smem);
   if (e != cudaSuccess) return e;
   if (occ < 1) return cudaErrorInvalidConfiguration;
-  LevelCoef<R> LC;
-  for (int l = 0; l < MAX_LEVELS; ++l) {
-    const StencilCoef<double> C = coefs(g.ldx[l], P);
-    LC.C[l] = C;
-    LC.CR[l] = StencilCoef<R>{R(C.c1), R(C.c2), R(C.c3), R(C.cko)};
-  }
+  LevelCoef<R> LC = level_coefs<R>(g, P);
+  FieldList fl = all_fields();
   GridView gv = g;
   Phys<R> ph = make_phys<R>(P);
   LevelScale ls = level_scale(g);
   ccz4_params Pg = P;
   StageArgs av = a;
-  void *args[] = {&gv, &ph, &LC, &ls, &Pg, (void *)&in, (void *)&ini, &tile, &mix, &av};
+  void *args[] = {&gv, &ph, &LC, &ls, &Pg, &fl, &tile, &mix, &der, (void *)&in, (void *)&ini, &av};
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;  // all blocks resident: the grid barrier may wait for every one
@@ -105,20 +101,20 @@ cudaError_t launch_fused_as(const GridView &g, const ccz4_params &P, double *til
 }
 
 template <int MODE>
-cudaError_t launch_fused_mode(const GridView &g, const ccz4_params &P, double *tile, double *mix, const double *in,
-                              const double *ini, const StageArgs &a, cudaStream_t s) {
+cudaError_t launch_fused_mode(const GridView &g, const ccz4_params &P, double *tile, double *mix, double *der,
+                              const double *in, const double *ini, const StageArgs &a, cudaStream_t s) {
   const bool mixed = P.precision == CCZ4_PREC_MIXED, mesh = g.src != nullptr;
   if (mixed)
-    return mesh ? launch_fused_as<MODE, float, true>(g, P, tile, mix, in, ini, a, s)
-                : launch_fused_as<MODE, float, false>(g, P, tile, mix, in, ini, a, s);
-  return mesh ? launch_fused_as<MODE, double, true>(g, P, tile, mix, in, ini, a, s)
-              : launch_fused_as<MODE, double, false>(g, P, tile, mix, in, ini, a, s);
+    return mesh ? launch_fused_as<MODE, float, true>(g, P, tile, mix, der, in, ini, a, s)
+                : launch_fused_as<MODE, float, false>(g, P, tile, mix, der, in, ini, a, s);
+  return mesh ? launch_fused_as<MODE, double, true>(g, P, tile, mix, der, in, ini, a, s)
+              : launch_fused_as<MODE, double, false>(g, P, tile, mix, der, in, ini, a, s);
 }
 
 }  // namespace
 
 cudaError_t prepare_fused() {
-  const int bytes = (int)fill_smem_bytes(FUSED_PF);
+  const int bytes = (int)derive_smem_bytes(FUSED_PF, false);
   for (int m = 0; m < 4; ++m)
     for (int x = 0; x < 2; ++x)
       for (int h = 0; h < 2; ++h) {
@@ -129,15 +125,15 @@ cudaError_t prepare_fused() {
 }
 
 cudaError_t launch_fused_stage(const GridView &g, const ccz4_params &P, int stage, double dt, double *tile,
-                               double *mix, const double *in, const double *ini, const double *U, double *acc,
-                               double *out, cudaStream_t s) {
+                               double *mix, double *der, const double *in, const double *ini, const double *U,
+                               double *acc, double *out, cudaStream_t s) {
   if (g.p != FUSED_PF || stage < 0 || stage > 3) return cudaErrorInvalidValue;
   const StageArgs a{U, acc, out, dt};
   switch (stage) {
-    case 0: return launch_fused_mode<0>(g, P, tile, mix, in, ini, a, s);
-    case 1: return launch_fused_mode<1>(g, P, tile, mix, in, ini, a, s);
-    case 2: return launch_fused_mode<2>(g, P, tile, mix, in, ini, a, s);
-    default: return launch_fused_mode<3>(g, P, tile, mix, in, ini, a, s);
+    case 0: return launch_fused_mode<0>(g, P, tile, mix, der, in, ini, a, s);
+    case 1: return launch_fused_mode<1>(g, P, tile, mix, der, in, ini, a, s);
+    case 2: return launch_fused_mode<2>(g, P, tile, mix, der, in, ini, a, s);
+    default: return launch_fused_mode<3>(g, P, tile, mix, der, in, ini, a, s);
   }
 }
 
