@@ -5,15 +5,15 @@
 //
 // A ccz4_fo holds 58-field state buffers on the geometry of a grid (its
 // patches, neighbour lookup and Sommerfeld ghost shell). Per RK4 stage:
-//  - first order: one halo fill of all 58 fields, the stage kernel (every
-//    variable evolved, red terms kept), the ghost-cell kernel;
-//  - second order with reconstruction: a halo fill of the 25 primaries, the
-//    reconstruction kernel (the auxiliary variables of every interior point
-//    from FD4 derivatives of the primaries, written into the stage's input),
-//    a halo fill of the 33 auxiliary variables, the stage kernel (the
-//    primaries evolved without red terms), the ghost-cell kernel; after the
-//    last stage the auxiliary variables are reconstructed from the new
-//    primaries. This is the extra mesh sweep the paper's second-order
+//  - first order: the derivative pass (derive.cuh) over all 58 fields, the
+//    stage kernel (every variable evolved, red terms kept; ghost cells too);
+//  - second order with reconstruction: the derivative pass over the 25
+//    primaries, the reconstruction kernel (the auxiliary variables of every
+//    interior point from the FD4 derivatives of the primaries, written into
+//    the stage's input), the derivative pass over the 33 auxiliary variables,
+//    the stage kernel (the primaries evolved without red terms; ghost cells
+//    too); after the last stage the auxiliary variables are reconstructed
+//    from the new primaries. This is the extra mesh sweep the paper's second-order
 //    formulation needs.
 // The ghost cells of every variable follow the radiative condition of the
 // Sommerfeld boundary (speed somm_speed[v] for the primaries, 1 for the
@@ -25,117 +25,34 @@
 namespace ccz4 {
 namespace {
 
-constexpr int FO_FILL_THREADS = 256;
-
-// Tile of fields [v0, v0 + nv) of a [58][S] state: [58][n_patches][T^3].
-__global__ void __launch_bounds__(FO_FILL_THREADS) fo_fill_kernel(GridView g, const double *__restrict__ src,
-                                                                  double *__restrict__ tile, int v0, int nv) {
-  extern __shared__ long long fo_idx[];
-  const int n = blockIdx.x;
-  const int p = g.p, T = g.T, T3 = (int)g.T3;
-  const int bx = __ldg(g.ijk + 3 * n) * p - HALO, by = __ldg(g.ijk + 3 * n + 1) * p - HALO,
-            bz = __ldg(g.ijk + 3 * n + 2) * p - HALO;
-  for (int t = threadIdx.x; t < T3; t += blockDim.x) {
-    const int lz = t / (T * T), ly = (t / T) % T, lx = t % T;
-    fo_idx[t] = locate(g, bx + lx, by + ly, bz + lz);
-  }
-  __syncthreads();
-  for (int v = v0; v < v0 + nv; ++v) {
-    const double *sv = src + v * g.S;
-    double *tv = tile + ((long long)v * g.n_patches + n) * g.T3;
-    for (int t = threadIdx.x; t < T3; t += blockDim.x) {
-      const long long s = fo_idx[t];
-      tv[t] = s >= 0 ? __ldg(sv + s) : 0.0;
-    }
-  }
-}
-
-
-
 // One thread per interior point: its auxiliary variables from the primaries'
-// tile, written into the state `out`.
-__global__ void __launch_bounds__(128) fo_reconstruct_kernel(GridView g, const double *__restrict__ tile,
+// first derivatives, written into the state `out`.
+__global__ void __launch_bounds__(128) fo_reconstruct_kernel(GridView g, const double *__restrict__ der,
                                                              double *__restrict__ out, double c1) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.n_points) return;
-  const Nbhd N = fo_nbhd(g, tile, i);
+  const FoView N = fo_view(g, der, out, i);
   const long long S = g.S;
   auto put = [&](int v, double val) { out[v * S + i] = val; };
   fo_reconstruct_point(N, c1, put);
 }
 
-// One thread per (Sommerfeld ghost cell, variable): the radiative condition
-// (Eq. exa_sommerfeld_inter) with the cell's static geometry, and the stage
-// update.
-template <int MODE>
-__global__ void __launch_bounds__(256) fo_ghost_kernel(GridView g, ccz4_params P, const double *__restrict__ in,
-                                                       const double *__restrict__ ini, FoStageArgs a) {
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int v = blockIdx.y;
-  if (id >= g.n_ghost) return;
-  const GhostGeo *gg = g.ghost_geo + id;
-  const long long sn = __ldg(&gg->sn);
-  if (sn < 0) return;
-  const double geo = __ldg(&gg->geo), ir = __ldg(&gg->ir);
-  double cv = 1.0;  // selected with static indices (no local copy of the parameters)
-#pragma unroll
-  for (int q = 0; q < NV; ++q)
-    if (q == v) cv = P.somm_speed[q];
-  const long long o = v * g.S + g.n_points + id;
-  const double qg = __ldg(in + o);
-  const double qn = __ldg(in + v * g.S + sn);
-  const double k = -cv * geo * (qg - qn) - cv * ir * (qg - __ldg(ini + o));
-  if (MODE < 0) {
-    a.out[o] = k;
-    return;
-  }
-  double acc = MODE == 0 ? 0.0 : a.acc[o];
-  const double un = rk_combine<(MODE < 0 ? 0 : MODE), double>(a.U[o], acc, k, a.dt);
-  if (MODE < 3) a.acc[o] = acc;
-  a.out[o] = un;
-}
-
-
-template <int MODE, bool RED, bool AUX>
-cudaError_t launch_interior(const GridView &g, const ccz4_params &P, const double *tile, const FoStageArgs &a,
-                            cudaStream_t s) {
-  if (g.p == 9)  // the paper's patch edge, with its strides compiled in
-    return launch_fo_interior_p9(MODE, RED, AUX, g, P, tile, a, s);
-  return launch_fo_interior_pf<MODE, RED, AUX, 0>(g, P, tile, a, s);
-}
-
-template <int MODE>
-cudaError_t launch_ghost(const GridView &g, const ccz4_params &P, const double *in, const double *ini,
-                         const FoStageArgs &a, cudaStream_t s) {
-  if (g.n_ghost == 0) return cudaSuccess;
-  const dim3 grid((unsigned)((g.n_ghost + 255) / 256), NVF);
-  fo_ghost_kernel<MODE><<<grid, 256, 0, s>>>(g, P, in, ini, a);
-  return cudaGetLastError();
-}
-
 // stage -1: plain right-hand side (all 58, red terms per `red`); 0..3: RK4 stage
 template <int MODE>
-cudaError_t launch_fo_mode(const GridView &g, const ccz4_params &P, bool first_order, const double *tile,
+cudaError_t launch_fo_mode(const GridView &g, const ccz4_params &P, bool first_order, const double *der,
                            const double *in, const double *ini, const FoStageArgs &a, cudaStream_t s) {
-  cudaError_t e;
-  if (MODE < 0)
-    e = first_order ? launch_interior<MODE, true, true>(g, P, tile, a, s)
-                    : launch_interior<MODE, false, true>(g, P, tile, a, s);
-  else
-    e = first_order ? launch_interior<MODE, true, true>(g, P, tile, a, s)
-                    : launch_interior<MODE, false, false>(g, P, tile, a, s);
-  if (e != cudaSuccess) return e;
-  return launch_ghost<MODE>(g, P, in, ini, a, s);
+  return first_order ? launch_fo_interior<MODE, true, true>(g, P, der, in, ini, a, s)
+                     : launch_fo_interior<MODE, false, (MODE < 0)>(g, P, der, in, ini, a, s);
 }
 
-cudaError_t launch_fo(int stage, const GridView &g, const ccz4_params &P, bool first_order, const double *tile,
+cudaError_t launch_fo(int stage, const GridView &g, const ccz4_params &P, bool first_order, const double *der,
                       const double *in, const double *ini, const FoStageArgs &a, cudaStream_t s) {
   switch (stage) {
-    case -1: return launch_fo_mode<-1>(g, P, first_order, tile, in, ini, a, s);
-    case 0: return launch_fo_mode<0>(g, P, first_order, tile, in, ini, a, s);
-    case 1: return launch_fo_mode<1>(g, P, first_order, tile, in, ini, a, s);
-    case 2: return launch_fo_mode<2>(g, P, first_order, tile, in, ini, a, s);
-    case 3: return launch_fo_mode<3>(g, P, first_order, tile, in, ini, a, s);
+    case -1: return launch_fo_mode<-1>(g, P, first_order, der, in, ini, a, s);
+    case 0: return launch_fo_mode<0>(g, P, first_order, der, in, ini, a, s);
+    case 1: return launch_fo_mode<1>(g, P, first_order, der, in, ini, a, s);
+    case 2: return launch_fo_mode<2>(g, P, first_order, der, in, ini, a, s);
+    case 3: return launch_fo_mode<3>(g, P, first_order, der, in, ini, a, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -149,7 +66,7 @@ struct ccz4_fo {
   ccz4_grid *g;
   int variant;
   double *buf[6];  // U, Y0, Y1, ACC, RHS, INI: [58][S]
-  double *tile;    // [58][n_patches][T^3]
+  double *der;     // derivative buffer, [4 x 58][n_points]
 };
 
 static const int kFoIn[4] = {CCZ4_BUF_U, CCZ4_BUF_Y0, CCZ4_BUF_Y1, CCZ4_BUF_Y0};
@@ -167,24 +84,23 @@ static const int kFoOut[4] = {CCZ4_BUF_Y0, CCZ4_BUF_Y1, CCZ4_BUF_Y0, CCZ4_BUF_U}
 static void fo_release(ccz4_fo *f) {
   if (!f) return;
   for (double *b : f->buf) cudaFree(b);
-  cudaFree(f->tile);
+  cudaFree(f->der);
   free(f);
 }
 
-static size_t fo_fill_smem(const GridView &v) { return sizeof(long long) * (size_t)v.T3; }
-
-static cudaError_t fo_fill(const ccz4_fo *f, const double *src, int v0, int nv, cudaStream_t s) {
-  const GridView &v = f->g->v;
-  if (v.n_patches == 0) return cudaSuccess;
-  fo_fill_kernel<<<v.n_patches, FO_FILL_THREADS, fo_fill_smem(v), s>>>(v, src, f->tile, v0, nv);
-  return cudaGetLastError();
+// The derivative pass over fields [v0, v0 + nv).
+static cudaError_t fo_derive(const ccz4_fo *f, const double *src, int v0, int nv, cudaStream_t s) {
+  FieldList fl;
+  fl.n = nv;
+  for (int k = 0; k < nv; ++k) fl.f[k] = (unsigned char)(v0 + k);
+  return launch_derive_fo(f->g->v, src, f->der, fl, s);
 }
 
 static cudaError_t fo_reconstruct_into(const ccz4_fo *f, double *state, cudaStream_t s) {
   const GridView &v = f->g->v;
-  cudaError_t e = fo_fill(f, state, 0, NV, s);
+  cudaError_t e = fo_derive(f, state, 0, NV, s);
   if (e != cudaSuccess || v.n_points == 0) return e;
-  fo_reconstruct_kernel<<<(unsigned)((v.n_points + 127) / 128), 128, 0, s>>>(v, f->tile, state, 1.0 / (12.0 * v.dx));
+  fo_reconstruct_kernel<<<(unsigned)((v.n_points + 127) / 128), 128, 0, s>>>(v, f->der, state, 1.0 / (12.0 * v.dx));
   return cudaGetLastError();
 }
 
@@ -231,15 +147,14 @@ extern "C" ccz4_status ccz4_fo_alloc(ccz4_grid *g, int variant, ccz4_fo **out) {
       return CCZ4_ERR_NOMEM;
     }
   }
-  const size_t tile = sizeof(double) * (size_t)NVF * (size_t)v.n_patches * (size_t)v.T3;
-  if (cudaMalloc(&f->tile, tile) != cudaSuccess) {
-    set_error("fo_alloc: cudaMalloc of the %zu-byte tile failed: %s", tile, cudaGetErrorString(cudaGetLastError()));
+  const size_t der = sizeof(double) * 4 * (size_t)NVF * (size_t)v.n_points;
+  if (der && cudaMalloc(&f->der, der) != cudaSuccess) {
+    set_error("fo_alloc: cudaMalloc of the %zu-byte derivative buffer failed: %s", der,
+              cudaGetErrorString(cudaGetLastError()));
     fo_release(f);
     return CCZ4_ERR_NOMEM;
   }
-  cudaError_t e = cudaFuncSetAttribute((const void *)fo_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fo_fill_smem(v));
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     set_error("fo_alloc: set-up failed: %s", cudaGetErrorString(e));
     fo_release(f);
@@ -309,27 +224,27 @@ extern "C" ccz4_status ccz4_fo_rhs(ccz4_fo *f, const ccz4_params *P, int in_buf,
   }
   cudaStream_t s = (cudaStream_t)stream;
   const double *in = f->buf[in_buf];
-  FO_TRY(fo_fill(f, in, 0, NVF, s));
+  FO_TRY(fo_derive(f, in, 0, NVF, s));
   FoStageArgs a{nullptr, nullptr, f->buf[out_buf], 0.0};
-  FO_TRY(launch_fo(-1, f->g->v, *P, f->variant == CCZ4_FO_FIRST_ORDER, f->tile, in, fo_ini(f), a, s));
+  FO_TRY(launch_fo(-1, f->g->v, *P, f->variant == CCZ4_FO_FIRST_ORDER, f->der, in, fo_ini(f), a, s));
   return CCZ4_OK;
 }
 
-// One RK4 stage: the fills (and, second order, the reconstruction), the
-// stage kernel and the ghost cells; stage 3 ends the step (enforcement in
+// One RK4 stage: the derivatives (and, second order, the reconstruction) and
+// the stage kernel; stage 3 ends the step (enforcement in
 // the stage kernel; second order: the auxiliary variables of U_{n+1}
 // reconstructed).
 static ccz4_status fo_stage(ccz4_fo *f, const ccz4_params *P, int stage, double dt, cudaStream_t s) {
   double *in = f->buf[kFoIn[stage]];
   const bool first = f->variant == CCZ4_FO_FIRST_ORDER;
   if (first) {
-    FO_TRY(fo_fill(f, in, 0, NVF, s));
+    FO_TRY(fo_derive(f, in, 0, NVF, s));
   } else {
     FO_TRY(fo_reconstruct_into(f, in, s));
-    FO_TRY(fo_fill(f, in, NV, NVF - NV, s));
+    FO_TRY(fo_derive(f, in, NV, NVF - NV, s));
   }
   FoStageArgs a{f->buf[CCZ4_BUF_U], f->buf[CCZ4_BUF_ACC], f->buf[kFoOut[stage]], dt};
-  FO_TRY(launch_fo(stage, f->g->v, *P, first, f->tile, in, fo_ini(f), a, s));
+  FO_TRY(launch_fo(stage, f->g->v, *P, first, f->der, in, fo_ini(f), a, s));
   if (stage == 3 && !first) FO_TRY(fo_reconstruct_into(f, f->buf[CCZ4_BUF_U], s));
   return CCZ4_OK;
 }

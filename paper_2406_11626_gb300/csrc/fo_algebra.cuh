@@ -27,12 +27,10 @@
 namespace ccz4 {
 
 // Index of a symmetric pair for the first-order algebra: the same table as
-// S6, in the recursive form on purpose. The first-order stage kernel runs
-// at 128 registers and spills several KB per thread; with this form the
-// arrays it indexes keep fixed places in local memory instead of being
-// allocated to registers and spilled, which measured 3.5 % faster per step
-// (144^3 puncture: 104.1 against 107.9 ms). The second-order kernels use
-// S6, whose indices fold so that their arrays stay in registers.
+// S6, in the recursive form, with which the arrays it indexes keep fixed
+// places in local memory instead of being allocated to registers and spilled
+// (first-order step at 90^3: 19.23 against 19.49 ms with S6; reconstructed
+// second order 13.58 against 13.44 ms).
 __host__ __device__ constexpr int S6_fo(int i, int j) {
   return i > j ? S6_fo(j, i) : (i == 0 ? j : (i == 1 ? 2 + j : 5));
 }
@@ -45,8 +43,9 @@ struct FoPhys {
   double mu;
 };
 
-template <bool RED, bool AUX, class Sink>
-__device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const Nbhd &N, const StencilCoef<double> &C,
+// NB: the point's view of the derivative buffer (FoView, fo_stage.cuh).
+template <bool RED, bool AUX, class Sink, class NB>
+__device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const StencilCoef<double> &C,
                                              Sink &sink) {
   using D = double;
   const Phys<D> &P = F.p;
@@ -536,8 +535,8 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const Nbhd &N, con
 // Auxiliary variables of one point from FD4 first derivatives of the
 // primaries (the reconstruction of Alg. fd4-so, Eq. auxiliary-variables):
 // out(v, value) receives A_k, B_k^i, D_kij = 1/2 d_k g~_ij and P_k.
-template <class Out>
-__device__ __forceinline__ void fo_reconstruct_point(const Nbhd &N, const double c1, Out &out) {
+template <class Out, class NB>
+__device__ __forceinline__ void fo_reconstruct_point(const NB &N, const double c1, Out &out) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const int s = N.st[k];

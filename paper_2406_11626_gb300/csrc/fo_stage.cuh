@@ -1,9 +1,8 @@
-// The stage kernel of the 58-variable formulations (ccz4_fo_*), shared by
-// fo.cu (the general instance) and fo_p9.cu (the instance compiled for 9^3
-// patches), so that the two compile in parallel.
+// The stage kernel of the 58-variable formulations (ccz4_fo_*).
 #ifndef CCZ4_FO_STAGE_CUH
 #define CCZ4_FO_STAGE_CUH
 
+#include "derive.h"
 #include "fo_algebra.cuh"
 
 #ifndef CCZ4_FO_MIN_BLOCKS
@@ -58,40 +57,72 @@ struct FoSink {
   }
 };
 
-// PF > 0: the patch edge is PF (the grid's p must equal it), so the tile
-// strides and the index divisions are compile-time constants.
-template <int PF = 0>
-__device__ __forceinline__ Nbhd fo_nbhd(const GridView &g, const double *tile, long long i) {
-  const int p = PF > 0 ? PF : g.p, T = PF > 0 ? PF + 2 * HALO : g.T;
-  const long long T3 = PF > 0 ? (long long)T * T * T : g.T3;
-  const int p3 = p * p * p;
-  const int n = (int)i / p3;
-  const int r = (int)(i - (long long)n * p3);
-  const int z = r / (p * p), y = (r / p) % p, x = r % p;
-  Nbhd N;
-  N.c = tile + n * T3 + ((long long)(z + HALO) * T + (y + HALO)) * T + (x + HALO);
-  N.fs = (long long)g.n_patches * T3;
-  N.st[0] = 1;
-  N.st[1] = T;
-  N.st[2] = T * T;
-  N.mix = nullptr;
-  N.ms = 0;
-  N.mixf = nullptr;
-  N.msf = 0;
-  return N;
+// One point's view of the state and of the derivative buffer (derive.h: slot
+// 4 v + k the first-derivative sum of field v along axis k, 4 v + 3 its
+// dissipation sum); the strides are the axes.
+struct FoView {
+  const double *c;   // field 0 of the state at the point
+  const double *d;   // slot 0 at the point
+  long long S, np;
+  int st[3];
+};
+template <class D>
+__device__ __forceinline__ D ld(const FoView &N, int v, int) { return N.c[v * N.S]; }
+template <class D>
+__device__ __forceinline__ D fd1(const FoView &N, int v, int axis, const D &c1) {
+  return __ldcs(N.d + (4 * v + axis) * N.np) * c1;
+}
+template <class D>
+__device__ __forceinline__ D ko_sum(const FoView &N, int v) { return __ldcs(N.d + (4 * v + 3) * N.np); }
+
+__device__ __forceinline__ FoView fo_view(const GridView &g, const double *der, const double *in, long long i) {
+  return FoView{in + i, der + i, g.S, g.n_points, {0, 1, 2}};
 }
 
-// One thread per interior point: the 58-variable right-hand side (RED: with
-// the red terms; AUX: the auxiliary variables' equations too) and the stage
-// update of what it evolves.
-template <int MODE, bool RED, bool AUX, int PF = 0>
-__global__ void __launch_bounds__(128, CCZ4_FO_MIN_BLOCKS) fo_interior_kernel(GridView g, FoPhys F,
-                                                                             StencilCoef<double> C,
-                                                                             const double *__restrict__ tile,
-                                                                             FoStageArgs a) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// All variables of one Sommerfeld ghost cell: the radiative condition (Eq.
+// exa_sommerfeld_inter) with the cell's static geometry, and the stage
+// update.
+template <int MODE>
+__device__ __forceinline__ void fo_ghost_cell(const GridView &g, const ccz4_params &P, const double *__restrict__ in,
+                                              const double *__restrict__ ini, const FoStageArgs &a, long long id) {
+  const GhostGeo *gg = g.ghost_geo + id;
+  const long long sn = __ldg(&gg->sn);
+  if (sn < 0) return;
+  const double geo = __ldg(&gg->geo), ir = __ldg(&gg->ir);
+#pragma unroll 4
+  for (int v = 0; v < NVF; ++v) {
+    const double cv = v < NV ? P.somm_speed[v] : 1.0;
+    const long long o = v * g.S + g.n_points + id;
+    const double qg = __ldg(in + o);
+    const double qn = __ldg(in + v * g.S + sn);
+    const double k = -cv * geo * (qg - qn) - cv * ir * (qg - __ldg(ini + o));
+    if (MODE < 0) {
+      a.out[o] = k;
+      continue;
+    }
+    double acc = MODE == 0 ? 0.0 : a.acc[o];
+    const double un = rk_combine<(MODE < 0 ? 0 : MODE), double>(a.U[o], acc, k, a.dt);
+    if (MODE < 3) a.acc[o] = acc;
+    a.out[o] = un;
+  }
+}
+
+// The first ghost_blocks blocks: one thread per ghost cell. The others: one
+// thread per interior point, the 58-variable right-hand side (RED: with the
+// red terms; AUX: the auxiliary variables' equations too) from the derivative
+// buffer and the stage update of what it evolves.
+template <int MODE, bool RED, bool AUX>
+__global__ void __launch_bounds__(128, CCZ4_FO_MIN_BLOCKS)
+    fo_interior_kernel(GridView g, FoPhys F, StencilCoef<double> C, ccz4_params P, const double *__restrict__ der,
+                       const double *__restrict__ in, const double *__restrict__ ini, FoStageArgs a, int ghost_blocks) {
+  if ((int)blockIdx.x < ghost_blocks) {
+    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id < g.n_ghost) fo_ghost_cell<MODE>(g, P, in, ini, a, id);
+    return;
+  }
+  const long long i = (long long)(blockIdx.x - ghost_blocks) * blockDim.x + threadIdx.x;
   if (i >= g.n_points) return;
-  const Nbhd N = fo_nbhd<PF>(g, tile, i);
+  const FoView N = fo_view(g, der, in, i);
   FoSink<MODE> sink{g.S, i, a};
   fo_rhs_point<RED, AUX>(F, N, C, sink);
   sink.finish();
@@ -106,23 +137,20 @@ inline StencilCoef<double> fo_coefs(double dx, double eps) {
   return C;
 }
 
-// Launches the stage kernel of one (MODE, RED, AUX) on every interior point.
-template <int MODE, bool RED, bool AUX, int PF>
-cudaError_t launch_fo_interior_pf(const GridView &g, const ccz4_params &P, const double *tile, const FoStageArgs &a,
-                                  cudaStream_t s) {
-  if (g.n_points == 0) return cudaSuccess;
-  FoPhys F{make_phys<double>(P), P.mu};
-  fo_interior_kernel<MODE, RED, AUX, PF><<<(unsigned)((g.n_points + 127) / 128), 128, 0, s>>>(
-      g, F, fo_coefs(g.dx, P.ko_eps), tile, a);
+// Launches the stage kernel of one (MODE, RED, AUX) on every ghost cell and interior point.
+template <int MODE, bool RED, bool AUX>
+cudaError_t launch_fo_interior(const GridView &g, const ccz4_params &P, const double *der, const double *in,
+                               const double *ini, const FoStageArgs &a, cudaStream_t s) {
+  const FoPhys F{make_phys<double>(P), P.mu};
+  const int t = g.n_points < 16LL * 152 * 128 ? 32 : 128;  // a small grid spreads over the SMs in shares of 32 points
+  const long long gb = (g.n_ghost + t - 1) / t, nb = (g.n_points + t - 1) / t;
+  if (gb + nb == 0) return cudaSuccess;
+  fo_interior_kernel<MODE, RED, AUX><<<(unsigned)(gb + nb), t, 0, s>>>(g, F, fo_coefs(g.dx, P.ko_eps), P, der, in, ini, a,
+                                                                       (int)gb);
   return cudaGetLastError();
 }
 
 }  // namespace
-
-// The instance for 9^3 patches (fo_p9.cu): mode -1..3, red, aux as the template arguments above.
-cudaError_t launch_fo_interior_p9(int mode, bool red, bool aux, const GridView &g, const ccz4_params &P,
-                                  const double *tile, const FoStageArgs &a, cudaStream_t s);
-
 }  // namespace ccz4
 
 #endif
