@@ -357,6 +357,7 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
   }
   prepare_fill_halos(v.p);
   prepare_derive();
+  prepare_constraints();
   if (v.p == 9) prepare_fused();
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
@@ -832,6 +833,21 @@ extern "C" ccz4_status ccz4_point_index(ccz4_grid *g, int n, const int *xyz, lon
   return CCZ4_OK;
 }
 
+// The derivative pass of a monitor: the sums of g~, A~, phi, K and, for psi_4,
+// Gamma-hat; the tiles and mixed derivatives of every field, as the halo fill
+// of the buffer leaves them.
+static cudaError_t monitor_derivatives(ccz4_grid *g, int buf, bool gamma_hat, cudaStream_t s) {
+  FieldList fl = all_fields();
+  for (int k = 0; k < fl.n; ++k) {
+    const int v = fl.f[k];
+    const bool sums = (v >= GXX && v <= GZZ) || (v >= AXX && v <= AZZ) || v == PHI || v == KTR ||
+                      (gamma_hat && v >= GHX && v <= GHZ);
+    if (!sums) fl.f[k] |= FIELD_NO_SUMS;
+  }
+  return launch_derive(g->v, g->buf[buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der, fl, false, false, true,
+                       s);
+}
+
 extern "C" ccz4_status ccz4_psi4(ccz4_grid *g, int in_buf, int out_buf, const double centre[3], void *stream) {
   if (check_grid(g)) return CCZ4_ERR_INVALID;
   if (!state_buffer(in_buf) || !state_buffer(out_buf) || in_buf == out_buf || !g->buf[in_buf] ||
@@ -840,8 +856,8 @@ extern "C" ccz4_status ccz4_psi4(ccz4_grid *g, int in_buf, int out_buf, const do
     return CCZ4_ERR_INVALID;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  CUDA_TRY(launch_fill_halos(g->v, g->buf[in_buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], s));
-  CUDA_TRY(launch_psi4(g->v, g->buf[CCZ4_BUF_TILE], centre, g->buf[out_buf], s));
+  CUDA_TRY(monitor_derivatives(g, in_buf, true, s));
+  CUDA_TRY(launch_psi4(g->v, g->der, g->buf[CCZ4_BUF_MIX], g->buf[in_buf], centre, g->buf[out_buf], s));
   return CCZ4_OK;
 }
 
@@ -853,9 +869,9 @@ extern "C" ccz4_status ccz4_constraints(ccz4_grid *g, int buf, double out[5], do
     return CCZ4_ERR_INVALID;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  CUDA_TRY(launch_fill_halos(g->v, g->buf[buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], s));
-  CUDA_TRY(launch_constraints(g->v, g->buf[CCZ4_BUF_TILE], dev_H, dev_M, g->red_partial, g->red_blocks,
-                              g->red_out, s));
+  CUDA_TRY(monitor_derivatives(g, buf, false, s));
+  CUDA_TRY(launch_constraints_der(g->v, g->der, g->buf[CCZ4_BUF_MIX], g->buf[buf], dev_H, dev_M, g->red_partial,
+                                  g->red_blocks, g->red_out, s));
   CUDA_TRY(cudaMemcpyAsync(g->host_out, g->red_out, sizeof(double) * 5, cudaMemcpyDeviceToHost, s));
   unsigned status = 0;
   CUDA_TRY(cudaMemcpyAsync(&status, g->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, s));

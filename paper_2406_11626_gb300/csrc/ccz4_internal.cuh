@@ -232,9 +232,10 @@ cudaError_t prepare_fused();
 cudaError_t launch_fused_stage(const GridView &g, const ccz4_params &P, int stage, double dt, double *tile,
                                double *mix, double *der, const double *in, const double *ini, const double *U,
                                double *acc, double *out, cudaStream_t s);
-// psi_4 at every interior point from the halo'd tiles: Re into out[0 .. n_points), Im into out[S ..),
-// the tetrad centred at centre (psi4.cu)
-cudaError_t launch_psi4(const GridView &g, const double *tile, const double centre[3], double *out, cudaStream_t s);
+// psi_4 at every interior point from the derivative pass over `in`: Re into out[0 .. n_points), Im into
+// out[S ..), the tetrad centred at centre (psi4.cu)
+cudaError_t launch_psi4(const GridView &g, const double *der, const double *mix, const double *in,
+                        const double centre[3], double *out, cudaStream_t s);
 // number of mixed second derivatives kept per point (d_xy, d_xz, d_yz of g~, alpha, beta, phi)
 constexpr int NMIX = 33;
 // largest patch edge whose halo'd tile of one field fits in the fill kernel's shared memory
@@ -248,6 +249,10 @@ cudaError_t launch_enforce(const GridView &g, double *U, cudaStream_t s);
 // restriction of level l onto the n_par parents par[] of level l-1 (children kid[n_par][27])
 cudaError_t launch_restrict(const GridView &g, const int *par, const int *kid, int n_par, double *U,
                             cudaStream_t s);
+// constraint monitors from halo'd tiles alone, or from the derivative pass over `in`
 cudaError_t launch_constraints(const GridView &g, const double *tile, double *H, double *M,
                                double *partial, int blocks, double *out5, cudaStream_t s);
+cudaError_t prepare_constraints();
+cudaError_t launch_constraints_der(const GridView &g, const double *der, const double *mix, const double *in, double *H,
+                                   double *M, double *partial, int blocks, double *out5, cudaStream_t s);
 }  // namespace ccz4

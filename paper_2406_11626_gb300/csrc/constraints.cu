@@ -6,206 +6,165 @@
 // NR_foccz4_modified_ricci with Z = 0: Gamma-hat replaced by the contracted
 // Christoffel symbol G~^k of the metric, whose derivative is taken through
 // the closing relations (d_k g~^ij = -2 D_k^ij and the derivative of the
-// Christoffel symbols), i.e. from first and second derivatives of g~.
+// Christoffel symbols), i.e. from first and second derivatives of g~. Only
+// its trace enters H, and the trace needs no tensor: with G~_kij, G~^k_ij the
+// Christoffel symbols of g~ and G~_k = g~^ij G~_kij, the terms of the
+// contracted derivative cancel against the quadratic ones to
+//   g~^ij R~_ij = g~^kn g~^ml (d_k d_m g~_ln - d_k d_l g~_mn)
+//                 + g~^ij g~^ml G~^k_im G~_kjl - G~^k G~_k,
+// and with the conformal factor
+//   phi^2 g~^ij R_ij = phi^2 g~^ij R~_ij + 4 phi (g~^ij d_i d_j phi - G~^k d_k phi)
+//                      - 6 g~^ij d_i phi d_j phi.
 #include "ccz4_algebra.cuh"
+#include "der_view.cuh"
 
 namespace ccz4 {
 namespace {
 
 constexpr int RED_THREADS = 256;
 
-__device__ void constraints_point(const Nbhd &N, const StencilCoef<double> &C, double &H, double M[3]) {
-  double g[6], A[6];
+// NB: the point's derivatives (DerView), or its neighbourhood in halo'd tiles (Nbhd).
+template <class NB>
+__device__ __forceinline__ void constraints_point(const NB &N, const StencilCoef<double> &C, double &H, double M[3]) {
+  double g[6], ig[6];
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    g[c] = N.at(GXX + c, 0);
-    A[c] = N.at(AXX + c, 0);
-  }
-  const double ph = N.at(PHI, 0), Kt = N.at(KTR, 0);
-  double dg[3][6], dA[3][6], dP[3], dK[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int s = N.st[k];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      dg[k][c] = fd1<double>(N, GXX + c, s, C.c1);
-      dA[k][c] = fd1<double>(N, AXX + c, s, C.c1);
-    }
-    dP[k] = fd1<double>(N, PHI, s, C.c1);
-    dK[k] = fd1<double>(N, KTR, s, C.c1);
-  }
-  double ig[6];
-  ig[0] = g[3] * g[5] - g[4] * g[4];
-  ig[1] = g[2] * g[4] - g[1] * g[5];
-  ig[2] = g[1] * g[4] - g[2] * g[3];
-  ig[3] = g[0] * g[5] - g[2] * g[2];
-  ig[4] = g[1] * g[2] - g[0] * g[4];
-  ig[5] = g[0] * g[3] - g[1] * g[1];
-  const double idet = 1.0 / (g[0] * ig[0] + g[1] * ig[1] + g[2] * ig[2]);
-#pragma unroll
-  for (int c = 0; c < 6; ++c) ig[c] *= idet;
-  const double w6[6] = {1.0, 2.0, 2.0, 1.0, 2.0, 1.0};
+  for (int c = 0; c < 6; ++c) g[c] = N.at(GXX + c, 0);
+  sym_inverse<double>(g, ig);
+  const double igw[6] = {ig[0], ig[1] + ig[1], ig[2] + ig[2], ig[3], ig[4] + ig[4], ig[5]};
   double Gd[3][6], Gu[3][6], Gc[3], Gl[3];
+  {
+    double dg[3][6];
 #pragma unroll
-  for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < 3; ++k)
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+      for (int c = 0; c < 6; ++c) dg[k][c] = fd1<double>(N, GXX + c, N.st[k], 0.5 * C.c1);  // (1/2) d_k g~_ij
 #pragma unroll
-      for (int j = i; j < 3; ++j)
-        Gd[k][S6(i, j)] = 0.5 * (dg[i][S6(j, k)] + dg[j][S6(i, k)] - dg[k][S6(i, j)]);
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j) Gd[k][S6(i, j)] = dg[i][S6(j, k)] + dg[j][S6(i, k)] - dg[k][S6(i, j)];
+  }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
 #pragma unroll
     for (int c = 0; c < 6; ++c)
-      Gu[k][c] = ig[S6(k, 0)] * Gd[0][c] + ig[S6(k, 1)] * Gd[1][c] + ig[S6(k, 2)] * Gd[2][c];
-    double s = 0.0, t = 0.0;
+      Gu[k][c] = fma(ig[S6(k, 0)], Gd[0][c], fma(ig[S6(k, 1)], Gd[1][c], ig[S6(k, 2)] * Gd[2][c]));
+    double s = igw[0] * Gu[k][0], t = igw[0] * Gd[k][0];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      s = fma(w6[c] * ig[c], Gu[k][c], s);
-      t = fma(w6[c] * ig[c], Gd[k][c], t);
+    for (int c = 1; c < 6; ++c) {
+      s = fma(igw[c], Gu[k][c], s);
+      t = fma(igw[c], Gd[k][c], t);
     }
     Gc[k] = s;  // G~^k
-    Gl[k] = t;  // G~_k = g~^ml G~_kml
+    Gl[k] = t;  // G~_k
   }
-  // second derivatives of g~: dd[c][kl]
-  double dd[6][6];
+  // the second derivatives, one component g~_ln at a time
+  double R = 0.0;
 #pragma unroll
-  for (int c = 0; c < 6; ++c)
+  for (int l = 0; l < 3; ++l)
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int n = l; n < 3; ++n) {
+      const int c = S6(l, n);
+      double dd[6];
 #pragma unroll
-      for (int l = k; l < 3; ++l) dd[c][S6(k, l)] = fdkl<double>(N, GXX + c, k, l, C);
-  // dIg[j][ml] = g~^ma g~^lb d_j g~_ab  (= -d_j g~^ml)
-  double dIg[3][6];
+      for (int k = 0; k < 3; ++k)
 #pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    double t[3][3];
+        for (int m = k; m < 3; ++m) dd[S6(k, m)] = fdkl<double>(N, GXX + c, k, m, C);
+      double s = 0.0, lap = 0.0;
 #pragma unroll
-    for (int m = 0; m < 3; ++m)
+      for (int k = 0; k < 3; ++k)
+        s = fma(ig[S6(k, n)], fma(ig[S6(0, l)], dd[S6(k, 0)], fma(ig[S6(1, l)], dd[S6(k, 1)], ig[S6(2, l)] * dd[S6(k, 2)])), s);
 #pragma unroll
-      for (int b = 0; b < 3; ++b)
-        t[m][b] = ig[S6(m, 0)] * dg[j][S6(0, b)] + ig[S6(m, 1)] * dg[j][S6(1, b)] + ig[S6(m, 2)] * dg[j][S6(2, b)];
-#pragma unroll
-    for (int m = 0; m < 3; ++m)
-#pragma unroll
-      for (int l = m; l < 3; ++l)
-        dIg[j][S6(m, l)] = t[m][0] * ig[S6(0, l)] + t[m][1] * ig[S6(1, l)] + t[m][2] * ig[S6(2, l)];
-  }
-  // d_j G~_n = -dIg[j]:G~_n.. + g~^ml (d_j d_m g~_ln - 1/2 d_j d_n g~_ml)
-  // d_j G~^k = -dIg[j][kn] G~_n + g~^kn d_j G~_n
-  double dGt[3][3];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    double dGl[3];
-#pragma unroll
-    for (int n = 0; n < 3; ++n) {
-      double s = 0.0;
-#pragma unroll
-      for (int c = 0; c < 6; ++c) s = fma(-w6[c] * dIg[j][c], Gd[n][c], s);
-#pragma unroll
-      for (int m = 0; m < 3; ++m)
-#pragma unroll
-        for (int l = 0; l < 3; ++l)
-          s = fma(ig[S6(m, l)], dd[S6(l, n)][S6(j, m)] - 0.5 * dd[S6(m, l)][S6(j, n)], s);
-      dGl[n] = s;
+      for (int q = 0; q < 6; ++q) lap = fma(igw[q], dd[q], lap);
+      // both orders of (l, n) give the same first sum
+      R = fma(-igw[c], lap, l == n ? R + s : fma(2.0, s, R));
     }
+  // the quadratic terms
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      double s = 0.0;
-#pragma unroll
-      for (int n = 0; n < 3; ++n) s += -dIg[j][S6(k, n)] * Gl[n] + ig[S6(k, n)] * dGl[n];
-      dGt[j][k] = s;
-    }
-  }
-  const double iph = 1.0 / ph;
-  double Pu[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) Pu[k] = ig[S6(k, 0)] * dP[0] + ig[S6(k, 1)] * dP[1] + ig[S6(k, 2)] * dP[2];
-  const double PP = Pu[0] * dP[0] + Pu[1] * dP[1] + Pu[2] * dP[2];
-  double cdph[6];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = i; j < 3; ++j) {
-      const int c = S6(i, j);
-      cdph[c] = fdkl<double>(N, PHI, i, j, C) - (Gu[0][c] * dP[0] + Gu[1][c] * dP[1] + Gu[2][c] * dP[2]);
-    }
-  double trcdph = 0.0;
-#pragma unroll
-  for (int c = 0; c < 6; ++c) trcdph = fma(w6[c] * ig[c], cdph[c], trcdph);
-  double Cm[3][3][3], Em[3][3][3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
+  for (int k = 0; k < 3; ++k) {
+    double E[3][3];  // G~_ki^m
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        Cm[k][i][m] = ig[S6(0, m)] * Gu[k][S6(0, i)] + ig[S6(1, m)] * Gu[k][S6(1, i)] + ig[S6(2, m)] * Gu[k][S6(2, i)];
-        Em[k][i][m] = ig[S6(0, m)] * Gd[k][S6(0, i)] + ig[S6(1, m)] * Gd[k][S6(1, i)] + ig[S6(2, m)] * Gd[k][S6(2, i)];
+      for (int m = 0; m < 3; ++m)
+        E[i][m] = fma(ig[S6(0, m)], Gd[k][S6(i, 0)], fma(ig[S6(1, m)], Gd[k][S6(i, 1)], ig[S6(2, m)] * Gd[k][S6(i, 2)]));
+    double y = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int m = i; m < 3; ++m) {
+        const double u = fma(ig[S6(i, 0)], E[0][m], fma(ig[S6(i, 1)], E[1][m], ig[S6(i, 2)] * E[2][m]));
+        y = fma(i == m ? u : u + u, Gu[k][S6(i, m)], y);
       }
-  double R = 0.0;
+    R += fma(-Gc[k], Gl[k], y);
+  }
+  const double ph = N.at(PHI, 0), Kt = N.at(KTR, 0);
+  double dP[3], Pu[3];
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+  for (int k = 0; k < 3; ++k) dP[k] = fd1<double>(N, PHI, N.st[k], C.c1);
 #pragma unroll
-    for (int j = i; j < 3; ++j) {
-      const int c = S6(i, j);
-      double lap = 0.0;
+  for (int k = 0; k < 3; ++k) Pu[k] = fma(ig[S6(k, 0)], dP[0], fma(ig[S6(k, 1)], dP[1], ig[S6(k, 2)] * dP[2]));
+  const double PP = fma(Pu[0], dP[0], fma(Pu[1], dP[1], Pu[2] * dP[2]));
+  double tr = fma(-Gc[0], dP[0], fma(-Gc[1], dP[1], -Gc[2] * dP[2]));
 #pragma unroll
-      for (int q = 0; q < 6; ++q) lap = fma(w6[q] * ig[q], dd[c][q], lap);
-      double t = -0.5 * lap;
+  for (int k = 0; k < 3; ++k)
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
-        t += 0.5 * (g[S6(k, i)] * dGt[j][k] + g[S6(k, j)] * dGt[i][k] + Gc[k] * dg[k][c]);
-      double x1 = 0.0, x2 = 0.0, q3 = 0.0;
+    for (int l = k; l < 3; ++l) tr = fma(igw[S6(k, l)], fdkl<double>(N, PHI, k, l, C), tr);
+  double A[6], Am[3][3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-          x1 = fma(Cm[k][i][m], Gd[j][S6(k, m)], x1);
-          x2 = fma(Cm[k][j][m], Gd[i][S6(k, m)], x2);
-          q3 = fma(Gu[k][S6(i, m)], Em[k][j][m], q3);
-        }
-      t += x1 + x2 + q3 + iph * (cdph[c] + g[c] * trcdph) - 2.0 * iph * iph * g[c] * PP;
-      R = fma(w6[c] * ig[c], t, R);
-    }
-  R *= ph * ph;
-  double Am[3][3];
+  for (int c = 0; c < 6; ++c) A[c] = N.at(AXX + c, 0);
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int m = 0; m < 3; ++m)
-      Am[i][m] = A[S6(i, 0)] * ig[S6(0, m)] + A[S6(i, 1)] * ig[S6(1, m)] + A[S6(i, 2)] * ig[S6(2, m)];
+      Am[i][m] = fma(A[S6(i, 0)], ig[S6(0, m)], fma(A[S6(i, 1)], ig[S6(1, m)], A[S6(i, 2)] * ig[S6(2, m)]));
   double AA = 0.0;
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int m = 0; m < 3; ++m) AA = fma(Am[i][m], Am[m][i], AA);
-  H = R + (2.0 / 3.0) * Kt * Kt - AA;
+  H = fma(ph, fma(ph, R, 4.0 * tr), fma(-6.0, PP, fma((2.0 / 3.0) * Kt, Kt, -AA)));
+  const double iph3 = -3.0 / ph;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    double s = 0.0;
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-      for (int l = 0; l < 3; ++l) s = fma(ig[S6(k, l)], dA[k][S6(l, i)], s);
+    M[i] = fd1<double>(N, KTR, N.st[i], (-2.0 / 3.0) * C.c1);
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
 #pragma unroll
-      for (int l = 0; l < 3; ++l) s = fma(-Gu[m][S6(l, i)], Am[m][l], s);
-      s = fma(-Gc[m], A[S6(i, m)], s);
-      s = fma(-3.0 * iph * A[S6(i, m)], Pu[m], s);
+      for (int l = 0; l < 3; ++l) M[i] = fma(-Gu[m][S6(l, i)], Am[m][l], M[i]);
+      M[i] = fma(fma(iph3, Pu[m], -Gc[m]), A[S6(i, m)], M[i]);
     }
-    M[i] = s - (2.0 / 3.0) * dK[i];
   }
+  // g~^kl d_k A~_li, one derivative at a time
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+#pragma unroll
+      for (int i = l; i < 3; ++i) {
+        const double d = fd1<double>(N, AXX + S6(l, i), N.st[k], C.c1);
+        M[i] = fma(ig[S6(k, l)], d, M[i]);
+        if (i != l) M[l] = fma(ig[S6(k, i)], d, M[l]);
+      }
 }
 
 struct ConsCoef {
   StencilCoef<double> C[MAX_LEVELS];
 };
 
-__global__ void __launch_bounds__(RED_THREADS) constraints_kernel(GridView g, ConsCoef LC,
-                                                                  const double *__restrict__ tile,
-                                                                  double *H, double *M, double *partial) {
+// What the monitors read: the derivative pass (DER), or halo'd tiles alone
+// (the caller's own, which have no derivatives beside them).
+struct ConsSrc {
+  const double *tile;
+  const double *der, *mix, *in;
+};
+
+// (From tiles: one block per SM, so that its stack stays within the context's
+// default and the first launch needs no larger local-memory pool.)
+template <bool DER>
+__global__ void __launch_bounds__(RED_THREADS, DER ? 2 : 1) constraints_kernel(GridView g, ConsCoef LC, ConsSrc src, double *H,
+                                                                     double *M, double *partial) {
   __shared__ double sh[5][RED_THREADS];
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
@@ -214,19 +173,23 @@ __global__ void __launch_bounds__(RED_THREADS) constraints_kernel(GridView g, Co
     const int p3 = p * p * p;  // 32-bit division: every state index is below 2^31
     const int n = (int)i / p3;
     const int r = (int)i - n * p3;
-    const int z = r / (p * p), y = (r / p) % p, x = r % p;
-    Nbhd N;
-    N.c = tile + n * g.T3 + ((long long)(z + HALO) * T + (y + HALO)) * T + (x + HALO);
-    N.fs = (long long)g.n_patches * g.T3;
-    N.st[0] = 1;
-    N.st[1] = T;
-    N.st[2] = T * T;
-    N.mix = nullptr;
-    N.ms = 0;
-    N.mixf = nullptr;
-    N.msf = 0;
     double h, m[3];
-    constraints_point(N, LC.C[patch_level(g, n)], h, m);
+    if constexpr (DER) {
+      constraints_point(der_view<false>(g, src.der, src.mix, src.in, i), LC.C[patch_level(g, n)], h, m);
+    } else {
+      const int z = r / (p * p), y = (r / p) % p, x = r % p;
+      Nbhd N;
+      N.c = src.tile + n * g.T3 + ((long long)(z + HALO) * T + (y + HALO)) * T + (x + HALO);
+      N.fs = (long long)g.n_patches * g.T3;
+      N.st[0] = 1;
+      N.st[1] = T;
+      N.st[2] = T * T;
+      N.mix = nullptr;
+      N.ms = 0;
+      N.mixf = nullptr;
+      N.msf = 0;
+      constraints_point(N, LC.C[patch_level(g, n)], h, m);
+    }
     if (H) H[i] = h;
     if (M) {
       M[i] = m[0];
@@ -406,8 +369,8 @@ __global__ void __launch_bounds__(256) enforce_kernel(GridView g, double *U) {
 
 int constraint_blocks(long long n_points) { return (int)((n_points + RED_THREADS - 1) / RED_THREADS); }
 
-cudaError_t launch_constraints(const GridView &g, const double *tile, double *H, double *M, double *partial,
-                               int blocks, double *out5, cudaStream_t s) {
+static cudaError_t launch_constraints_from(const GridView &g, const ConsSrc &src, double *H, double *M, double *partial,
+                                           int blocks, double *out5, cudaStream_t s) {
   ConsCoef LC;
   for (int l = 0; l < MAX_LEVELS; ++l) {
     const double dx = g.ldx[l];
@@ -417,12 +380,32 @@ cudaError_t launch_constraints(const GridView &g, const double *tile, double *H,
     LC.C[l].cko = 0.0;
   }
   if (blocks > 0) {
-    constraints_kernel<<<blocks, RED_THREADS, 0, s>>>(g, LC, tile, H, M, partial);
+    if (src.der) constraints_kernel<true><<<blocks, RED_THREADS, 0, s>>>(g, LC, src, H, M, partial);
+    else constraints_kernel<false><<<blocks, RED_THREADS, 0, s>>>(g, LC, src, H, M, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   reduce_partials<<<1, RED_THREADS, 0, s>>>(partial, blocks, (double)g.n_leaf_points, out5);
   return cudaGetLastError();
+}
+
+cudaError_t launch_constraints(const GridView &g, const double *tile, double *H, double *M, double *partial,
+                               int blocks, double *out5, cudaStream_t s) {
+  return launch_constraints_from(g, ConsSrc{tile, nullptr, nullptr, nullptr}, H, M, partial, blocks, out5, s);
+}
+
+// Loads the kernels of the monitors that take tiles alone (a kernel's first
+// launch may take device memory for its code, and their caller may have none
+// to give); once per grid.
+cudaError_t prepare_constraints() {
+  cudaFuncAttributes a;
+  cudaError_t e = cudaFuncGetAttributes(&a, constraints_kernel<false>);
+  return e == cudaSuccess ? cudaFuncGetAttributes(&a, reduce_partials) : e;
+}
+
+cudaError_t launch_constraints_der(const GridView &g, const double *der, const double *mix, const double *in, double *H,
+                                   double *M, double *partial, int blocks, double *out5, cudaStream_t s) {
+  return launch_constraints_from(g, ConsSrc{nullptr, der, mix, in}, H, M, partial, blocks, out5, s);
 }
 
 cudaError_t launch_constraints_excluded(const GridView &g, const double *H, const double *M, int n_centres,

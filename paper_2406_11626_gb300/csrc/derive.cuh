@@ -215,9 +215,11 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
 #pragma unroll
       for (int k = 0; k < 8; ++k) c[k] = __ldg(&ep->src[k]);
       const int r = __ldg(&ep->r), t = __ldg(&ep->t);
-      for (int j = group; j < fl.n; j += groups)
-        __stcs(tile + ((long long)fl.f[j] * g.n_patches + n) * T3 + t,
-               interp_value(c, r & 3, (r >> 2) & 3, (r >> 4) & 3, src + fl.f[j] * g.S));
+      for (int j = group; j < fl.n; j += groups) {
+        const int v = fl.f[j] & ~FIELD_NO_SUMS;
+        __stcs(tile + ((long long)v * g.n_patches + n) * T3 + t,
+               interp_value(c, r & 3, (r >> 2) & 3, (r >> 4) & 3, src + v * g.S));
+      }
     }
   } else if (SRC == FROM_LEVEL) {
     const int bx = __ldg(g.ijk + 3 * n) * p - HALO;
@@ -242,7 +244,8 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
   for (int r = 0; r < ROUNDS; ++r) at[r] = PF > 0 ? centre_at(threadIdx.x + r * THREADS) : 0;
   constexpr int JM = (1 << JOB_BITS) - 1;
   for (int j = group; j < fl.n; j += groups) {
-    const int v = fl.f[j];
+    const int v = fl.f[j] & ~FIELD_NO_SUMS;
+    const bool sums = (fl.f[j] & FIELD_NO_SUMS) == 0;
     const double *sv = src + (long long)v * g.S;
     double *tv = tile + ((long long)v * g.n_patches + n) * T3;
     const int slot = NF == NV ? mix_slot(v) : -1;
@@ -334,7 +337,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
           mixed_out(ext, e, pe, cmix, cmixf, f32, mix, np, pbase, slot + 2, q);
         }
       }
-      if (!RAW) {
+      if (!RAW && sums) {
         __syncthreads();  // the exponents take the widened region's place
         for (int t = threadIdx.x; t < T3; t += THREADS) {
           unsigned e;
@@ -344,6 +347,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
         __syncthreads();
       }
     }
+    if (!sums) continue;
     const bool f32 = der_f32(MIXED, v);
     double *dd = der + (MIXED ? (v == ALPHA ? 0 : 7) : 4 * v) * np + pbase;
     double *dp = MIXED ? dd + 4 * np : der + (4 * NF + 3 * (second ? slot / 3 : 0)) * np + pbase;

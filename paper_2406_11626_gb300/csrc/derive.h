@@ -22,7 +22,9 @@ constexpr int DER_D = 14;        // FP64 slots of the mixed precision
 constexpr int DER_F = 4 * 23;    // FP32 slots before the pure second sums
 __host__ __device__ __forceinline__ constexpr bool der_f32(bool mixed, int v) { return mixed && v != ALPHA && v != PHI; }
 
-// Fields that a derivative pass takes.
+// Fields that a derivative pass takes; FIELD_NO_SUMS marks one of which only
+// the tile and the mixed derivatives are wanted.
+constexpr int FIELD_NO_SUMS = 0x80;
 struct FieldList {
   unsigned char f[64];
   int n;
