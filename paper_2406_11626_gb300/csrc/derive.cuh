@@ -50,22 +50,6 @@ __device__ __forceinline__ long long fx_sar(long long x, unsigned s) {
   return r;
 }
 
-// v units of 2^(e - 1075 - K) as FP32: the two halves converted and joined in one
-// rounding, then two exact scalings (a result outside the FP32 range becomes
-// zero or infinite, as the FP32 conversions of the mixed precision do).
-template <int K>
-__device__ __forceinline__ float fx_outf(long long v, unsigned e) {
-  const float f = fmaf(__int2float_rn((int)(v >> 32)), 4294967296.0f, __uint2float_rn((unsigned)v));
-  const int s = (int)e - 896;  // FP32 exponent field of 2^(e - 1023)
-  const float sc = s < 1 ? 0.0f : s > 254 ? __uint_as_float(0x7F800000u) : __uint_as_float((unsigned)s << 23);
-  return f == 0.0f ? 0.0f : (f * (K == 4 ? 1.3877787807814457e-17f : 5.5511151231257827e-17f)) * sc;  // 2^-(52 + K)
-}
-template <int K, class O>
-__device__ __forceinline__ O fx_result(long long v, unsigned e) {
-  if constexpr (std::is_same<O, float>::value) return fx_outf<K>(v, e);
-  else return fx_out<K>(v, (e << 21) | FX_LOW);
-}
-
 // The stencil sums of one point whose largest neighbour lies outside [FX_FLOOR, FX_TOP), in FP64.
 template <bool SECOND>
 __device__ __noinline__ void point_sums_fp64(const long long *w, const unsigned *ex, int T, double *out) {
@@ -89,8 +73,8 @@ __device__ __noinline__ void point_sums_fp64(const long long *w, const unsigned 
 
 // The stencil sums of the point at w, ex: out[0..2] first derivatives, out[3]
 // dissipation, out[4..6] pure second derivatives.
-template <bool SECOND, class O>
-__device__ __forceinline__ void point_sums(const long long *w, const unsigned *ex, int T, O *out) {
+template <bool SECOND>
+__device__ __forceinline__ void point_sums(const long long *w, const unsigned *ex, int T, double *out) {
   const int st[3] = {1, T, T * T};
   const unsigned e0 = ex[0];
   unsigned ep[3][3], em[3][3], e = e0;
@@ -103,12 +87,10 @@ __device__ __forceinline__ void point_sums(const long long *w, const unsigned *e
       e = max(e, max(ep[k][j], em[k][j]));
     }
   if (e - FX_FLOOR >= FX_TOP - FX_FLOOR && e != 0u) {  // (all zero: the sums below are zero)
-    double d[7];
-    point_sums_fp64<SECOND>(w, ex, T, d);
-#pragma unroll
-    for (int q = 0; q < (SECOND ? 7 : 4); ++q) out[q] = cvt<O>(d[q]);
+    point_sums_fp64<SECOND>(w, ex, T, out);
     return;
   }
+  const unsigned u = (e << 21) | FX_LOW;
   const long long q = fx_sar(w[0], e - e0) >> 2;
   long long s1 = 0, s2 = 0, s3 = 0;
 #pragma unroll
@@ -117,18 +99,48 @@ __device__ __forceinline__ void point_sums(const long long *w, const unsigned *e
     const long long p1 = fx_sar(w[s], e - ep[k][0]), m1 = fx_sar(w[-s], e - em[k][0]);
     const long long p2 = fx_sar(w[2 * s], e - ep[k][1]), m2 = fx_sar(w[-2 * s], e - em[k][1]);
     const long long t1 = p1 + m1, t2 = p2 + m2;
-    out[k] = fx_result<4, O>((p1 - m1) * 8 - (p2 - m2), e);
-    if (SECOND) out[4 + k] = fx_result<2, O>(((t1 >> 2) - 2 * q) * 16 - (t2 >> 2) + 2 * q, e);
+    out[k] = fx_out<4>((p1 - m1) * 8 - (p2 - m2), u);
+    if (SECOND) out[4 + k] = fx_out<2>(((t1 >> 2) - 2 * q) * 16 - (t2 >> 2) + 2 * q, u);
     s1 += t1;
     s2 += t2;
     s3 += fx_sar(w[3 * s], e - ep[k][2]) + fx_sar(w[-3 * s], e - em[k][2]);
   }
-  out[3] = fx_result<2, O>((((s1 >> 2) - 4 * q) * 5 - 2 * (s2 >> 2)) * 3 + (s3 >> 2), e);
+  out[3] = fx_out<2>((((s1 >> 2) - 4 * q) * 5 - 2 * (s2 >> 2)) * 3 + (s3 >> 2), u);
+}
+
+// The same in FP32 from split pairs (mixed precision), whose FP32 pipe is
+// wider than the integer one: first differences (hi+ - hi-) + (lo+ - lo-),
+// second differences from error-free differences of the high parts (the
+// reasons stand at sp_second in ccz4_algebra.cuh). On the 144^3 puncture the
+// integer sums with FP32 results took the mixed step to 15.8 ms, the pairs
+// to @@.
+template <bool SECOND>
+__device__ __forceinline__ void point_sums(const float2 *t, const unsigned *, int T, float *out) {
+  const int st[3] = {1, T, T * T};
+  const float2 c = t[0];
+  float ko = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    float b[3], d[2];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const float2 p = t[(j + 1) * st[k]], m = t[-(j + 1) * st[k]];
+      float ep, em;
+      const float dp = sp_two_diff<float>(p.x, c.x, ep), dm = sp_two_diff<float>(m.x, c.x, em);
+      b[j] = (dp + dm) + ((ep + em) + fmaf(-2.0f, c.y, p.y + m.y));
+      if (j < 2) d[j] = (p.x - m.x) + (p.y - m.y);
+    }
+    out[k] = fmaf(8.0f, d[0], -d[1]);
+    if (SECOND) out[4 + k] = fmaf(16.0f, b[0], -b[1]);
+    const float s = fmaf(15.0f, b[0], fmaf(-6.0f, b[1], b[2]));
+    ko = k == 0 ? s : ko + s;
+  }
+  out[3] = ko;
 }
 
 // The same from raw FP64 values, for patch edges whose tile leaves no room for the exponents.
-template <bool SECOND, class O>
-__device__ __forceinline__ void point_sums_raw(const double *t, int T, O *out) {
+template <bool SECOND>
+__device__ __forceinline__ void point_sums_raw(const double *t, int T, double *out) {
   const int st[3] = {1, T, T * T};
   double p[3][3], m[3][3], d1[3], d2[3], ko;
 #pragma unroll
@@ -141,24 +153,16 @@ __device__ __forceinline__ void point_sums_raw(const double *t, int T, O *out) {
   fx_axes<true, SECOND>(t[0], p, m, d1, d2, ko);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    out[k] = cvt<O>(d1[k]);
-    if (SECOND) out[4 + k] = cvt<O>(d2[k]);
+    out[k] = d1[k];
+    if (SECOND) out[4 + k] = d2[k];
   }
-  out[3] = cvt<O>(ko);
+  out[3] = ko;
 }
 
 // Where a patch's tile comes from: gathered through the neighbour lookup of a
 // single level, or through a refined mesh's table, or read from the tile
 // buffer that a halo fill has written.
 enum { FROM_LEVEL = 0, FROM_MESH = 1, FROM_TILE = 2 };
-
-// First sums of the mixed derivatives from the raw FP64 tile; FP32 sums for
-// the fields whose mixed derivatives the mixed precision keeps in FP32.
-__device__ __forceinline__ void mixed_first(double *ext, int e, const double *ts, int c0, int s, bool f32) {
-  const double a = ts[c0 + s] - ts[c0 - s], b = ts[c0 + 2 * s] - ts[c0 - 2 * s];
-  if (f32) reinterpret_cast<float *>(ext)[e] = fmaf(8.0f, cvt<float>(a), -cvt<float>(b));
-  else ext[e] = fma(8.0, a, -b);
-}
 
 // Doubles that the widened region of the mixed derivatives takes, and the
 // place of the exponents with it: a field's mixed derivatives are done before
@@ -270,7 +274,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
       }
       __syncthreads();
     }
-    const bool second = slot >= 0;
+    const bool second = slot >= 0, pair = der_f32(MIXED, v);  // pair: the tile holds split pairs
     for (int t0 = threadIdx.x; t0 < T3; t0 += BATCH * THREADS) {
       double val[BATCH];
 #pragma unroll
@@ -291,10 +295,10 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
         const int t = t0 + u * THREADS;
         if (t >= T3) continue;
         double w = val[u];
-        if (SRC == FROM_TILE && der_f32(MIXED, v))  // a split pair: its value
-          w = cvt<double>(__int_as_float(__double2loint(w))) + cvt<double>(__int_as_float(__double2hiint(w)));
         if (SRC != FROM_TILE && tile_out) __stcs(tv + t, w);
-        if (!RAW && (!second || SRC == FROM_TILE)) {
+        if (pair) {
+          ts[t] = SRC == FROM_TILE ? w : split_pair(w);
+        } else if (!RAW && (!second || SRC == FROM_TILE)) {
           unsigned e;
           reinterpret_cast<long long *>(ts)[t] = fx_word(w, e);
           ex[t] = e;
@@ -306,20 +310,19 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
     __syncthreads();
     if (second && SRC != FROM_TILE) {
       // the mixed derivatives, as the halo fill forms them
-      const bool f32 = MIXED && mix_fslot(slot) >= 0;
 #pragma unroll 1
       for (int pass = 0; pass < (wide ? 1 : 3); ++pass) {
         const int si = pass == 0 ? T : T * T;
         for (int e = threadIdx.x; e < next; e += THREADS) {
           const int a = e % pe - 2, b = (e / pe) % p, c = e / (pe * p);
           const int x = pass == 2 ? b : a, y = pass == 2 ? a : b;
-          mixed_first(ext, e, ts, ((c + HALO) * T + (y + HALO)) * T + (x + HALO), si, f32);
+          mixed_in(ext, e, ts, ((c + HALO) * T + (y + HALO)) * T + (x + HALO), si, pair);
         }
         __syncthreads();
         for (int q = threadIdx.x; q < p3; q += THREADS) {
           const int x = q % p, y = (q / p) % p, z = q / (p * p);
           const int a = pass == 2 ? y : x, b = pass == 2 ? x : y;
-          mixed_out(ext, (z * p + b) * pe + (a + 2), 1, cmix, cmixf, f32, mix, np, pbase, slot + pass, q);
+          mixed_out(ext, (z * p + b) * pe + (a + 2), 1, cmix, cmixf, pair, mix, np, pbase, slot + pass, q);
         }
         __syncthreads();
       }
@@ -327,17 +330,17 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
         for (int e = threadIdx.x; e < pe * pe * p; e += THREADS) {
           const int a = e % pe - 2, b = (e / pe) % pe - 2, c = e / (pe * pe);
           if ((a < 0 || a >= p) && (b < 0 || b >= p)) continue;
-          mixed_first(ext, e, ts, ((c + HALO) * T + (b + HALO)) * T + (a + HALO), T * T, f32);
+          mixed_in(ext, e, ts, ((c + HALO) * T + (b + HALO)) * T + (a + HALO), T * T, pair);
         }
         __syncthreads();
         for (int q = threadIdx.x; q < p3; q += THREADS) {
           const int x = q % p, y = (q / p) % p, z = q / (p * p);
           const int e = (z * pe + (y + 2)) * pe + (x + 2);
-          mixed_out(ext, e, 1, cmix, cmixf, f32, mix, np, pbase, slot + 1, q);
-          mixed_out(ext, e, pe, cmix, cmixf, f32, mix, np, pbase, slot + 2, q);
+          mixed_out(ext, e, 1, cmix, cmixf, pair, mix, np, pbase, slot + 1, q);
+          mixed_out(ext, e, pe, cmix, cmixf, pair, mix, np, pbase, slot + 2, q);
         }
       }
-      if (!RAW && sums) {
+      if (!RAW && sums && !pair) {
         __syncthreads();  // the exponents take the widened region's place
         for (int t = threadIdx.x; t < T3; t += THREADS) {
           unsigned e;
@@ -348,7 +351,6 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
       }
     }
     if (!sums) continue;
-    const bool f32 = der_f32(MIXED, v);
     double *dd = der + (MIXED ? (v == ALPHA ? 0 : 7) : 4 * v) * np + pbase;
     double *dp = MIXED ? dd + 4 * np : der + (4 * NF + 3 * (second ? slot / 3 : 0)) * np + pbase;
     float *fd = reinterpret_cast<float *>(der + DER_D * np) + (long long)(4 * der_f(v)) * np + pbase;
@@ -358,8 +360,10 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
       constexpr bool SECOND = decltype(is_second)::value;
       auto point = [&](int q, int c0) {
         O o[7];
-        if constexpr (RAW) point_sums_raw<SECOND, O>(ts + c0, T, o);
-        else point_sums<SECOND, O>(reinterpret_cast<const long long *>(ts) + c0, ex + c0, T, o);
+        if constexpr (std::is_same<O, float>::value)
+          point_sums<SECOND>(reinterpret_cast<const float2 *>(ts) + c0, ex, T, o);
+        else if constexpr (RAW) point_sums_raw<SECOND>(ts + c0, T, o);
+        else point_sums<SECOND>(reinterpret_cast<const long long *>(ts) + c0, ex + c0, T, o);
         O *a, *b;
         if constexpr (std::is_same<O, float>::value) {
           a = fd + q;
@@ -390,7 +394,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
     if constexpr (NF != NV) {
       each(std::false_type(), 0.0);
     } else if constexpr (MIXED) {
-      if (!f32) each(std::true_type(), 0.0);
+      if (!pair) each(std::true_type(), 0.0);
       else if (second) each(std::true_type(), 0.0f);
       else each(std::false_type(), 0.0f);
     } else {

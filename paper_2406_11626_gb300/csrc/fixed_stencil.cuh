@@ -100,12 +100,42 @@ __host__ __device__ __forceinline__ double fx_out(int64_t v, unsigned unit) {
   return a ? fx_from_bits(w) : 0.0;
 }
 
+#ifdef __CUDACC__
+// The same by the conversion instruction, which runs on the FP64 pipe (one of
+// its slots instead of about 20 integer instructions): to nearest, ties to even.
+template <int K>
+__device__ __forceinline__ double fx_out_cvt(long long v, unsigned unit) {
+  const double d = __ll2double_rn(v);
+  const int hi = __double2hiint(d) + (int)(((unit >> 21) - (1075u + K)) << 20);
+  return v ? __hiloint2double(hi, __double2loint(d)) : 0.0;
+}
+#endif
+
 // 8 (a1 - b1) - (a2 - b2): the first-derivative stencil of the values at +1, -1, +2, -2
 __host__ __device__ __forceinline__ double fx_first(double a1, double b1, double a2, double b2) {
   const unsigned u = fx_unit(fx_max(fx_max(fx_key(a1), fx_key(b1)), fx_max(fx_key(a2), fx_key(b2))));
   if (fx_outside(u)) return fma(8.0, a1 - b1, -(a2 - b2));
   const int64_t d1 = fx_in(a1, u) - fx_in(b1, u), d2 = fx_in(a2, u) - fx_in(b2, u);
   return fx_out<4>(d1 * 8 - d2, u);
+}
+
+// The FP64 side of fx_laplacian: out of line, or the compiler evaluates it ahead of the branch.
+__host__ __device__ __noinline__ inline double fx_laplacian_fp64(double c, double a, double b, double d, double e, double f,
+                                                          double g) {
+  return fma(-6.0, c, ((a + b) + (d + e)) + (f + g));
+}
+
+// The sum of the six values v minus 6 c (the 7-point Laplacian without 1 / h^2).
+__host__ __device__ __forceinline__ double fx_laplacian(double c, const double (&v)[6]) {
+  unsigned key = fx_key(c);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) key = fx_max(key, fx_key(v[k]));
+  const unsigned u = fx_unit(key);
+  if (fx_outside(u)) return fx_laplacian_fp64(c, v[0], v[1], v[2], v[3], v[4], v[5]);
+  int64_t s = fx_in(c, u) * -6;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) s += fx_in(v[k], u);
+  return fx_out<4>(s, u);
 }
 
 // From the centre c and the neighbours p[k][j], m[k][j] at distance j + 1 along

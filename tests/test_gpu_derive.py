@@ -37,7 +37,7 @@ def test_rhs_over_patch_edges(p, npv, bc):
 @pytest.mark.parametrize("prec,bar", [("fp64", 1e-13), ("mixed", 1e-7)])
 def test_stages_from_filled_tiles_equal_the_step(prec, bar):
     """rk_stage takes its derivatives from the tiles of a halo fill, a step
-    straight from the state: the same values (mixed: tiles hold 48 bits)."""
+    straight from the state: the same values."""
     from paper_2406_11626_gb300 import ccz4 as C
     cfg = I.single_puncture_config(p=9, n_side=2, half_width=1.0)
     U, G = random_state(9, cfg.np, cfg.origin, cfg.dx, cfg.ijk(), 3, "sommerfeld", amp=0.01, base="puncture")
