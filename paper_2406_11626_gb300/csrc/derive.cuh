@@ -28,14 +28,15 @@ namespace {
 
 // The word and the exponent under which a tile value waits in shared memory:
 // its mantissa as a signed integer of 57 bits and its biased exponent; the
-// value's own bits where the exponent is FX_TOP or more, 0 for zero (and for
-// subnormal values).
+// value's own bits where the exponent is FX_TOP or more. (Zero and subnormal
+// values keep exponent 0: beside any value of exponent FX_FLOOR or more they
+// are shifted out.)
 __device__ __forceinline__ long long fx_word(double u, unsigned &e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(u);
   e = (unsigned)(b >> 52) & 0x7FFu;
   const unsigned long long m = ((b << 4) & 0x00FFFFFFFFFFFFF0ull) | 0x0100000000000000ull;
   const unsigned long long n = (unsigned long long)((long long)b >> 63);
-  return e >= FX_TOP ? (long long)b : e == 0u ? 0 : (long long)((m ^ n) - n);
+  return e >= FX_TOP ? (long long)b : (long long)((m ^ n) - n);
 }
 __device__ __forceinline__ double fx_value(long long w, unsigned e) {
   if (e >= FX_TOP) return __longlong_as_double(w);
@@ -86,8 +87,13 @@ __device__ __forceinline__ void point_sums(const long long *w, const unsigned *e
       em[k][j] = ex[-(j + 1) * st[k]];
       e = max(e, max(ep[k][j], em[k][j]));
     }
-  if (e - FX_FLOOR >= FX_TOP - FX_FLOOR && e != 0u) {  // (all zero: the sums below are zero)
-    point_sums_fp64<SECOND>(w, ex, T, out);
+  if (e - FX_FLOOR >= FX_TOP - FX_FLOOR) {
+    if (e == 0u) {
+#pragma unroll
+      for (int q = 0; q < (SECOND ? 7 : 4); ++q) out[q] = 0.0;
+    } else {
+      point_sums_fp64<SECOND>(w, ex, T, out);
+    }
     return;
   }
   const unsigned u = (e << 21) | FX_LOW;
@@ -100,12 +106,12 @@ __device__ __forceinline__ void point_sums(const long long *w, const unsigned *e
     const long long p2 = fx_sar(w[2 * s], e - ep[k][1]), m2 = fx_sar(w[-2 * s], e - em[k][1]);
     const long long t1 = p1 + m1, t2 = p2 + m2;
     out[k] = fx_out<4>((p1 - m1) * 8 - (p2 - m2), u);
-    if (SECOND) out[4 + k] = fx_out<2>(((t1 >> 2) - 2 * q) * 16 - (t2 >> 2) + 2 * q, u);
+    if (SECOND) out[4 + k] = fx_out_cvt<2>(((t1 >> 2) - 2 * q) * 16 - (t2 >> 2) + 2 * q, u);
     s1 += t1;
     s2 += t2;
     s3 += fx_sar(w[3 * s], e - ep[k][2]) + fx_sar(w[-3 * s], e - em[k][2]);
   }
-  out[3] = fx_out<2>((((s1 >> 2) - 4 * q) * 5 - 2 * (s2 >> 2)) * 3 + (s3 >> 2), u);
+  out[3] = fx_out_cvt<2>((((s1 >> 2) - 4 * q) * 5 - 2 * (s2 >> 2)) * 3 + (s3 >> 2), u);
 }
 
 // The same in FP32 from split pairs (mixed precision), whose FP32 pipe is
@@ -113,7 +119,7 @@ __device__ __forceinline__ void point_sums(const long long *w, const unsigned *e
 // second differences from error-free differences of the high parts (the
 // reasons stand at sp_second in ccz4_algebra.cuh). On the 144^3 puncture the
 // integer sums with FP32 results took the mixed step to 15.8 ms, the pairs
-// to @@.
+// to 15.3.
 template <bool SECOND>
 __device__ __forceinline__ void point_sums(const float2 *t, const unsigned *, int T, float *out) {
   const int st[3] = {1, T, T * T};
@@ -192,7 +198,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
                                              double *__restrict__ mix, double *__restrict__ der, const LevelScale &ls,
                                              const FieldList &fl, int n, int group, int groups, bool tile_out,
                                              double *smem) {
-  constexpr int BATCH = 8;
+  constexpr int BATCH = PF == 9 && THREADS == 256 ? 7 : 8;  // 15^3 tile points: two rounds of 7 x 256
   const int p = PF > 0 ? PF : g.p, T = PF > 0 ? PF + 2 * HALO : g.T;
   const int T3 = PF > 0 ? T * T * T : (int)g.T3;
   const int pe = p + 4, next = pe * p * p, p3 = p * p * p;
