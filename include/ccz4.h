@@ -547,11 +547,11 @@ ccz4_status ccz4_tracers_free(ccz4_tracers *t);
 /* Launch shapes (a tuning choice; results are identical): the flat algebra
    kernel asks the default number of resident 128-thread blocks per SM
    (CCZ4_STAGE_SHAPE_DEFAULT), one more (MORE_BLOCKS, fewer registers per
-   thread) or one fewer (FEWER_BLOCKS, more registers); SPLIT, the stencil
-   values of a point before its algebra, is what every launch does by now
-   and equals the default; the derivative pass and the halo fill run 256
-   threads per patch (DEFAULT), 512 (WIDE) or 128 (NARROW; the pass's shapes
-   exist for 9^3 patches), the fill with 8 independent loads per thread in its
+   thread) or one fewer (FEWER_BLOCKS, more registers); SPLIT takes the
+   derivatives of all points before the algebra in a launch of its own, also on
+   the large FP64 grids of 9^3 patches where the default runs the two side by
+   side; the halo fill and the derivative pass (the pass: mixed precision, 9^3
+   patches) run 256 threads per patch (DEFAULT), 512 (WIDE) or 128 (NARROW), the fill with 8 independent loads per thread in its
    gather or 16 (DEEP). Drops a captured step graph. CCZ4_ERR_INVALID for an
    unknown shape. */
 enum { CCZ4_STAGE_SHAPE_DEFAULT = 0, CCZ4_STAGE_SHAPE_MORE_BLOCKS = 1, CCZ4_STAGE_SHAPE_FEWER_BLOCKS = 2,

@@ -94,6 +94,16 @@ extern "C" ccz4_status ccz4_set_allocator(ccz4_alloc_fn alloc, ccz4_dealloc_fn d
   return CCZ4_OK;
 }
 
+// Whether FP64 stages with derivatives beside the algebra pay. A patch costs
+// 2.3 us of the two launches (1000 patches of 9^3: 9.4 ms a step); in one launch
+// every 152 patches cost a round of 270 us and the first patch's derivatives
+// another 0.6 of one: a grid pays from 1.3 times fewer rounds on (343 patches:
+// 3.3 ms a step in two launches, 3.7 in one; 1000: 9.4 and 8.3).
+static bool pair_pays(int patches) {
+  const long long rounds = (patches + 151) / 152;
+  return 13LL * patches >= (10 * rounds + 6) * 152;
+}
+
 static size_t der_bytes(const GridView &v) { return sizeof(double) * (size_t)DER_SLOTS * (size_t)v.n_points; }
 
 // A large buffer of a grid from its allocator; NULL with the error message set on failure.
@@ -359,6 +369,7 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
   prepare_derive();
   prepare_constraints();
   if (v.p == 9) prepare_fused();
+  g->pair = v.p == 9 && pair_pays(v.n_patches) && prepare_pair(mesh != nullptr) == cudaSuccess;
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     set_error("grid set-up failed: %s", cudaGetErrorString(e));
@@ -596,16 +607,18 @@ static ccz4_status stage_kernel(ccz4_grid *g, const ccz4_params *P, int stage, d
 }
 
 // One RK4 stage of a step: the derivative pass and the algebra kernel as two
-// launches, or (CCZ4_LAUNCH_FUSED) both in one cooperative launch; the
-// restriction after stage 3 stays a launch of its own.
+// launches, on large FP64 grids in the default launch mode and shape as one
+// (stage_pair.cuh, the same arithmetic), or (CCZ4_LAUNCH_FUSED) both in one
+// cooperative launch; the restriction after stage 3 stays a launch of its own.
 static ccz4_status step_stage(ccz4_grid *g, const ccz4_params *P, int stage, double dt, cudaStream_t s) {
-  if (!g->fused) {
+  const bool pair = g->pair && !g->fused && !g->v.queue && g->v.stage_shape == 0 && P->precision != CCZ4_PREC_MIXED;
+  if (!g->fused && !pair) {
     CUDA_TRY(derivatives(g, P, kStageIn[stage], s));
     return stage_kernel(g, P, stage, dt, s);
   }
-  CUDA_TRY(launch_fused_stage(g->v, *P, stage, dt, g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der,
-                              g->buf[kStageIn[stage]], ini_ptr(g), g->buf[CCZ4_BUF_U], g->buf[CCZ4_BUF_ACC],
-                              g->buf[kStageOut[stage]], s));
+  const auto launch = pair ? launch_pair_stage : launch_fused_stage;
+  CUDA_TRY(launch(g->v, *P, stage, dt, g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der, g->buf[kStageIn[stage]],
+                  ini_ptr(g), g->buf[CCZ4_BUF_U], g->buf[CCZ4_BUF_ACC], g->buf[kStageOut[stage]], s));
   if (stage == 3 && g->v.n_levels > 1) return restrict_levels(g, g->buf[kStageOut[stage]], s);
   return CCZ4_OK;
 }

@@ -213,6 +213,7 @@ struct ccz4_grid {
   ccz4_dealloc_fn dealloc;
   void *alloc_ctx;
   int fused;                    // CCZ4_LAUNCH_FUSED: one cooperative launch per RK stage (p = 9)
+  int pair;                     // FP64 stages in one launch, derivatives beside the algebra (pair_pays)
   double *der;                  // derivative buffer, [DER_SLOTS][n_points] (derive.cuh), from the same allocator
 };
 
@@ -232,6 +233,13 @@ cudaError_t prepare_fused();
 cudaError_t launch_fused_stage(const GridView &g, const ccz4_params &P, int stage, double dt, double *tile,
                                double *mix, double *der, const double *in, const double *ini, const double *U,
                                double *acc, double *out, cudaStream_t s);
+// One FP64 RK stage with the derivative pass beside the algebra (stage_pair.cuh), p = 9 only. prepare_pair
+// raises the shared-memory limit and checks the registers of the launch (once per grid, outside any
+// stream capture).
+cudaError_t prepare_pair(bool mesh);
+cudaError_t launch_pair_stage(const GridView &g, const ccz4_params &P, int stage, double dt, double *tile, double *mix,
+                              double *der, const double *in, const double *ini, const double *U, double *acc, double *out,
+                              cudaStream_t s);
 // psi_4 at every interior point from the derivative pass over `in`: Re into out[0 .. n_points), Im into
 // out[S ..), the tetrad centred at centre (psi4.cu)
 cudaError_t launch_psi4(const GridView &g, const double *der, const double *mix, const double *in,

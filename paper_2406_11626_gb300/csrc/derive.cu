@@ -1,5 +1,5 @@
 // The derivative pass (derive.cuh): kernels and launches.
-#include "derive.cuh"
+#include "derive_edge.cuh"
 
 namespace ccz4 {
 namespace {
@@ -11,6 +11,26 @@ __global__ void __launch_bounds__(FILL_SHAPE_THREADS[SHAPE], (PF == 9 ? 1024 : 7
   extern __shared__ double smem[];
   derive_patch<SRC, MIXED, RAW, FILL_SHAPE_THREADS[SHAPE], PF, NF>(g, src, tile, mix, der, ls, fl, blockIdx.x,
                                                                    blockIdx.y, gridDim.y, tile_out, smem);
+}
+
+template <int SRC, int PF>
+__global__ void __launch_bounds__(EdgeShape<PF>::threads, EdgeShape<PF>::blocks)
+    derive_edge_kernel(GridView g, const double *__restrict__ src, double *tile, double *__restrict__ mix,
+                       double *__restrict__ der, LevelScale ls, FieldList fl) {
+  extern __shared__ double smem[];
+  derive_edge<SRC, EdgeShape<PF>::threads, PF, true>(g, src, tile, mix, der, ls, fl, blockIdx.x, blockIdx.y, gridDim.y,
+                                                     smem, threadIdx.x, 0);
+}
+
+// One field per block, 9^3 patches: small grids, whose every block is resident at once.
+constexpr int ONE_THREADS = 256;
+template <int SRC>
+__global__ void __launch_bounds__(ONE_THREADS, 4)
+    derive_field_kernel(GridView g, const double *__restrict__ src, double *tile, double *__restrict__ mix,
+                        double *__restrict__ der, LevelScale ls, FieldList fl) {
+  extern __shared__ double smem[];
+  derive_edge<SRC, ONE_THREADS, 9, true, true>(g, src, tile, mix, der, ls, fl, blockIdx.x, blockIdx.y, fl.n, smem,
+                                               threadIdx.x, 0);
 }
 
 // Field groups per patch. A block's set-up (the source table) is shared by
@@ -33,6 +53,19 @@ cudaError_t launch_one(const GridView &g, const double *src, double *tile, doubl
   return cudaGetLastError();
 }
 
+template <int SRC, int PF>
+cudaError_t launch_fixed(const GridView &g, const double *src, double *tile, double *mix, double *der,
+                         const FieldList &fl, cudaStream_t s) {
+  if (PF == 9 && field_groups(g, fl) == fl.n) {
+    derive_field_kernel<SRC><<<dim3(g.n_patches, fl.n), ONE_THREADS, edge_smem_bytes(9, true), s>>>(
+        g, src, tile, mix, der, level_scale(g), fl);
+    return cudaGetLastError();
+  }
+  derive_edge_kernel<SRC, PF><<<dim3(g.n_patches, field_groups(g, fl)), EdgeShape<PF>::threads, edge_smem_bytes(PF), s>>>(
+      g, src, tile, mix, der, level_scale(g), fl);
+  return cudaGetLastError();
+}
+
 template <int SRC, bool MIXED, int SHAPE>
 cudaError_t launch_edge(const GridView &g, const double *src, double *tile, double *mix, double *der,
                         const FieldList &fl, bool tile_out, cudaStream_t s) {
@@ -48,7 +81,16 @@ cudaError_t launch_edge(const GridView &g, const double *src, double *tile, doub
 template <int SRC, bool MIXED>
 cudaError_t launch_shape(const GridView &g, const double *src, double *tile, double *mix, double *der,
                          const FieldList &fl, bool tile_out, cudaStream_t s) {
-  if constexpr (SRC != FROM_TILE) {
+  if constexpr (SRC != FROM_TILE && !MIXED) {
+    // All 25 fields (a right-hand side): the edges of the study of patch sizes that leave room for the
+    // widened first derivatives. The monitors' passes, which leave the FP64 pipe idle and write the
+    // tiles too, stay with the general body (constraints at 144^3: 5.84 ms with it, 6.09 otherwise).
+    if (!tile_out) {
+      if (g.p == 9) return launch_fixed<SRC, 9>(g, src, tile, mix, der, fl, s);
+      if (g.p == 12) return launch_fixed<SRC, 12>(g, src, tile, mix, der, fl, s);
+      if (g.p == 6) return launch_fixed<SRC, 6>(g, src, tile, mix, der, fl, s);
+    }
+  } else if constexpr (SRC != FROM_TILE) {
     if (g.fill_shape == 1) return launch_edge<SRC, MIXED, 1>(g, src, tile, mix, der, fl, tile_out, s);
     if (g.fill_shape == 3) return launch_edge<SRC, MIXED, 3>(g, src, tile, mix, der, fl, tile_out, s);
   }
@@ -69,12 +111,26 @@ int largest_edge(bool raw) {
   return q;
 }
 
+template <int SRC, int PF>
+cudaError_t prepare_fixed() {
+  return cudaFuncSetAttribute(derive_edge_kernel<SRC, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)edge_smem_bytes(PF));
+}
+
 template <int SRC, bool MIXED>
 cudaError_t prepare_source() {
   cudaError_t e = prepare_one<SRC, MIXED, false, 0, 9, NV>(9);
+  if constexpr (SRC != FROM_TILE && !MIXED) {
+    if (e == cudaSuccess) e = prepare_fixed<SRC, 9>();
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(derive_field_kernel<SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)edge_smem_bytes(9, true));
+    if (e == cudaSuccess) e = prepare_fixed<SRC, 12>();
+    if (e == cudaSuccess) e = prepare_fixed<SRC, 6>();
+  }
   if (e == cudaSuccess) e = prepare_one<SRC, MIXED, false, 0, 0, NV>(largest_edge(false));
   if (e == cudaSuccess) e = prepare_one<SRC, MIXED, true, 0, 0, NV>(largest_edge(true));
-  if constexpr (SRC != FROM_TILE) {
+  if constexpr (SRC != FROM_TILE && MIXED) {
     if (e == cudaSuccess) e = prepare_one<SRC, MIXED, false, 1, 9, NV>(9);
     if (e == cudaSuccess) e = prepare_one<SRC, MIXED, false, 3, 9, NV>(9);
   }

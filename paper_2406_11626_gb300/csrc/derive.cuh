@@ -51,15 +51,28 @@ __device__ __forceinline__ long long fx_sar(long long x, unsigned s) {
   return r;
 }
 
+// A zero that the compiler cannot move or foresee: what depends on it is not evaluated ahead of the
+// branch it stands in.
+__device__ __forceinline__ int here_zero() {
+  int z;
+  asm volatile("mov.u32 %0, 0;" : "=r"(z));
+  return z;
+}
+
 // The stencil sums of one point whose largest neighbour lies outside [FX_FLOOR, FX_TOP), in FP64.
-template <bool SECOND>
-__device__ __noinline__ void point_sums_fp64(const long long *w, const unsigned *ex, int T, double *out) {
+// Inline: a call's registers would be its callee's choice.
+template <bool SECOND, class E>
+__device__ __forceinline__ void point_sums_fp64(const long long *w, const E *ex, int T, double *out) {
+  const int z = here_zero();
+  w += z;
+  ex += z;
   const int st[3] = {1, T, T * T};
   const double c = fx_value(w[0], ex[0]);
   double s[3] = {0.0, 0.0, 0.0};
-#pragma unroll 1
+#pragma unroll
   for (int k = 0; k < 3; ++k) {
     double p[3], m[3];
+#pragma unroll
     for (int j = 0; j < 3; ++j) {
       const int o = (j + 1) * st[k];
       p[j] = fx_value(w[o], ex[o]);
@@ -72,10 +85,18 @@ __device__ __noinline__ void point_sums_fp64(const long long *w, const unsigned 
   out[3] = fma(-60.0, c, fma(15.0, s[0], fma(-6.0, s[1], s[2])));
 }
 
+template <bool CVT>
+__device__ __forceinline__ double fx_return(long long v, unsigned unit) {
+  if constexpr (CVT) return fx_out_cvt<2>(v, unit);
+  else return fx_out<2, true>(v, unit);
+}
+
 // The stencil sums of the point at w, ex: out[0..2] first derivatives, out[3]
-// dissipation, out[4..6] pure second derivatives.
-template <bool SECOND>
-__device__ __forceinline__ void point_sums(const long long *w, const unsigned *ex, int T, double *out) {
+// dissipation, out[4..6] pure second derivatives. CVT: the second sums return by
+// the conversion instruction, or else in integers with the same rounding (for a
+// kernel whose other warps hold the FP64 pipe).
+template <bool SECOND, bool CVT = true, class E>
+__device__ __forceinline__ void point_sums(const long long *w, const E *ex, int T, double *out) {
   const int st[3] = {1, T, T * T};
   const unsigned e0 = ex[0];
   unsigned ep[3][3], em[3][3], e = e0;
@@ -106,12 +127,12 @@ __device__ __forceinline__ void point_sums(const long long *w, const unsigned *e
     const long long p2 = fx_sar(w[2 * s], e - ep[k][1]), m2 = fx_sar(w[-2 * s], e - em[k][1]);
     const long long t1 = p1 + m1, t2 = p2 + m2;
     out[k] = fx_out<4>((p1 - m1) * 8 - (p2 - m2), u);
-    if (SECOND) out[4 + k] = fx_out_cvt<2>(((t1 >> 2) - 2 * q) * 16 - (t2 >> 2) + 2 * q, u);
+    if (SECOND) out[4 + k] = fx_return<CVT>(((t1 >> 2) - 2 * q) * 16 - (t2 >> 2) + 2 * q, u);
     s1 += t1;
     s2 += t2;
     s3 += fx_sar(w[3 * s], e - ep[k][2]) + fx_sar(w[-3 * s], e - em[k][2]);
   }
-  out[3] = fx_out_cvt<2>((((s1 >> 2) - 4 * q) * 5 - 2 * (s2 >> 2)) * 3 + (s3 >> 2), u);
+  out[3] = fx_return<CVT>((((s1 >> 2) - 4 * q) * 5 - 2 * (s2 >> 2)) * 3 + (s3 >> 2), u);
 }
 
 // The same in FP32 from split pairs (mixed precision), whose FP32 pipe is

@@ -84,8 +84,9 @@ __host__ __device__ __forceinline__ int64_t fx_in(double u, unsigned unit) {
   return (int64_t)((a ^ n) - n);
 }
 
-// v units of 2^(e - 1075 - K) as FP64, rounded to nearest (ties away from zero)
-template <int K>
+// v units of 2^(e - 1075 - K) as FP64, rounded to nearest (ties away from zero; EVEN: to even, as the
+// conversion instruction rounds)
+template <int K, bool EVEN = false>
 __host__ __device__ __forceinline__ double fx_out(int64_t v, unsigned unit) {
   const uint64_t n = (uint64_t)(v >> 63), a = ((uint64_t)v ^ n) - n;
 #ifdef __CUDA_ARCH__
@@ -94,7 +95,8 @@ __host__ __device__ __forceinline__ double fx_out(int64_t v, unsigned unit) {
   const int z = a ? __builtin_clzll(a) : 64;
 #endif
   const uint64_t t = a << (z & 63);                 // top bit set (0 for v = 0)
-  const uint64_t r = (t >> 11) + ((t >> 10) & 1u);  // 53 bits, a carry goes into the exponent
+  const unsigned up = EVEN && (t & 0x3FFu) == 0 ? (unsigned)(t >> 11) & 1u : 1u;
+  const uint64_t r = (t >> 11) + ((unsigned)(t >> 10) & up);  // 53 bits, a carry goes into the exponent
   const uint64_t e = (uint64_t)((unit >> 21) + 10u - K - (unsigned)z) << 52;
   const uint64_t w = ((n & 0x8000000000000000ull) | e) + r;
   return a ? fx_from_bits(w) : 0.0;

@@ -12,6 +12,7 @@
 #define CCZ4_DER_LOAD __ldcg
 #include <cooperative_groups.h>
 
+#include "derive_edge.cuh"
 #include "stage_kernels.cuh"
 
 namespace ccz4 {
@@ -27,8 +28,11 @@ __global__ void __launch_bounds__(FUSED_THREADS, (StageBlocks<R, 0>::value))
                        const double *__restrict__ ini, StageArgs a) {
   extern __shared__ double smem[];
   for (int n = blockIdx.x; n < g.n_patches; n += gridDim.x) {
-    derive_patch<MESH ? FROM_MESH : FROM_LEVEL, std::is_same<R, float>::value, false, FUSED_THREADS, FUSED_PF, NV>(
-        g, in, tile, mix, der, ls, fl, n, 0, 1, false, smem);
+    constexpr int SRC = MESH ? FROM_MESH : FROM_LEVEL;
+    if constexpr (std::is_same<R, float>::value)
+      derive_patch<SRC, true, false, FUSED_THREADS, FUSED_PF, NV>(g, in, tile, mix, der, ls, fl, n, 0, 1, false, smem);
+    else
+      derive_edge<SRC, FUSED_THREADS, FUSED_PF, true>(g, in, tile, mix, der, ls, fl, n, 0, 1, smem, threadIdx.x, 0);
     __syncthreads();  // the next patch's source table overwrites this one's shared memory
   }
   cooperative_groups::this_grid().sync();
@@ -45,6 +49,11 @@ __global__ void __launch_bounds__(FUSED_THREADS, (StageBlocks<R, 0>::value))
       if (i < g.n_points) stage_point<MODE, R, MESH>(g, P, LC, b, a, i);
     }
   }
+}
+
+template <class R>
+size_t fused_smem_bytes() {
+  return std::is_same<R, float>::value ? derive_smem_bytes(FUSED_PF, false) : edge_smem_bytes(FUSED_PF);
 }
 
 template <int MODE, class R, bool MESH>
@@ -72,7 +81,7 @@ template <int MODE, class R, bool MESH>
 cudaError_t launch_fused_as(const GridView &g, const ccz4_params &P, double *tile, double *mix, double *der,
                             const double *in, const double *ini, const StageArgs &a, cudaStream_t s) {
   const void *fn = fused_fn<MODE, R, MESH>();
-  const size_t smem = derive_smem_bytes(FUSED_PF, false);
+  const size_t smem = fused_smem_bytes<R>();
   int dev = 0, sms = 0, occ = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -114,10 +123,10 @@ cudaError_t launch_fused_mode(const GridView &g, const ccz4_params &P, double *t
 }  // namespace
 
 cudaError_t prepare_fused() {
-  const int bytes = (int)derive_smem_bytes(FUSED_PF, false);
   for (int m = 0; m < 4; ++m)
     for (int x = 0; x < 2; ++x)
       for (int h = 0; h < 2; ++h) {
+        const int bytes = (int)(x ? fused_smem_bytes<float>() : fused_smem_bytes<double>());
         cudaError_t e = cudaFuncSetAttribute(fused_any(m, x, h), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess) return e;
       }
