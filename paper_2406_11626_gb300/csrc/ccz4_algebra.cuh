@@ -615,6 +615,7 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
   // Gd[k][ij] = G~_kij = (d_i g~_jk + d_j g~_ik - d_k g~_ij) / 2 ; Gu[k][ij] = G~^k_ij
   R Gd[3][6], Gu[3][6], Gc[3];
   R advg[6], Ghdg[6];  // beta^k d_k g~_ij and Gamma-hat^k d_k g~_ij
+  R dg[3][6];          // (1/2) d_k g~_ij
   {
     // half the derivatives, so that the 1/2 of G~_kij costs nothing; the
     // contractions with beta and Gamma-hat take them doubled (all exact
@@ -622,18 +623,21 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
     const R c1h = R(0.5) * CR.c1;
     const R be2[3] = {be[0] + be[0], be[1] + be[1], be[2] + be[2]};
     const R Gh2[3] = {Gh[0] + Gh[0], Gh[1] + Gh[1], Gh[2] + Gh[2]};
-    R dg[3][6];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
-      for (int c = 0; c < 6; ++c) dg[k][c] = d1o<D, R>(N, GXX + c, N.st[k], c1h);  // (1/2) d_k g~_ij
+      for (int c = 0; c < 6; ++c) dg[k][c] = d1o<D, R>(N, GXX + c, N.st[k], c1h);
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
       for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = i; j < 3; ++j)
-          Gd[k][S6(i, j)] = dg[i][S6(j, k)] + dg[j][S6(i, k)] - dg[k][S6(i, j)];
+          // two of the three derivatives are the same where k is i or j, and where i is j
+          Gd[k][S6(i, j)] = k == i   ? dg[j][S6(i, k)]
+                            : k == j ? dg[i][S6(j, k)]
+                            : i == j ? fmaT(R(2.0), dg[i][S6(i, k)], -dg[k][S6(i, i)])
+                                     : dg[i][S6(j, k)] + dg[j][S6(i, k)] - dg[k][S6(i, j)];
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       advg[c] = fmaT(be2[0], dg[0][c], fmaT(be2[1], dg[1][c], be2[2] * dg[2][c]));
@@ -660,8 +664,9 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
   CCZ4_MARK("christoffel");
 
   // ---- quadratic Christoffel part of the Ricci tensor -------------------------
-  // Cm[k][i][m] = g~^lm G~^k_li. With it, g~^lm G~^k_li G~_jkm = sum_km Cm[k][i][m] G~_jkm
-  // and g~^lm G~^k_im G~_klj = sum_kl Cm[k][i][l] G~_klj; Q6_ij collects the three terms.
+  // Cm[k][i][m] = g~^lm G~^k_li. With it the three terms are
+  // sum_km Cm[k][i][m] (G~_jkm + G~_kmj) + sum_km Cm[k][j][m] G~_ikm, where G~_jkm + G~_kmj = d_m g~_jk
+  // and G~_ikm is symmetric in k and m.
   R Q6[6];
   {
     R Cm[3][3][3];
@@ -673,25 +678,23 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
         for (int m = 0; m < 3; ++m)
           Cm[k][i][m] = fmaT(ig[S6(0, m)], Gu[k][S6(0, i)],
                              fmaT(ig[S6(1, m)], Gu[k][S6(1, i)], ig[S6(2, m)] * Gu[k][S6(2, i)]));
-    R X[3][3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) {
+      const R Cs[3] = {Cm[0][j][1] + Cm[1][j][0], Cm[0][j][2] + Cm[2][j][0], Cm[1][j][2] + Cm[2][j][1]};
 #pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        R s = Cm[0][i][0] * Gd[j][S6(0, 0)];
+      for (int i = 0; i <= j; ++i) {
+        R x = Cm[0][j][0] * Gd[i][0];
+        x = fmaT(Cm[1][j][1], Gd[i][3], x);
+        x = fmaT(Cm[2][j][2], Gd[i][5], x);
+        x = fmaT(Cs[0], Gd[i][1], x);
+        x = fmaT(Cs[1], Gd[i][2], x);
+        x = fmaT(Cs[2], Gd[i][4], x);
+        R y = Cm[0][i][0] * dg[0][S6(j, 0)];
 #pragma unroll
-        for (int q = 1; q < 9; ++q) s = fmaT(Cm[q / 3][i][q % 3], Gd[j][S6(q / 3, q % 3)], s);
-        X[i][j] = s;
+        for (int q = 1; q < 9; ++q) y = fmaT(Cm[q / 3][i][q % 3], dg[q % 3][S6(j, q / 3)], y);
+        Q6[S6(i, j)] = fmaT(R(2.0), y, x);
       }
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = i; j < 3; ++j) {
-        R q3 = X[i][j] + X[j][i];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) q3 = fmaT(Cm[q / 3][i][q % 3], Gd[q / 3][S6(q % 3, j)], q3);
-        Q6[S6(i, j)] = q3;
-      }
+    }
   }
   CCZ4_MARK("ricci quadratic");
 
@@ -801,8 +804,12 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
 #pragma unroll
         for (int q = 1; q < 6; ++q) lap = fmaT(igwc[q], dd[q], lap);
         R u = Ghdg[c];
+        if (i == j) {
+          u = fmaT(R(2.0), fmaT(g[S6(0, i)], dG[i][0], fmaT(g[S6(1, i)], dG[i][1], g[S6(2, i)] * dG[i][2])), u);
+        } else {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) u = fmaT(g[S6(k, i)], dG[j][k], fmaT(g[S6(k, j)], dG[i][k], u));
+          for (int k = 0; k < 3; ++k) u = fmaT(g[S6(k, i)], dG[j][k], fmaT(g[S6(k, j)], dG[i][k], u));
+        }
         RZ[c] = fmaT(R(-0.5), lap, fmaT(R(0.5), u, Q6[c] + phiRZ[c]));
       }
   }
@@ -818,7 +825,7 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
   R A[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) A[c] = centre<D, R>(N, AXX + c);
-  R Au[6], AgA[6];
+  R Au[6], AgA[6], trA;
   {
     R Am[3][3];  // A~_i^m = A~_il g~^lm
 #pragma unroll
@@ -826,6 +833,7 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
 #pragma unroll
       for (int m = 0; m < 3; ++m)
         Am[i][m] = fmaT(A[S6(i, 0)], ig[S6(0, m)], fmaT(A[S6(i, 1)], ig[S6(1, m)], A[S6(i, 2)] * ig[S6(2, m)]));
+    trA = Am[0][0] + Am[1][1] + Am[2][2];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -834,8 +842,6 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
         AgA[S6(i, j)] = fmaT(Am[i][0], A[S6(0, j)], fmaT(Am[i][1], A[S6(1, j)], Am[i][2] * A[S6(2, j)]));
       }
   }
-  const R trA = fmaT(igw[0], A[0], fmaT(igw[1], A[1], fmaT(igw[2], A[2], fmaT(igw[3], A[3],
-                fmaT(igw[4], A[4], igw[5] * A[5])))));
   const R Auw[6] = {Au[0], Au[1] + Au[1], Au[2] + Au[2], Au[3], Au[4] + Au[4], Au[5]};
   R AA = A[0] * Auw[0];
 #pragma unroll
@@ -865,15 +871,6 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
   const R Kc = fmaT(-P.c2, Th, Kt);  // K - 2 c Theta
   const R al2 = al + al;
   {
-    // Lie-derivative parts: Xg_ij = g~_ki B_j^k, XA_ij = A~_ki B_j^k, used as X_ij + X_ji
-    R Xg[3][3], XA[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        Xg[i][j] = fmaT(g[S6(0, i)], dB[j][0], fmaT(g[S6(1, i)], dB[j][1], g[S6(2, i)] * dB[j][2]));
-        XA[i][j] = fmaT(A[S6(0, i)], dB[j][0], fmaT(A[S6(1, i)], dB[j][1], A[S6(2, i)] * dB[j][2]));
-      }
     const R trMx = fmaT(al, trRZ, -trDDa);  // g~^ij (-nabla_i nabla_j alpha + alpha RZ_ij)
     const R sg = fmaT(twothird * al, trA, -trB23) - P.itau * (det - R(1.0));
     const R ph2al = ph2 * al;
@@ -884,11 +881,22 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
 #pragma unroll
       for (int j = i; j < 3; ++j) {
         const int c = S6(i, j);
-        sink(GXX + c, add_ko<D, R>(fmaT(g[c], sg, fmaT(-al2, A[c], advg[c] + (Xg[i][j] + Xg[j][i]))), kog[c], C, CR));
-        R advA = XA[i][j] + XA[j][i];  // the advection and Lie-derivative terms
+        // the advection and Lie-derivative terms, beta^k d_k T_ij + T_ki B_j^k + T_kj B_i^k
+        R lg = advg[c], lA = bec1[0] * d1u<D, R>(N, AXX + c, N.st[0]);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) advA = fmaT(bec1[k], d1u<D, R>(N, AXX + c, N.st[k]), advA);
-        const R rA = fmaT(ph2al, RZ[c], fmaT(-ph2, DDa[c], fmaT(g[c], sA1, fmaT(A[c], sA2, fmaT(-al2, AgA[c], advA)))));
+        for (int k = 1; k < 3; ++k) lA = fmaT(bec1[k], d1u<D, R>(N, AXX + c, N.st[k]), lA);
+        if (i == j) {
+          lg = fmaT(R(2.0), fmaT(g[S6(0, i)], dB[i][0], fmaT(g[S6(1, i)], dB[i][1], g[S6(2, i)] * dB[i][2])), lg);
+          lA = fmaT(R(2.0), fmaT(A[S6(0, i)], dB[i][0], fmaT(A[S6(1, i)], dB[i][1], A[S6(2, i)] * dB[i][2])), lA);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            lg = fmaT(g[S6(k, i)], dB[j][k], fmaT(g[S6(k, j)], dB[i][k], lg));
+            lA = fmaT(A[S6(k, i)], dB[j][k], fmaT(A[S6(k, j)], dB[i][k], lA));
+          }
+        }
+        sink(GXX + c, add_ko<D, R>(fmaT(g[c], sg, fmaT(-al2, A[c], lg)), kog[c], C, CR));
+        const R rA = fmaT(ph2al, RZ[c], fmaT(-ph2, DDa[c], fmaT(g[c], sA1, fmaT(A[c], sA2, fmaT(-al2, AgA[c], lA)))));
         sink(AXX + c, add_ko<D, R>(rA, kosum<D, R>(N, AXX + c), C, CR));
       }
   }
@@ -952,23 +960,30 @@ __host__ __device__ __forceinline__ void ccz4_rhs_point(const Phys<R> &P, NB &N,
   R wv[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) wv[k] = fmaT(al2c, dT[k], fmaT(-al43c, dK[k], fmaT(P.s3, gdivB[k], -Th2 * da[k])));
+  // -(G~^k - k3h (Gamma-hat^k - G~^k)) contracts with B_k^i; FP64 path: A~^ij with
+  // one vector, -6 alpha P_j / phi - 2 A_j (mixed path: the P_j / phi part in D)
+  R yv[3], av[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    yv[k] = fmaT(k3h, dGam[k], -Gc[k]);
+    if constexpr (SAME) av[k] = fmaT(-al6 * iph, dPD[k], -(da[k] + da[k]));
+  }
   R dbK[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    const R AuA = fmaT(Au[S6(i, 0)], da[0], fmaT(Au[S6(i, 1)], da[1], Au[S6(i, 2)] * da[2]));
-    const R ZB = fmaT(dGam[0], dB[0][i], fmaT(dGam[1], dB[1][i], dGam[2] * dB[2][i]));
-    // the 3 A~^ij P_j / phi term, in D
-    const D AuP = fmaT(cvt<D>(Au[S6(i, 0)]), dPD[0], fmaT(cvt<D>(Au[S6(i, 1)]), dPD[1], cvt<D>(Au[S6(i, 2)]) * dPD[2]));
-    const R AuPphi = cvt<R>(AuP * iph);
     R t = fmaT(ig[S6(i, 0)], wv[0], fmaT(ig[S6(i, 1)], wv[1], fmaT(ig[S6(i, 2)], wv[2], lapB[i])));
     t = fmaT(al2, GA[i], t);
     t = fmaT(trB23, Gc[i], t);
-    t = fmaT(-al6, AuPphi, t);
-    t = fmaT(R(-2.0), AuA, t);
+    if constexpr (SAME) {
+      t = fmaT(Au[S6(i, 0)], av[0], fmaT(Au[S6(i, 1)], av[1], fmaT(Au[S6(i, 2)], av[2], t)));
+    } else {
+      const R AuA = fmaT(Au[S6(i, 0)], da[0], fmaT(Au[S6(i, 1)], da[1], Au[S6(i, 2)] * da[2]));
+      const D AuP = fmaT(cvt<D>(Au[S6(i, 0)]), dPD[0], fmaT(cvt<D>(Au[S6(i, 1)]), dPD[1], cvt<D>(Au[S6(i, 2)]) * dPD[2]));
+      t = fmaT(R(-2.0), AuA, fmaT(-al6, cvt<R>(AuP * iph), t));
+    }
     t = fmaT(zc, dGam[i], t);
-    t = fmaT(k3h, ZB, t);
-    // - G~^k B_k^i; d_t Gamma-hat^i - beta^k d_k Gamma-hat^i
-    dbK[i] = fmaT(-Gc[0], dB[0][i], fmaT(-Gc[1], dB[1][i], fmaT(-Gc[2], dB[2][i], t)));
+    // d_t Gamma-hat^i - beta^k d_k Gamma-hat^i
+    dbK[i] = fmaT(yv[0], dB[0][i], fmaT(yv[1], dB[1][i], fmaT(yv[2], dB[2][i], t)));
     sink(GHX + i, add_ko<D, R>(advGh[i] + dbK[i], kosum<D, R>(N, GHX + i), C, CR));
   }
   if (P.shift == CCZ4_SHIFT_GAMMA_DRIVER) {
