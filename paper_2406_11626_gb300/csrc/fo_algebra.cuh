@@ -74,6 +74,14 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
   for (int k = 0; k < 3; ++k)
 #pragma unroll
     for (int c = 0; c < 6; ++c) Dv[k][c] = ld<D>(N, FD + 6 * k + c, 0);
+  // first differences are taken without 1 / (12 dx) and their contractions carry it: with
+  // beta, with g~^ij, or once in the sum (fewer FP64 multiplies)
+  const D h1 = D(0.5) * c1, alc = al * c1;
+  D bec[3], igc[6];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) bec[i] = be[i] * c1;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) igc[c] = ig[c] * c1;
   // G~_lij = D_ijl + D_jil - D_lij (lowered), G~^k_ij = g~^kl G~_lij, G~^k = g~^ij G~^k_ij
   D Gd[3][6], Gu[3][6], Gc[3];
 #pragma unroll
@@ -81,7 +89,12 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-      for (int j = i; j < 3; ++j) Gd[l][S6_fo(i, j)] = Dv[i][S6_fo(j, l)] + Dv[j][S6_fo(i, l)] - Dv[l][S6_fo(i, j)];
+      for (int j = i; j < 3; ++j)
+        // two of the three are the same where l is i or j, and where i is j
+        Gd[l][S6_fo(i, j)] = l == i   ? Dv[j][S6_fo(i, l)]
+                             : l == j ? Dv[i][S6_fo(j, l)]
+                             : i == j ? fmaT(D(2.0), Dv[i][S6_fo(i, l)], -Dv[l][S6_fo(i, i)])
+                                      : Dv[i][S6_fo(j, l)] + Dv[j][S6_fo(i, l)] - Dv[l][S6_fo(i, j)];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
 #pragma unroll
@@ -100,31 +113,29 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
   D At[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) At[c] = ld<D>(N, AXX + c, 0);
-  const D trA = fmaT(igw[0], At[0], fmaT(igw[1], At[1], fmaT(igw[2], At[2], fmaT(igw[3], At[3],
-                fmaT(igw[4], At[4], igw[5] * At[5])))));
   const D trB = B[0][0] + B[1][1] + B[2][2];
-  const D third = 1.0 / 3.0, twothird = 2.0 / 3.0;
+  const D third = 1.0 / 3.0, twothird = 2.0 / 3.0, trB23 = twothird * trB;
 
   // ---- derivatives of B: d_(k B_j)^m, the advection of B, g~^kl d_k B_l^i, d_(k B_l)^l ----
   D sB[6][3], advB[3][3], lapB[3], gdivB[3];
   {
-    D dB[3][3][3];  // dB[k][l][i] = d_k B_l^i
+    D dB[3][3][3];  // dB[k][l][i] = 12 dx d_k B_l^i
 #pragma unroll
     for (int l = 0; l < 3; ++l)
 #pragma unroll
       for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) dB[k][l][i] = fd1<D>(N, FB + 3 * l + i, N.st[k], c1);
+        for (int k = 0; k < 3; ++k) dB[k][l][i] = d1u<D, D>(N, FB + 3 * l + i, N.st[k]);
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
-      for (int i = 0; i < 3; ++i) advB[k][i] = fmaT(be[0], dB[0][k][i], fmaT(be[1], dB[1][k][i], be[2] * dB[2][k][i]));
+      for (int i = 0; i < 3; ++i) advB[k][i] = fmaT(bec[0], dB[0][k][i], fmaT(bec[1], dB[1][k][i], bec[2] * dB[2][k][i]));
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
       for (int j = k; j < 3; ++j)
 #pragma unroll
-        for (int m = 0; m < 3; ++m) sB[S6_fo(k, j)][m] = D(0.5) * (dB[k][j][m] + dB[j][k][m]);
+        for (int m = 0; m < 3; ++m) sB[S6_fo(k, j)][m] = k == j ? c1 * dB[k][k][m] : h1 * (dB[k][j][m] + dB[j][k][m]);
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -139,29 +150,29 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
   // ---- derivatives of A and P: d_(i A_j), d_(i P_j), advection, the curl of P ------------
   D ddA[6], ddP[6], advA[3], advP[3], curlP[3];  // curlP[k][j] as (yz, zx, xy): d_y P_z - d_z P_y, ...
   {
-    D dA[3][3], dP[3][3];  // dA[k][i] = d_k A_i
+    D dA[3][3], dP[3][3];  // dA[k][i] = 12 dx d_k A_i
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        dA[k][i] = fd1<D>(N, FA + i, N.st[k], c1);
-        dP[k][i] = fd1<D>(N, FP + i, N.st[k], c1);
+        dA[k][i] = d1u<D, D>(N, FA + i, N.st[k]);
+        dP[k][i] = d1u<D, D>(N, FP + i, N.st[k]);
       }
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int j = i; j < 3; ++j) {
-        ddA[S6_fo(i, j)] = D(0.5) * (dA[i][j] + dA[j][i]);
-        ddP[S6_fo(i, j)] = D(0.5) * (dP[i][j] + dP[j][i]);
+        ddA[S6_fo(i, j)] = i == j ? c1 * dA[i][i] : h1 * (dA[i][j] + dA[j][i]);
+        ddP[S6_fo(i, j)] = i == j ? c1 * dP[i][i] : h1 * (dP[i][j] + dP[j][i]);
       }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      advA[k] = fmaT(be[0], dA[0][k], fmaT(be[1], dA[1][k], be[2] * dA[2][k]));
-      advP[k] = fmaT(be[0], dP[0][k], fmaT(be[1], dP[1][k], be[2] * dP[2][k]));
+      advA[k] = fmaT(bec[0], dA[0][k], fmaT(bec[1], dA[1][k], bec[2] * dA[2][k]));
+      advP[k] = fmaT(bec[0], dP[0][k], fmaT(bec[1], dP[1][k], bec[2] * dP[2][k]));
     }
-    curlP[0] = dP[1][2] - dP[2][1];
-    curlP[1] = dP[2][0] - dP[0][2];
-    curlP[2] = dP[0][1] - dP[1][0];
+    curlP[0] = c1 * (dP[1][2] - dP[2][1]);
+    curlP[1] = c1 * (dP[2][0] - dP[0][2]);
+    curlP[2] = c1 * (dP[0][1] - dP[1][0]);
   }
 
   // ---- derivatives of A~: its advection and g~^nm d_k A~_nm --------------------------------
@@ -173,17 +184,17 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
       D a = 0.0;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const D d = fd1<D>(N, AXX + c, N.st[k], c1);
-        a = fmaT(be[k], d, a);
+        const D d = d1u<D, D>(N, AXX + c, N.st[k]);
+        a = fmaT(bec[k], d, a);
         s[k] = fmaT(igw[c], d, s[k]);
       }
       advAt[c] = a;
     }
 #pragma unroll
-    for (int k = 0; k < 3; ++k) gdAt[k] = s[k];
+    for (int k = 0; k < 3; ++k) gdAt[k] = c1 * s[k];
   }
   // D_k^nm A~_nm = A~^ab D_kab, with A~^ab = g~^an g~^bm A~_nm
-  D Au[6];
+  D Au[6], trA;
   {
     D Am[3][3];
 #pragma unroll
@@ -191,6 +202,7 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
 #pragma unroll
       for (int m = 0; m < 3; ++m)
         Am[i][m] = fmaT(At[S6_fo(i, 0)], ig[S6_fo(0, m)], fmaT(At[S6_fo(i, 1)], ig[S6_fo(1, m)], At[S6_fo(i, 2)] * ig[S6_fo(2, m)]));
+    trA = Am[0][0] + Am[1][1] + Am[2][2];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -210,7 +222,7 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
   // ---- derivatives of D: g~^kl d_k D_lij (the Laplacian of g~), the D_kij equation and,
   //      with the red terms, the mu term g~^ij g~^nl (d_k D_ljn - d_l D_kjn) of B ---------------
   D lapg[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  D m2[3][3];
+  D m2[3][3];  // without 1 / (12 dx)
 #pragma unroll
   for (int k = 0; k < 3; ++k)
 #pragma unroll
@@ -222,12 +234,12 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
     for (int a = 0; a < 3; ++a) {  // derivative direction
       D M[6];
 #pragma unroll
-      for (int c = 0; c < 6; ++c) M[c] = fd1<D>(N, FD + 6 * b + c, N.st[a], c1);  // d_a D_b,c
-      const D w = ig[S6_fo(a, b)];
+      for (int c = 0; c < 6; ++c) M[c] = d1u<D, D>(N, FD + 6 * b + c, N.st[a]);  // 12 dx d_a D_b,c
+      const D w = igc[S6_fo(a, b)];
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
         lapg[c] = fmaT(w, M[c], lapg[c]);
-        advD[c] = fmaT(be[a], M[c], advD[c]);
+        advD[c] = fmaT(bec[a], M[c], advD[c]);
       }
       if (RED && AUX && driver) {
         // H = g~^-1 M g~^-1; term 1 adds H[i][b] to m2[a][i], term 2 subtracts H[i][a] from m2[b][i]
@@ -249,23 +261,36 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
     }
     if (AUX) {
       // the D_bij equation: advection, shift terms, -alpha d_b A~_ij, the B D terms, -A_b (A~ - g~ tr A~ / 3)
-      const D sgd = gdivB[b];
+      // (the terms with g~_ij share one coefficient)
+      D cg = fmaT(third * trA, Av[b], -P.s3 * gdivB[b]);
+      if (RED) cg = fmaT(third * al, fmaT(D(-2.0), DuA[b], gdAt[b]), cg);
+      const D s15 = D(1.5) * P.s3;
 #pragma unroll
       for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = i; j < 3; ++j) {
           const int c = S6_fo(i, j);
-          D sh = third * g[c] * sgd;
+          D sh = D(0.0), r = fmaT(-trB23, Dv[b][c], advD[c]);
+          if (i == j) {
+            D BD = D(0.0);
 #pragma unroll
-          for (int m = 0; m < 3; ++m) sh = fmaT(D(-0.5), fmaT(g[S6_fo(m, i)], sB[S6_fo(b, j)][m], g[S6_fo(m, j)] * sB[S6_fo(b, i)][m]), sh);
-          D BD = advD[c] - twothird * trB * Dv[b][c];
+            for (int l = 0; l < 3; ++l) {
+              sh = fmaT(g[S6_fo(l, i)], sB[S6_fo(b, i)][l], sh);
+              BD = fmaT(B[i][l], Dv[b][S6_fo(l, i)], BD);
+              r = fmaT(B[b][l], Dv[l][c], r);
+            }
+            sh = sh + sh;
+            r = fmaT(D(2.0), BD, r);
+          } else {
 #pragma unroll
-          for (int l = 0; l < 3; ++l)
-            BD = fmaT(B[b][l], Dv[l][c], fmaT(B[j][l], Dv[b][S6_fo(l, i)], fmaT(B[i][l], Dv[b][S6_fo(l, j)], BD)));
-          D r = fmaT(-P.s3 * D(3.0), sh, BD);
-          r = fmaT(-al, fd1<D>(N, AXX + c, N.st[b], c1), r);
-          r = fmaT(-Av[b], fmaT(-third * g[c], trA, At[c]), r);
-          if (RED) r = fmaT(al * third * g[c], fmaT(D(-2.0), DuA[b], gdAt[b]), r);
+            for (int l = 0; l < 3; ++l) {
+              sh = fmaT(g[S6_fo(l, i)], sB[S6_fo(b, j)][l], fmaT(g[S6_fo(l, j)], sB[S6_fo(b, i)][l], sh));
+              r = fmaT(B[b][l], Dv[l][c], fmaT(B[j][l], Dv[b][S6_fo(l, i)], fmaT(B[i][l], Dv[b][S6_fo(l, j)], r)));
+            }
+          }
+          r = fmaT(s15, sh, r);
+          r = fmaT(-alc, d1u<D, D>(N, AXX + c, N.st[b]), r);
+          r = fmaT(g[c], cg, fmaT(-Av[b], At[c], r));
           sink(FD + 6 * b + c, fmaT(C.cko, ko_sum<D>(N, FD + 6 * b + c), r));
         }
     }
@@ -285,25 +310,24 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
 #pragma unroll
           for (int m = 0; m < 3; ++m)
             Cm[k][i][m] = fmaT(ig[S6_fo(0, m)], Gu[k][S6_fo(0, i)], fmaT(ig[S6_fo(1, m)], Gu[k][S6_fo(1, i)], ig[S6_fo(2, m)] * Gu[k][S6_fo(2, i)]));
-      D X[3][3];
+      // as in ccz4_rhs_point: G~_jkm + G~_kmj = 2 D_mjk, and G~_ikm symmetric in k and m
 #pragma unroll
-      for (int i = 0; i < 3; ++i)
+      for (int j = 0; j < 3; ++j) {
+        const D Cs[3] = {Cm[0][j][1] + Cm[1][j][0], Cm[0][j][2] + Cm[2][j][0], Cm[1][j][2] + Cm[2][j][1]};
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          D s = Cm[0][i][0] * Gd[j][S6_fo(0, 0)];
+        for (int i = 0; i <= j; ++i) {
+          D x = Cm[0][j][0] * Gd[i][0];
+          x = fmaT(Cm[1][j][1], Gd[i][3], x);
+          x = fmaT(Cm[2][j][2], Gd[i][5], x);
+          x = fmaT(Cs[0], Gd[i][1], x);
+          x = fmaT(Cs[1], Gd[i][2], x);
+          x = fmaT(Cs[2], Gd[i][4], x);
+          D y = Cm[0][i][0] * Dv[0][S6_fo(j, 0)];
 #pragma unroll
-          for (int q = 1; q < 9; ++q) s = fmaT(Cm[q / 3][i][q % 3], Gd[j][S6_fo(q / 3, q % 3)], s);
-          X[i][j] = s;
+          for (int q = 1; q < 9; ++q) y = fmaT(Cm[q / 3][i][q % 3], Dv[q % 3][S6_fo(j, q / 3)], y);
+          Q6[S6_fo(i, j)] = fmaT(D(2.0), y, x);
         }
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = i; j < 3; ++j) {
-          D q3 = X[i][j] + X[j][i];
-#pragma unroll
-          for (int q = 0; q < 9; ++q) q3 = fmaT(Cm[q / 3][i][q % 3], Gd[q / 3][S6_fo(q % 3, j)], q3);
-          Q6[S6_fo(i, j)] = q3;
-        }
+      }
     }
     // conformal-factor part and nabla nabla alpha
     const D PP = fmaT(Pv[0], fmaT(ig[0], Pv[0], fmaT(igw[1], Pv[1], igw[2] * Pv[2])),
@@ -322,11 +346,11 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
     const D iphPP = iph * PP;
     const D gco = (trcdph - dGP) - (iphPP + iphPP);
     // d_j Gamma-hat^k: g~_k(i d_j) Gamma-hat^k and the advection of Gamma-hat
-    D dGh[3][3];  // dGh[j][k] = d_j Gamma-hat^k
+    D dGh[3][3];  // dGh[j][k] = 12 dx d_j Gamma-hat^k
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
-      for (int j = 0; j < 3; ++j) dGh[j][k] = fd1<D>(N, GHX + k, N.st[j], c1);
+      for (int j = 0; j < 3; ++j) dGh[j][k] = d1u<D, D>(N, GHX + k, N.st[j]);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -334,17 +358,18 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
         const int c = S6_fo(i, j);
         D u = D(0.0);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) u = fmaT(g[S6_fo(k, i)], dGh[j][k], fmaT(g[S6_fo(k, j)], dGh[i][k], u));
+        for (int k = 0; k < 3; ++k) u = i == j ? fmaT(g[S6_fo(k, i)], dGh[i][k], u)
+                                               : fmaT(g[S6_fo(k, i)], dGh[j][k], fmaT(g[S6_fo(k, j)], dGh[i][k], u));
         D GD = Gh[0] * Dv[0][c];  // Gamma-hat^k D_kij = 1/2 Gamma-hat^k d_k g~_ij
         GD = fmaT(Gh[1], Dv[1][c], fmaT(Gh[2], Dv[2][c], GD));
         const D zt = fmaT(Z2[i], Pv[j], Z2[j] * Pv[i]);
         const D phiRZ = iph * (cdph[c] + fmaT(g[c], gco, zt));
-        RZ[c] = fmaT(D(0.5), u, Q6[c] + GD + phiRZ - lapg[c]);
+        RZ[c] = fmaT(i == j ? c1 : h1, u, Q6[c] + GD + phiRZ - lapg[c]);
         const D DDaD = fmaT(iph, fmaT(Pv[i], Av[j], fmaT(Pv[j], Av[i], -g[c] * PA)), ddA[c]);
         DDa[c] = fmaT(-Gu[0][c], Av[0], fmaT(-Gu[1][c], Av[1], fmaT(-Gu[2][c], Av[2], DDaD)));
       }
 #pragma unroll
-    for (int i = 0; i < 3; ++i) advGh[i] = fmaT(be[0], dGh[0][i], fmaT(be[1], dGh[1][i], be[2] * dGh[2][i]));
+    for (int i = 0; i < 3; ++i) advGh[i] = fmaT(bec[0], dGh[0][i], fmaT(bec[1], dGh[1][i], bec[2] * dGh[2][i]));
   }
   D trRZ = igw[0] * RZ[0], trDDa = igw[0] * DDa[0];
 #pragma unroll
@@ -377,9 +402,9 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
   }
   {
     const D trMx = fmaT(al, trRZ, -trDDa);
-    const D sg = fmaT(twothird * al, trA, -twothird * trB) - P.itau * (det - D(1.0));
+    const D sg = fmaT(twothird * al, trA, -trB23) - P.itau * (det - D(1.0));
     const D sA1 = -third * ph2 * trMx;
-    const D sA2 = fmaT(al, Kc, -twothird * trB);
+    const D sA2 = fmaT(al, Kc, -trB23);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -388,13 +413,20 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
         D lie = D(0.0), lieA = D(0.0), adv = D(0.0);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          lie = fmaT(g[S6_fo(k, i)], B[j][k], fmaT(g[S6_fo(k, j)], B[i][k], lie));
-          lieA = fmaT(At[S6_fo(k, i)], B[j][k], fmaT(At[S6_fo(k, j)], B[i][k], lieA));
           adv = fmaT(be[k], Dv[k][c], adv);
+          if (i == j) {
+            lie = fmaT(g[S6_fo(k, i)], B[i][k], lie);
+            lieA = fmaT(At[S6_fo(k, i)], B[i][k], lieA);
+          } else {
+            lie = fmaT(g[S6_fo(k, i)], B[j][k], fmaT(g[S6_fo(k, j)], B[i][k], lie));
+            lieA = fmaT(At[S6_fo(k, i)], B[j][k], fmaT(At[S6_fo(k, j)], B[i][k], lieA));
+          }
         }
-        sink(GXX + c, fmaT(C.cko, ko_sum<D>(N, GXX + c), fmaT(g[c], sg, fmaT(-al2, At[c], fmaT(D(2.0), adv, lie)))));
+        lie = i == j ? D(2.0) * (adv + lie) : fmaT(D(2.0), adv, lie);
+        lieA = i == j ? fmaT(D(2.0), lieA, advAt[c]) : advAt[c] + lieA;
+        sink(GXX + c, fmaT(C.cko, ko_sum<D>(N, GXX + c), fmaT(g[c], sg, fmaT(-al2, At[c], lie))));
         const D rA = fmaT(ph2 * al, RZ[c], fmaT(-ph2, DDa[c], fmaT(g[c], sA1, fmaT(At[c], sA2,
-                     fmaT(-al2, AgA[c], advAt[c] + lieA)))));
+                     fmaT(-al2, AgA[c], lieA)))));
         sink(AXX + c, fmaT(C.cko, ko_sum<D>(N, AXX + c), rA));
       }
   }
@@ -426,7 +458,7 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
   D dbK[3];  // d_t Gamma-hat^i - beta^k d_k Gamma-hat^i (before dissipation)
   {
     const D al43 = D(4.0 / 3.0) * al;
-    const D zc = D(0.5) * fmaT(-al43, Kt, fmaT(-al2, P.kappa1, P.k3x2 * twothird * trB));
+    const D zc = D(0.5) * fmaT(-al43, Kt, fmaT(-al2, P.kappa1, P.k3x2 * trB23));
     const D k3h = D(-0.5) * P.k3x2;
     D wv[3];
 #pragma unroll
@@ -434,22 +466,24 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
       wv[k] = fmaT(al2, dT[k], fmaT(-al43, dK[k], fmaT(P.s3, gdivB[k], -(Th + Th) * Av[k])));
       if (RED) wv[k] = fmaT(al2, fmaT(D(-2.0), DuA[k], gdAt[k]), wv[k]);
     }
+    D av[3], yv[3];  // -6 alpha P / phi - 2 A, contracted with A~^ij; -G~^k + k3h (Gamma-hat^k - G~^k), with B_k^i
+    const D al6p = D(-6.0) * al * iph;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      av[k] = fmaT(al6p, Pv[k], -(Av[k] + Av[k]));
+      yv[k] = fmaT(k3h, dGam[k], -Gc[k]);
+    }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       D GA = Gu[i][0] * Auw[0];
 #pragma unroll
       for (int c = 1; c < 6; ++c) GA = fmaT(Gu[i][c], Auw[c], GA);
-      const D AuA = fmaT(Au[S6_fo(i, 0)], Av[0], fmaT(Au[S6_fo(i, 1)], Av[1], Au[S6_fo(i, 2)] * Av[2]));
-      const D AuP = fmaT(Au[S6_fo(i, 0)], Pv[0], fmaT(Au[S6_fo(i, 1)], Pv[1], Au[S6_fo(i, 2)] * Pv[2])) * iph;
-      const D ZB = fmaT(dGam[0], B[0][i], fmaT(dGam[1], B[1][i], dGam[2] * B[2][i]));
       D t = fmaT(ig[S6_fo(i, 0)], wv[0], fmaT(ig[S6_fo(i, 1)], wv[1], fmaT(ig[S6_fo(i, 2)], wv[2], lapB[i])));
       t = fmaT(al2, GA, t);
-      t = fmaT(twothird * trB, Gc[i], t);
-      t = fmaT(D(-6.0) * al, AuP, t);
-      t = fmaT(D(-2.0), AuA, t);
+      t = fmaT(trB23, Gc[i], t);
+      t = fmaT(Au[S6_fo(i, 0)], av[0], fmaT(Au[S6_fo(i, 1)], av[1], fmaT(Au[S6_fo(i, 2)], av[2], t)));
       t = fmaT(zc, dGam[i], t);
-      t = fmaT(k3h, ZB, t);
-      dbK[i] = fmaT(-Gc[0], B[0][i], fmaT(-Gc[1], B[1][i], fmaT(-Gc[2], B[2][i], t)));
+      dbK[i] = fmaT(yv[0], B[0][i], fmaT(yv[1], B[1][i], fmaT(yv[2], B[2][i], t)));
       sink(GHX + i, fmaT(C.cko, ko_sum<D>(N, GHX + i), advGh[i] + dbK[i]));
     }
   }
@@ -462,13 +496,13 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
     for (int k = 0; k < 3; ++k)
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        const D db = fd1<D>(N, BBX + i, N.st[k], c1);  // d_k b^i
-        advb[i] = fmaT(be[k], db, advb[i]);
+        const D db = d1u<D, D>(N, BBX + i, N.st[k]);  // 12 dx d_k b^i
+        advb[i] = fmaT(bec[k], db, advb[i]);
         if (AUX) {
           // Eq. NR_foccz4_B^i_j: advection, f d_k b^i, B_k^l B_l^i, and the mu terms
           D r = D(0.0);
           if (driver) {
-            r = fmaT(P.f, db, advB[k][i]);
+            r = fmaT(P.f * c1, db, advB[k][i]);
 #pragma unroll
             for (int l = 0; l < 3; ++l) r = fmaT(B[k][l], B[l][i], r);
             if (RED) {
@@ -482,8 +516,8 @@ __device__ __forceinline__ void fo_rhs_point(const FoPhys &F, const NB &N, const
                 const D cp = ((k + 1) % 3 == j) ? curlP[o] : -curlP[o];
                 m1 = fmaT(ig[S6_fo(i, j)], cp, m1);
               }
-              const D amu = al * al * F.mu;
-              r = fmaT(-amu * iph, m1, fmaT(amu, m2[k][i], r));
+              const D amu = al * al * F.mu, amuc = amu * c1;
+              r = fmaT(-amu * iph, m1, fmaT(amuc, m2[k][i], r));
             }
           }
           sink(FB + 3 * k + i, fmaT(C.cko, ko_sum<D>(N, FB + 3 * k + i), r));

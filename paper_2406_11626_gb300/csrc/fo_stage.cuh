@@ -72,6 +72,8 @@ template <class D>
 __device__ __forceinline__ D fd1(const FoView &N, int v, int axis, const D &c1) {
   return __ldcs(N.d + (4 * v + axis) * N.np) * c1;
 }
+template <class D, class R>
+__device__ __forceinline__ D d1u(const FoView &N, int v, int axis) { return __ldcs(N.d + (4 * v + axis) * N.np); }
 template <class D>
 __device__ __forceinline__ D ko_sum(const FoView &N, int v) { return __ldcs(N.d + (4 * v + 3) * N.np); }
 
@@ -111,6 +113,11 @@ __device__ __forceinline__ void fo_ghost_cell(const GridView &g, const ccz4_para
 // thread per interior point, the 58-variable right-hand side (RED: with the
 // red terms; AUX: the auxiliary variables' equations too) from the derivative
 // buffer and the stage update of what it evolves.
+// The FP64 pipe holds it (ncu: 86 % busy; 3, 4 and 5 blocks within 1 %), so what
+// counts is its FP64 operations: first differences unscaled, the terms of the
+// D_kij equation with g~_ij under one coefficient, and the savings of
+// ccz4_rhs_point took one step at 54^3 from 4.59 to 4.11 ms, at 90^3 from 18.8
+// to 16.7 (reconstructed second order 13.1 to 12.0).
 template <int MODE, bool RED, bool AUX>
 __global__ void __launch_bounds__(128, CCZ4_FO_MIN_BLOCKS)
     fo_interior_kernel(GridView g, FoPhys F, StencilCoef<double> C, ccz4_params P, const double *__restrict__ der,
