@@ -177,6 +177,8 @@ __device__ __forceinline__ long long locate(const GridView &g, int x, int y, int
 // Host-side helpers implemented in ccz4_capi.cu.
 namespace ccz4 {
 void set_error(const char *fmt, ...);
+// Gives every page of a host array that a copy is about to write its memory (ccz4_capi.cu).
+void back_host_pages(void *p, size_t bytes);
 }
 
 struct ccz4_grid {

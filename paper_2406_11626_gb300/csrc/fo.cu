@@ -188,6 +188,8 @@ static ccz4_status fo_copy(ccz4_fo *f, int buf, double *U, double *G, bool to_de
       FO_TRY(cudaMemcpy2DAsync(d + v.n_points, dp, G, sizeof(double) * v.n_ghost, sizeof(double) * v.n_ghost, NVF,
                                cudaMemcpyHostToDevice, s));
   } else {
+    back_host_pages(U, sizeof(double) * (size_t)v.n_points * NVF);
+    if (v.n_ghost) back_host_pages(G, sizeof(double) * (size_t)v.n_ghost * NVF);
     FO_TRY(cudaMemcpy2DAsync(U, sizeof(double) * v.n_points, d, dp, sizeof(double) * v.n_points, NVF,
                              cudaMemcpyDeviceToHost, s));
     if (v.n_ghost)
