@@ -1,5 +1,5 @@
 // Host side of the C ABI declared in include/ccz4.h: grid allocation and
-// validation, host <-> device copies, and the orchestration of halo fill,
+// validation, host <-> device copies, and the orchestration of derivative pass,
 // right-hand side, RK4 stages and constraint monitors. Every compute step
 // runs in the kernels of halo.cu, rhs.cu and constraints.cu.
 #include <stdarg.h>
@@ -95,14 +95,16 @@ extern "C" ccz4_status ccz4_set_allocator(ccz4_alloc_fn alloc, ccz4_dealloc_fn d
   return CCZ4_OK;
 }
 
-// Whether FP64 stages with derivatives beside the algebra pay. A patch costs
-// 2.3 us of the two launches (1000 patches of 9^3: 9.4 ms a step); in one launch
-// every 152 patches cost a round of 270 us and the first patch's derivatives
-// another 0.6 of one: a grid pays from 1.3 times fewer rounds on (343 patches:
-// 3.3 ms a step in two launches, 3.7 in one; 1000: 9.4 and 8.3).
-static bool pair_pays(int patches) {
+// Whether FP64 stages with derivatives beside the algebra pay. In one launch
+// every 152 patches cost a round of 260 us a stage and the first patch's
+// derivatives another 0.6 of one; in two launches 152 patches cost 1.3 times as
+// much as a round (a step of 539 patches 4.97 ms in two launches, 4.73 in one; of
+// 1000 8.88 and 7.85; of 1728 15.0 and 13.0). Patches of a refined mesh have
+// longer derivatives (interpolated halo points): 1.17 times and 1.05 of a round
+// (432 patches 4.33 ms in two launches, 4.77 in one; 2240 19.8 and 18.9).
+static bool pair_pays(int patches, bool mesh) {
   const long long rounds = (patches + 151) / 152;
-  return 13LL * patches >= (10 * rounds + 6) * 152;
+  return mesh ? 117LL * patches >= (100 * rounds + 105) * 152 : 13LL * patches >= (10 * rounds + 6) * 152;
 }
 
 static size_t der_bytes(const GridView &v) { return sizeof(double) * (size_t)DER_SLOTS * (size_t)v.n_points; }
@@ -370,7 +372,7 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
   prepare_derive();
   prepare_constraints();
   if (v.p == 9) prepare_fused();
-  g->pair = v.p == 9 && pair_pays(v.n_patches) && prepare_pair(mesh != nullptr) == cudaSuccess;
+  g->pair = v.p == 9 && pair_pays(v.n_patches, mesh != nullptr) && prepare_pair(mesh != nullptr) == cudaSuccess;
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     set_error("grid set-up failed: %s", cudaGetErrorString(e));

@@ -57,8 +57,8 @@ def test_one_launch_equals_two(npv, bc):
 
 def test_one_launch_equals_two_on_a_mesh():
     from paper_2406_11626_gb300 import ccz4 as C
-    level, ijk = I.refined_mesh((5,) * 3, [((1,) * 3, (4,) * 3)])  # 854 patches
-    cfg = I.MeshConfig(name="", p=9, np=(5,) * 3, origin=(-2.4,) * 3, dx=0.11, bc="sommerfeld", params=PUNC, dt=0.003,
+    level, ijk = I.refined_mesh((7,) * 3, [((1,) * 3, (5, 4, 5))])  # 1639 patches: meshes below about 1100 keep two launches
+    cfg = I.MeshConfig(name="", p=9, np=(7,) * 3, origin=(-3.4,) * 3, dx=0.11, bc="sommerfeld", params=PUNC, dt=0.003,
                        steps=1, level=level, mesh_ijk=ijk)
     grid = C.Grid.from_config(cfg)
     _same(grid, C.make_params(**PUNC), cfg.dt, 8)
