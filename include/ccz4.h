@@ -452,7 +452,7 @@ ccz4_status ccz4_mesh_plan(const ccz4_mesh_desc *desc, long long *n_interp, int 
    points of every level are done; CCZ4_LAUNCH_FUSED, for grids of 9^3
    patches only (CCZ4_ERR_INVALID otherwise), runs each RK stage of
    ccz4_step and ccz4_step_graph as one cooperative launch sized to the
-   resident blocks: the halo fill of every patch, a grid-wide barrier, the
+   resident blocks: the derivatives of every patch, a grid-wide barrier, the
    interior points of all levels and the Sommerfeld ghost cells (the
    restriction of a mesh stays a launch of its own; ccz4_rk_stage,
    ccz4_fill_halos and the tuning shapes keep the separate kernels).

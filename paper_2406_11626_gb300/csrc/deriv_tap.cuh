@@ -1,4 +1,4 @@
-// Two-phase evaluation of the mixed-precision stage kernel.
+// Two-phase evaluation of the mixed-precision right-hand side from tiles (a host check of its templates).
 //
 // DerivTap stands in for the neighbourhood (Nbhd) of ccz4_rhs_point. In
 // the recording phase (TAP_RECORD) every stencil value the right-hand side

@@ -2,8 +2,8 @@
 // electric and magnetic parts of the Weyl tensor in their Z4 form
 // (Eqs. eq_NR_psi4_E_ij, eq_NR_psi4_B_ij, vacuum), contracted with mbar of
 // the Gram-Schmidt tetrad (Eqs. eq_NR_psi4_m_conj,
-// eq_NR_psi_code_implementation). A monitor, evaluated from the halo'd
-// tiles of the halo fill in FP64 with the stage kernel's stencils; Re and Im
+// eq_NR_psi_code_implementation). A monitor, evaluated in FP64 from the
+// derivative pass; Re and Im
 // go to fields 0 and 1 of a state-shaped buffer, where the particle tracers
 // can sample them (the paper attaches psi_4 to the solution vector and
 // interpolates it onto tracers arranged on a sphere).

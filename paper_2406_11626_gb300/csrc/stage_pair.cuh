@@ -18,8 +18,9 @@
 // 39.0, 384 + 256 (56, 152) 32.8, 512 + 256 (48, 144) 32.6, 512 + 384 (40, 112)
 // 31.7, two blocks of 256 + 128 (56, 128) 33.3, this split 31.6: the algebra
 // wants the 12 warps to cover its latency, the derivatives 12 to keep up. With
-// their conversions to FP64 in integers (CVT false) 30.4. What bounds it now:
-// the FP64 pipe (1320 operations a point are 28.1 ms).
+// their conversions to FP64 in integers (CVT false) 30.4, and 28.5 since the
+// algebra needs 100 operations a point less. What bounds it now: the FP64 pipe
+// (1215 operations a point are 23.1 ms) and the stalls that 12 warps leave open.
 //
 // Mixed precision keeps two launches: there the derivative pass is the longer
 // part and wants the whole SM (15.0 ms against 15.2 at best).
