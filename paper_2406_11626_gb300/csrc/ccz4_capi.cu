@@ -100,8 +100,9 @@ extern "C" ccz4_status ccz4_set_allocator(ccz4_alloc_fn alloc, ccz4_dealloc_fn d
 // derivatives another 0.6 of one; in two launches 152 patches cost 1.3 times as
 // much as a round (a step of 539 patches 4.97 ms in two launches, 4.73 in one; of
 // 1000 8.88 and 7.85; of 1728 15.0 and 13.0). Patches of a refined mesh have
-// longer derivatives (interpolated halo points): 1.17 times and 1.05 of a round
-// (432 patches 4.33 ms in two launches, 4.77 in one; 2240 19.8 and 18.9).
+// longer derivatives (interpolated halo points): 1.17 times and 1.05 of a round,
+// taken with equal parts (432 patches 4.33 ms in two launches, 4.77 in one; 2240
+// 19.8 and 18.9, 17.7 with the parts that meshes have now).
 static bool pair_pays(int patches, bool mesh) {
   const long long rounds = (patches + 151) / 152;
   return mesh ? 117LL * patches >= (100 * rounds + 105) * 152 : 13LL * patches >= (10 * rounds + 6) * 152;
