@@ -4,12 +4,12 @@
 namespace ccz4 {
 namespace {
 
-template <int SRC, bool MIXED, bool RAW, int SHAPE, int PF, int NF>
+template <int SRC, bool MIXED, int SHAPE, int PF, int NF>
 __global__ void __launch_bounds__(FILL_SHAPE_THREADS[SHAPE], (PF == 9 ? 1024 : 768) / FILL_SHAPE_THREADS[SHAPE])
     derive_kernel(GridView g, const double *__restrict__ src, double *tile, double *__restrict__ mix,
                   double *__restrict__ der, LevelScale ls, FieldList fl, bool tile_out) {
   extern __shared__ double smem[];
-  derive_patch<SRC, MIXED, RAW, FILL_SHAPE_THREADS[SHAPE], PF, NF>(g, src, tile, mix, der, ls, fl, blockIdx.x,
+  derive_patch<SRC, MIXED, FILL_SHAPE_THREADS[SHAPE], PF, NF>(g, src, tile, mix, der, ls, fl, blockIdx.x,
                                                                    blockIdx.y, gridDim.y, tile_out, smem);
 }
 
@@ -44,11 +44,11 @@ int field_groups(const GridView &g, const FieldList &fl) {
   return k < fl.n ? k : fl.n;
 }
 
-template <int SRC, bool MIXED, bool RAW, int SHAPE, int PF, int NF>
+template <int SRC, bool MIXED, int SHAPE, int PF, int NF>
 cudaError_t launch_one(const GridView &g, const double *src, double *tile, double *mix, double *der,
                        const FieldList &fl, bool tile_out, cudaStream_t s) {
   const dim3 grid(g.n_patches, field_groups(g, fl));
-  derive_kernel<SRC, MIXED, RAW, SHAPE, PF, NF><<<grid, FILL_SHAPE_THREADS[SHAPE], derive_smem_bytes(g.p, RAW), s>>>(
+  derive_kernel<SRC, MIXED, SHAPE, PF, NF><<<grid, FILL_SHAPE_THREADS[SHAPE], derive_smem_bytes(g.p), s>>>(
       g, src, tile, mix, der, level_scale(g), fl, tile_out);
   return cudaGetLastError();
 }
@@ -69,10 +69,9 @@ cudaError_t launch_fixed(const GridView &g, const double *src, double *tile, dou
 template <int SRC, bool MIXED, int SHAPE>
 cudaError_t launch_edge(const GridView &g, const double *src, double *tile, double *mix, double *der,
                         const FieldList &fl, bool tile_out, cudaStream_t s) {
-  if (g.p == 9) return launch_one<SRC, MIXED, false, SHAPE, 9, NV>(g, src, tile, mix, der, fl, tile_out, s);
+  if (g.p == 9) return launch_one<SRC, MIXED, SHAPE, 9, NV>(g, src, tile, mix, der, fl, tile_out, s);
   if constexpr (SHAPE == 0) {
-    if (derive_raw(g.p)) return launch_one<SRC, MIXED, true, 0, 0, NV>(g, src, tile, mix, der, fl, tile_out, s);
-    return launch_one<SRC, MIXED, false, 0, 0, NV>(g, src, tile, mix, der, fl, tile_out, s);
+    return launch_one<SRC, MIXED, 0, 0, NV>(g, src, tile, mix, der, fl, tile_out, s);
   } else {
     return launch_edge<SRC, MIXED, 0>(g, src, tile, mix, der, fl, tile_out, s);
   }
@@ -97,18 +96,10 @@ cudaError_t launch_shape(const GridView &g, const double *src, double *tile, dou
   return launch_edge<SRC, MIXED, 0>(g, src, tile, mix, der, fl, tile_out, s);
 }
 
-template <int SRC, bool MIXED, bool RAW, int SHAPE, int PF, int NF>
+template <int SRC, bool MIXED, int SHAPE, int PF, int NF>
 cudaError_t prepare_one(int p) {
-  return cudaFuncSetAttribute(derive_kernel<SRC, MIXED, RAW, SHAPE, PF, NF>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)derive_smem_bytes(p, RAW));
-}
-
-// The largest dynamic shared memory that any grid asks of the general instances.
-int largest_edge(bool raw) {
-  int q = 1;
-  for (int p = 1; p <= MAX_P; ++p)
-    if (derive_raw(p) == raw) q = p;
-  return q;
+  return cudaFuncSetAttribute(derive_kernel<SRC, MIXED, SHAPE, PF, NF>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)derive_smem_bytes(p));
 }
 
 template <int SRC, int PF>
@@ -119,7 +110,7 @@ cudaError_t prepare_fixed() {
 
 template <int SRC, bool MIXED>
 cudaError_t prepare_source() {
-  cudaError_t e = prepare_one<SRC, MIXED, false, 0, 9, NV>(9);
+  cudaError_t e = prepare_one<SRC, MIXED, 0, 9, NV>(9);
   if constexpr (SRC != FROM_TILE && !MIXED) {
     if (e == cudaSuccess) e = prepare_fixed<SRC, 9>();
     if (e == cudaSuccess)
@@ -128,11 +119,10 @@ cudaError_t prepare_source() {
     if (e == cudaSuccess) e = prepare_fixed<SRC, 12>();
     if (e == cudaSuccess) e = prepare_fixed<SRC, 6>();
   }
-  if (e == cudaSuccess) e = prepare_one<SRC, MIXED, false, 0, 0, NV>(largest_edge(false));
-  if (e == cudaSuccess) e = prepare_one<SRC, MIXED, true, 0, 0, NV>(largest_edge(true));
+  if (e == cudaSuccess) e = prepare_one<SRC, MIXED, 0, 0, NV>(MAX_P);
   if constexpr (SRC != FROM_TILE && MIXED) {
-    if (e == cudaSuccess) e = prepare_one<SRC, MIXED, false, 1, 9, NV>(9);
-    if (e == cudaSuccess) e = prepare_one<SRC, MIXED, false, 3, 9, NV>(9);
+    if (e == cudaSuccess) e = prepare_one<SRC, MIXED, 1, 9, NV>(9);
+    if (e == cudaSuccess) e = prepare_one<SRC, MIXED, 3, 9, NV>(9);
   }
   return e;
 }
@@ -146,9 +136,8 @@ cudaError_t prepare_derive() {
   if (e == cudaSuccess) e = prepare_source<FROM_MESH, true>();
   if (e == cudaSuccess) e = prepare_source<FROM_TILE, false>();
   if (e == cudaSuccess) e = prepare_source<FROM_TILE, true>();
-  if (e == cudaSuccess) e = prepare_one<FROM_LEVEL, false, false, 0, 9, 58>(9);
-  if (e == cudaSuccess) e = prepare_one<FROM_LEVEL, false, false, 0, 0, 58>(largest_edge(false));
-  if (e == cudaSuccess) e = prepare_one<FROM_LEVEL, false, true, 0, 0, 58>(largest_edge(true));
+  if (e == cudaSuccess) e = prepare_one<FROM_LEVEL, false, 0, 9, 58>(9);
+  if (e == cudaSuccess) e = prepare_one<FROM_LEVEL, false, 0, 0, 58>(MAX_P);
   return e;
 }
 
@@ -176,10 +165,8 @@ cudaError_t launch_derive(const GridView &g, const double *src, double *tile, do
 
 cudaError_t launch_derive_fo(const GridView &g, const double *src, double *der, const FieldList &fl, cudaStream_t s) {
   if (g.n_patches == 0 || fl.n == 0) return cudaSuccess;
-  if (g.p == 9) return launch_one<FROM_LEVEL, false, false, 0, 9, 58>(g, src, nullptr, nullptr, der, fl, false, s);
-  if (derive_raw(g.p))
-    return launch_one<FROM_LEVEL, false, true, 0, 0, 58>(g, src, nullptr, nullptr, der, fl, false, s);
-  return launch_one<FROM_LEVEL, false, false, 0, 0, 58>(g, src, nullptr, nullptr, der, fl, false, s);
+  if (g.p == 9) return launch_one<FROM_LEVEL, false, 0, 9, 58>(g, src, nullptr, nullptr, der, fl, false, s);
+  return launch_one<FROM_LEVEL, false, 0, 0, 58>(g, src, nullptr, nullptr, der, fl, false, s);
 }
 
 }  // namespace ccz4

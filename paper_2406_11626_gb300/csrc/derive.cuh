@@ -165,27 +165,6 @@ __device__ __forceinline__ void point_sums(const float2 *t, const unsigned *, in
   out[3] = ko;
 }
 
-// The same from raw FP64 values, for patch edges whose tile leaves no room for the exponents.
-template <bool SECOND>
-__device__ __forceinline__ void point_sums_raw(const double *t, int T, double *out) {
-  const int st[3] = {1, T, T * T};
-  double p[3][3], m[3][3], d1[3], d2[3], ko;
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      p[k][j] = t[(j + 1) * st[k]];
-      m[k][j] = t[-(j + 1) * st[k]];
-    }
-  fx_axes<true, SECOND>(t[0], p, m, d1, d2, ko);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    out[k] = d1[k];
-    if (SECOND) out[4 + k] = d2[k];
-  }
-  out[3] = ko;
-}
-
 // Where a patch's tile comes from: gathered through the neighbour lookup of a
 // single level, or through a refined mesh's table, or read from the tile
 // buffer that a halo fill has written.
@@ -193,28 +172,26 @@ enum { FROM_LEVEL = 0, FROM_MESH = 1, FROM_TILE = 2 };
 
 // Doubles that the widened region of the mixed derivatives takes, and the
 // place of the exponents with it: a field's mixed derivatives are done before
-// its exponents are written, so the two share their place (unless RAW, which
-// keeps no exponents).
+// its exponents are written, so the two share their place.
 __host__ __device__ constexpr int derive_ext(int p) {
   return fill_wide(p) ? (p + 4) * (p + 4) * p : (p + 4) * p * p;
 }
-__host__ __device__ constexpr int derive_shared(int p, bool raw) {
-  const int T3 = (p + 2 * HALO) * (p + 2 * HALO) * (p + 2 * HALO), e = derive_ext(p), x = raw ? 0 : (T3 + 1) / 2;
+__host__ __device__ constexpr int derive_shared(int p) {
+  const int T3 = (p + 2 * HALO) * (p + 2 * HALO) * (p + 2 * HALO), e = derive_ext(p), x = (T3 + 1) / 2;
   return e > x ? e : x;
 }
 // Shared memory of a block: the tile's words, the shared place above and the
 // source table (not FROM_TILE). 54 KB at a patch edge of 9: four blocks per SM.
-inline size_t derive_smem_bytes(int p, bool raw) {
+inline size_t derive_smem_bytes(int p) {
   const size_t T = (size_t)p + 2 * HALO, T3 = T * T * T;
-  return T3 * (8 + 4) + 8 * (size_t)derive_shared(p, raw);
+  return T3 * (8 + 4) + 8 * (size_t)derive_shared(p);
 }
-inline bool derive_raw(int p) { return derive_smem_bytes(p, false) > FILL_SMEM_LIMIT; }
 
 // The fields group, group + groups, ... of the list, of patch n, by one block
 // of THREADS threads. NF: fields of the formulation (25, or 58 without second
 // derivatives). tile: the tile buffer; interpolated halo points of a mesh pass
 // through it, tile_out (FP64) has the whole tile written to it, FROM_TILE reads it.
-template <int SRC, bool MIXED, bool RAW, int THREADS, int PF, int NF>
+template <int SRC, bool MIXED, int THREADS, int PF, int NF>
 __device__ __forceinline__ void derive_patch(const GridView &g, const double *__restrict__ src, double *tile,
                                              double *__restrict__ mix, double *__restrict__ der, const LevelScale &ls,
                                              const FieldList &fl, int n, int group, int groups, bool tile_out,
@@ -227,7 +204,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
   double *ts = smem;
   double *ext = ts + T3;
   unsigned *ex = reinterpret_cast<unsigned *>(ext);
-  int *idx = reinterpret_cast<int *>(ext + derive_shared(p, RAW));
+  int *idx = reinterpret_cast<int *>(ext + derive_shared(p));
   constexpr bool MESH = SRC == FROM_MESH;
   int e0 = 0, e1 = 0, xb0 = 0, nx = 0, yb0 = 0, ny = 0;
   if (MESH) {
@@ -325,7 +302,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
         if (SRC != FROM_TILE && tile_out) __stcs(tv + t, w);
         if (pair) {
           ts[t] = SRC == FROM_TILE ? w : split_pair(w);
-        } else if (!RAW && (!second || SRC == FROM_TILE)) {
+        } else if (!second || SRC == FROM_TILE) {
           unsigned e;
           reinterpret_cast<long long *>(ts)[t] = fx_word(w, e);
           ex[t] = e;
@@ -367,7 +344,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
           mixed_out(ext, e, pe, cmix, cmixf, pair, mix, np, pbase, slot + 2, q);
         }
       }
-      if (!RAW && sums && !pair) {
+      if (sums && !pair) {
         __syncthreads();  // the exponents take the widened region's place
         for (int t = threadIdx.x; t < T3; t += THREADS) {
           unsigned e;
@@ -389,7 +366,6 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
         O o[7];
         if constexpr (std::is_same<O, float>::value)
           point_sums<SECOND>(reinterpret_cast<const float2 *>(ts) + c0, ex, T, o);
-        else if constexpr (RAW) point_sums_raw<SECOND>(ts + c0, T, o);
         else point_sums<SECOND>(reinterpret_cast<const long long *>(ts) + c0, ex + c0, T, o);
         O *a, *b;
         if constexpr (std::is_same<O, float>::value) {

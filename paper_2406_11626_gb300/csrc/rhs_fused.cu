@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, (StageBlocks<R, 0>::value))
   for (int n = blockIdx.x; n < g.n_patches; n += gridDim.x) {
     constexpr int SRC = MESH ? FROM_MESH : FROM_LEVEL;
     if constexpr (std::is_same<R, float>::value)
-      derive_patch<SRC, true, false, FUSED_THREADS, FUSED_PF, NV>(g, in, tile, mix, der, ls, fl, n, 0, 1, false, smem);
+      derive_patch<SRC, true, FUSED_THREADS, FUSED_PF, NV>(g, in, tile, mix, der, ls, fl, n, 0, 1, false, smem);
     else
       derive_edge<SRC, FUSED_THREADS, FUSED_PF, true>(g, in, tile, mix, der, ls, fl, n, 0, 1, smem, threadIdx.x, 0);
     __syncthreads();  // the next patch's source table overwrites this one's shared memory
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, (StageBlocks<R, 0>::value))
 
 template <class R>
 size_t fused_smem_bytes() {
-  return std::is_same<R, float>::value ? derive_smem_bytes(FUSED_PF, false) : edge_smem_bytes(FUSED_PF);
+  return std::is_same<R, float>::value ? derive_smem_bytes(FUSED_PF) : edge_smem_bytes(FUSED_PF);
 }
 
 template <int MODE, class R, bool MESH>
