@@ -26,113 +26,12 @@ namespace ccz4 {
 
 namespace {
 
-// The word and the exponent under which a tile value waits in shared memory:
-// its mantissa as a signed integer of 57 bits and its biased exponent; the
-// value's own bits where the exponent is FX_TOP or more. (Zero and subnormal
-// values keep exponent 0: beside any value of exponent FX_FLOOR or more they
-// are shifted out.)
-__device__ __forceinline__ long long fx_word(double u, unsigned &e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(u);
-  e = (unsigned)(b >> 52) & 0x7FFu;
-  const unsigned long long m = ((b << 4) & 0x00FFFFFFFFFFFFF0ull) | 0x0100000000000000ull;
-  const unsigned long long n = (unsigned long long)((long long)b >> 63);
-  return e >= FX_TOP ? (long long)b : (long long)((m ^ n) - n);
-}
-__device__ __forceinline__ double fx_value(long long w, unsigned e) {
-  if (e >= FX_TOP) return __longlong_as_double(w);
-  if (e == 0) return 0.0;
-  const unsigned long long n = (unsigned long long)(w >> 63), a = ((unsigned long long)w ^ n) - n;
-  return __longlong_as_double((long long)((n & 0x8000000000000000ull) | ((unsigned long long)e << 52) |
-                                          ((a >> 4) & 0x000FFFFFFFFFFFFFull)));
-}
-__device__ __forceinline__ long long fx_sar(long long x, unsigned s) {
-  long long r;
-  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));  // all sign bits beyond 63
-  return r;
-}
-
-// A zero that the compiler cannot move or foresee: what depends on it is not evaluated ahead of the
-// branch it stands in.
-__device__ __forceinline__ int here_zero() {
-  int z;
-  asm volatile("mov.u32 %0, 0;" : "=r"(z));
-  return z;
-}
-
-// The stencil sums of one point whose largest neighbour lies outside [FX_FLOOR, FX_TOP), in FP64.
-// Inline: a call's registers would be its callee's choice.
-template <bool SECOND, class E>
-__device__ __forceinline__ void point_sums_fp64(const long long *w, const E *ex, int T, double *out) {
-  const int z = here_zero();
-  w += z;
-  ex += z;
-  const int st[3] = {1, T, T * T};
-  const double c = fx_value(w[0], ex[0]);
-  double s[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    double p[3], m[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int o = (j + 1) * st[k];
-      p[j] = fx_value(w[o], ex[o]);
-      m[j] = fx_value(w[-o], ex[-o]);
-      s[j] += p[j] + m[j];
-    }
-    out[k] = fma(8.0, p[0] - m[0], -(p[1] - m[1]));
-    if (SECOND) out[4 + k] = fma(-30.0, c, fma(16.0, p[0] + m[0], -(p[1] + m[1])));
-  }
-  out[3] = fma(-60.0, c, fma(15.0, s[0], fma(-6.0, s[1], s[2])));
-}
-
-template <bool CVT>
-__device__ __forceinline__ double fx_return(long long v, unsigned unit) {
-  if constexpr (CVT) return fx_out_cvt<2>(v, unit);
-  else return fx_out<2, true>(v, unit);
-}
-
-// The stencil sums of the point at w, ex: out[0..2] first derivatives, out[3]
-// dissipation, out[4..6] pure second derivatives. CVT: the second sums return by
-// the conversion instruction, or else in integers with the same rounding (for a
-// kernel whose other warps hold the FP64 pipe).
+// The stencil sums of the point at w, ex in a tile of edge T: out[0..2] first
+// derivatives, out[3] dissipation, out[4..6] pure second derivatives. CVT: as fx_return.
 template <bool SECOND, bool CVT = true, class E>
-__device__ __forceinline__ void point_sums(const long long *w, const E *ex, int T, double *out) {
+__device__ __forceinline__ void point_sums(const int64_t *w, const E *ex, int T, double *out) {
   const int st[3] = {1, T, T * T};
-  const unsigned e0 = ex[0];
-  unsigned ep[3][3], em[3][3], e = e0;
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      ep[k][j] = ex[(j + 1) * st[k]];
-      em[k][j] = ex[-(j + 1) * st[k]];
-      e = max(e, max(ep[k][j], em[k][j]));
-    }
-  if (e - FX_FLOOR >= FX_TOP - FX_FLOOR) {
-    if (e == 0u) {
-#pragma unroll
-      for (int q = 0; q < (SECOND ? 7 : 4); ++q) out[q] = 0.0;
-    } else {
-      point_sums_fp64<SECOND>(w, ex, T, out);
-    }
-    return;
-  }
-  const unsigned u = (e << 21) | FX_LOW;
-  const long long q = fx_sar(w[0], e - e0) >> 2;
-  long long s1 = 0, s2 = 0, s3 = 0;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int s = st[k];
-    const long long p1 = fx_sar(w[s], e - ep[k][0]), m1 = fx_sar(w[-s], e - em[k][0]);
-    const long long p2 = fx_sar(w[2 * s], e - ep[k][1]), m2 = fx_sar(w[-2 * s], e - em[k][1]);
-    const long long t1 = p1 + m1, t2 = p2 + m2;
-    out[k] = fx_out<4>((p1 - m1) * 8 - (p2 - m2), u);
-    if (SECOND) out[4 + k] = fx_return<CVT>(((t1 >> 2) - 2 * q) * 16 - (t2 >> 2) + 2 * q, u);
-    s1 += t1;
-    s2 += t2;
-    s3 += fx_sar(w[3 * s], e - ep[k][2]) + fx_sar(w[-3 * s], e - em[k][2]);
-  }
-  out[3] = fx_return<CVT>((((s1 >> 2) - 4 * q) * 5 - 2 * (s2 >> 2)) * 3 + (s3 >> 2), u);
+  fx_point<SECOND, CVT>(w, ex, st, out);
 }
 
 // The same in FP32 from split pairs (mixed precision), whose FP32 pipe is
@@ -304,7 +203,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
           ts[t] = SRC == FROM_TILE ? w : split_pair(w);
         } else if (!second || SRC == FROM_TILE) {
           unsigned e;
-          reinterpret_cast<long long *>(ts)[t] = fx_word(w, e);
+          reinterpret_cast<int64_t *>(ts)[t] = fx_word(w, e);
           ex[t] = e;
         } else {
           ts[t] = w;
@@ -348,7 +247,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
         __syncthreads();  // the exponents take the widened region's place
         for (int t = threadIdx.x; t < T3; t += THREADS) {
           unsigned e;
-          reinterpret_cast<long long *>(ts)[t] = fx_word(ts[t], e);
+          reinterpret_cast<int64_t *>(ts)[t] = fx_word(ts[t], e);
           ex[t] = e;
         }
         __syncthreads();
@@ -366,7 +265,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
         O o[7];
         if constexpr (std::is_same<O, float>::value)
           point_sums<SECOND>(reinterpret_cast<const float2 *>(ts) + c0, ex, T, o);
-        else point_sums<SECOND>(reinterpret_cast<const long long *>(ts) + c0, ex + c0, T, o);
+        else point_sums<SECOND>(reinterpret_cast<const int64_t *>(ts) + c0, ex + c0, T, o);
         O *a, *b;
         if constexpr (std::is_same<O, float>::value) {
           a = fd + q;

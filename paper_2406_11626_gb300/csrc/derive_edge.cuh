@@ -24,31 +24,7 @@ namespace ccz4 {
 namespace {
 
 // First-derivative sum along stride s of FP64 values in shared memory.
-__device__ __forceinline__ double first_of(const double *e, int s) {
-  const double a1 = e[s], b1 = e[-s], a2 = e[2 * s], b2 = e[-2 * s];
-  const unsigned u = fx_unit(fx_max(fx_max(fx_key(a1), fx_key(b1)), fx_max(fx_key(a2), fx_key(b2))));
-  if (fx_outside(u)) {
-    e += here_zero();
-    return fma(8.0, e[s] - e[-s], -(e[2 * s] - e[-2 * s]));
-  }
-  const int64_t d1 = fx_in(a1, u) - fx_in(b1, u), d2 = fx_in(a2, u) - fx_in(b2, u);
-  return fx_out<4>(d1 * 8 - d2, u);
-}
-
-// First-derivative sum along stride s of words alone (the widened rim), as point_sums takes it.
-__device__ __forceinline__ double first_sum_fp64(const long long *w, const unsigned short *ex, int s) {
-  const int z = here_zero();
-  w += z;
-  ex += z;
-  return fma(8.0, fx_value(w[s], ex[s]) - fx_value(w[-s], ex[-s]),
-             -(fx_value(w[2 * s], ex[2 * s]) - fx_value(w[-2 * s], ex[-2 * s])));
-}
-__device__ __forceinline__ double first_sum(const long long *w, const unsigned short *ex, int s) {
-  const unsigned a = ex[s], b = ex[-s], c = ex[2 * s], d = ex[-2 * s], e = max(max(a, b), max(c, d));
-  if (e - FX_FLOOR >= FX_TOP - FX_FLOOR) return e == 0u ? 0.0 : first_sum_fp64(w, ex, s);
-  const long long p = fx_sar(w[s], e - a) - fx_sar(w[-s], e - b), m = fx_sar(w[2 * s], e - c) - fx_sar(w[-2 * s], e - d);
-  return fx_out<4>(p * 8 - m, (e << 21) | FX_LOW);
-}
+__device__ __forceinline__ double first_of(const double *e, int s) { return fx_first(e[s], e[-s], e[2 * s], e[-2 * s]); }
 
 // A barrier of the THREADS threads (whole warps) that share barrier `bar`.
 template <int THREADS>
@@ -150,7 +126,7 @@ __device__ __forceinline__ void derive_edge(const GridView &g, const double *__r
   constexpr int BATCH = (T3 + THREADS - 1) / THREADS <= 10 ? (T3 + THREADS - 1) / THREADS : 7;
   constexpr int ROUNDS = (P3 + THREADS - 1) / THREADS;
   constexpr bool MESH = SRC == FROM_MESH;
-  long long *tw = reinterpret_cast<long long *>(smem);
+  int64_t *tw = reinterpret_cast<int64_t *>(smem);
   double *Ez = smem + T3, *Ey = Ez + EDGE_EZ(PF);
   int *idx = reinterpret_cast<int *>(ONE ? Ez : Ey + EDGE_EY(PF));
   unsigned short *ex = reinterpret_cast<unsigned short *>(ONE ? reinterpret_cast<int *>(Ey + EDGE_EY(PF)) : idx + T3);
@@ -237,7 +213,7 @@ __device__ __forceinline__ void derive_edge(const GridView &g, const double *__r
           const int far = a < 2 ? a - 2 : PF + a - 2;  // -2, -1, PF, PF + 1
           const int x = in_y ? b : far, y = in_y ? far : b;
           const int c = (z + HALO) * T2 + (y + HALO) * T + (x + HALO);
-          const double f = first_sum(tw + c, ex + c, along_z ? T2 : T);
+          const double f = fx_first_sum(tw + c, ex + c, along_z ? T2 : T);
           if (along_z) Ez[(z * PE + (y + 2)) * PE + (x + 2)] = f;
           else Ey[(z * PF + y) * PE + (x + 2)] = f;
         }
