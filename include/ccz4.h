@@ -135,14 +135,19 @@ typedef struct ccz4_grid ccz4_grid;
 
 /* Creates a grid on the current device and allocates its buffers (Sec.
    "Spatial Discretisation": p^3 patches with K = 3 halo layers). The
-   descriptor and its ijk array are copied. Buffers start zeroed. On error
-   *out is set to NULL. */
+   descriptor and its ijk array are copied. Buffers start zeroed. Besides
+   the CCZ4_BUF_* buffers a grid holds a derivative buffer of 133 doubles a
+   point for all its points, for a part of them on a grid of more than 2^23
+   points (or than the environment variable CCZ4_DERIVE_POINTS says) and
+   where memory is short; results do not depend on it. On error *out is set
+   to NULL. */
 ccz4_status ccz4_alloc_patches(const ccz4_grid_desc *desc, ccz4_grid **out);
 
 /* Device-memory allocator for the large buffers of grids created from now
-   on (the CCZ4_BUF_* state buffers, the halo tiles and the mixed
-   derivatives of ccz4_alloc_patches and ccz4_alloc_mesh), so that a host
-   framework's caching allocator can supply them: alloc(ctx, bytes, stream)
+   on (the CCZ4_BUF_* state buffers, the halo tiles, the mixed derivatives
+   and the derivative buffer of ccz4_alloc_patches and ccz4_alloc_mesh), so
+   that a host framework's caching allocator can supply them (it may be
+   asked again for less after it refused the derivative buffer): alloc(ctx, bytes, stream)
    returns a device pointer (aligned to 256 bytes, like cudaMalloc) or NULL
    on failure; dealloc(ctx, ptr, bytes, stream) releases one. stream is
    NULL (the legacy default stream): the library synchronises the device
@@ -488,8 +493,9 @@ ccz4_status ccz4_set_launch(ccz4_grid *g, int mode);
    each [58][field stride] in the grid's layout; the stages use them as
    ccz4_stage_buffers says.
    ccz4_fo_alloc: CCZ4_ERR_INVALID for a refined mesh or an unknown
-   variant; CCZ4_ERR_NOMEM if the device memory runs out (about
-   58 x 8 bytes x (6 state buffers + 4.6 tile copies) per point).
+   variant; CCZ4_ERR_NOMEM if the device memory runs out (58 x 8 bytes x
+   (6 state buffers + 4 derivative sums) per point; the sums of a part of
+   the points as for a grid).
    ccz4_fo_upload / ccz4_fo_download: host U [58][n_points] (the grid's
    point order) and G [58][n_ghost]; synchronous.
    ccz4_fo_rhs: the right-hand side of all 58 (with the red terms only in

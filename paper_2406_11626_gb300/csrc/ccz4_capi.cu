@@ -108,7 +108,69 @@ static bool pair_pays(int patches, bool mesh) {
   return mesh ? 117LL * patches >= (100 * rounds + 105) * 152 : 13LL * patches >= (10 * rounds + 6) * 152;
 }
 
-static size_t der_bytes(const GridView &v) { return sizeof(double) * (size_t)DER_SLOTS * (size_t)v.n_points; }
+// Points of a derivative buffer: WINDOW_CAP at most (8.9 GB of 133 doubles a point, beside the 299 doubles that
+// a point of a grid of 9^3 patches takes otherwise), less where memory is short, so that the buffer does not bound
+// the size of a grid. A larger grid takes its derivatives and what reads them in equal windows, each of which
+// costs a launch's ramp and last wave twice a stage: a mixed step of 144^3 15.0 ms in one window, 15.7 in two,
+// 16.3 in three; of three levels of 5.5 M points 28.6, 29.2 in two, 30.4 in four. FP64 stages in one launch need
+// two patches a block of the buffer and no windows. CCZ4_DERIVE_POINTS sets another bound.
+constexpr long long WINDOW_CAP = 1ll << 23;
+
+// Windows of k * unit patches, unit the least number whose points fill whole blocks of the monitors' sums.
+static int window_unit(const GridView &v) {
+  const int p3 = v.p * v.p * v.p;
+  int u = 256;
+  for (int q = p3; u > 1 && q % 2 == 0; q /= 2) u /= 2;
+  return u;
+}
+int ccz4::smaller_window(const GridView &v, int patches) {
+  const int unit = window_unit(v), w = (patches / 2 + unit - 1) / unit * unit;
+  return w < patches ? w : 0;
+}
+
+int ccz4::fitting_window(const GridView &v, int slots) {
+  const char *e = getenv("CCZ4_DERIVE_POINTS");
+  const long long set = e ? atoll(e) : 0, cap = set > 0 ? set : WINDOW_CAP;
+  int w = v.n_patches;
+  if (v.n_points > cap) {
+    const long long unit = window_unit(v), windows = (v.n_points + cap - 1) / cap;
+    const long long even = ((v.n_patches + windows - 1) / windows + unit - 1) / unit * unit;
+    if (even < w) w = (int)even;
+  }
+  size_t free_b = 0, total_b = 0;
+  if (slots == 0 || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return w;
+  const size_t patch = sizeof(double) * (size_t)slots * (size_t)(v.p * v.p * v.p);
+  while (patch * (size_t)w > free_b / 2) {
+    const int smaller = smaller_window(v, w);
+    if (smaller == 0) break;
+    w = smaller;
+  }
+  return w;
+}
+
+// Whether the buffer holds the two patches of each block that the one-launch stages keep (stage_pair.cuh).
+static bool pair_fits(const GridView &v) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return v.wcap >= v.n_patches || v.wcap >= 2 * sms;
+}
+
+static size_t der_bytes(const GridView &v) {
+  return sizeof(double) * (size_t)DER_SLOTS * (size_t)v.wcap * (size_t)(v.p * v.p * v.p);
+}
+
+// f on the view of each window of the grid.
+template <class F>
+static ccz4_status each_window(const ccz4_grid *g, F f) {
+  GridView v = g->v;
+  for (v.w0 = 0; v.w0 < g->v.n_patches; v.w0 += v.wcap) {
+    v.wn = g->v.n_patches - v.w0 < v.wcap ? g->v.n_patches - v.w0 : v.wcap;
+    const ccz4_status st = f(v);
+    if (st != CCZ4_OK) return st;
+  }
+  return CCZ4_OK;
+}
 
 // A large buffer of a grid from its allocator; NULL with the error message set on failure.
 static double *large_alloc(ccz4_grid *g, size_t bytes) {
@@ -324,10 +386,6 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
     }
     cudaMemset(g->buf[b], 0, bytes);
   }
-  if (v.n_points > 0 && !(g->der = large_alloc(g, der_bytes(v)))) {
-    free_all(g);
-    return CCZ4_ERR_NOMEM;
-  }
   g->red_blocks = constraint_blocks(v.n_points);
   bool ok = cudaMalloc(&g->d_ijk, sizeof(int) * 3 * (size_t)d->n_patches) == cudaSuccess &&
             cudaMalloc(&g->d_owner, sizeof(int) * (size_t)slots) == cudaSuccess &&
@@ -369,11 +427,19 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
       return CCZ4_ERR_NOMEM;
     }
   }
+  v.wcap = fitting_window(v, g->alloc ? 0 : DER_SLOTS);  // (an allocator knows its memory)
+  while (v.n_points > 0 && !(g->der = large_alloc(g, der_bytes(v)))) {
+    v.wcap = smaller_window(v, v.wcap);
+    if (v.wcap > 0) continue;
+    free_all(g);
+    return CCZ4_ERR_NOMEM;
+  }
+  g_err[0] = 0;  // of a larger buffer
   prepare_fill_halos(v.p);
   prepare_derive();
   prepare_constraints();
   if (v.p == 9) prepare_fused();
-  g->pair = v.p == 9 && pair_pays(v.n_patches, mesh != nullptr) && prepare_pair(mesh != nullptr) == cudaSuccess;
+  g->pair = v.p == 9 && pair_fits(v) && pair_pays(v.n_patches, mesh != nullptr) && prepare_pair(mesh != nullptr) == cudaSuccess;
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     set_error("grid set-up failed: %s", cudaGetErrorString(e));
@@ -595,9 +661,9 @@ static const double *ini_ptr(ccz4_grid *g) {
   return g->buf[CCZ4_BUF_INI] ? g->buf[CCZ4_BUF_INI] : g->buf[CCZ4_BUF_U];
 }
 
-// The derivative pass of a state buffer as the algebra for P needs it.
-static cudaError_t derivatives(ccz4_grid *g, const ccz4_params *P, int buf, cudaStream_t s) {
-  return launch_derive(g->v, g->buf[buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der, all_fields(),
+// The derivative pass over a window of a state buffer as the algebra for P needs it.
+static cudaError_t derivatives(ccz4_grid *g, const GridView &w, const ccz4_params *P, int buf, cudaStream_t s) {
+  return launch_derive(w, g->buf[buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der, all_fields(),
                        P->precision == CCZ4_PREC_MIXED, false, false, s);
 }
 
@@ -609,9 +675,11 @@ extern "C" ccz4_status ccz4_rhs(ccz4_grid *g, const ccz4_params *P, int in_buf, 
     return CCZ4_ERR_INVALID;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  CUDA_TRY(derivatives(g, P, in_buf, s));
-  CUDA_TRY(launch_rhs(g->v, *P, g->der, g->buf[CCZ4_BUF_MIX], g->buf[in_buf], ini_ptr(g), g->buf[out_buf], s));
-  return CCZ4_OK;
+  return each_window(g, [&](const GridView &w) {
+    CUDA_TRY(derivatives(g, w, P, in_buf, s));
+    CUDA_TRY(launch_rhs(w, *P, g->der, g->buf[CCZ4_BUF_MIX], g->buf[in_buf], ini_ptr(g), g->buf[out_buf], s));
+    return CCZ4_OK;
+  });
 }
 
 static const int kStageIn[4] = {CCZ4_BUF_U, CCZ4_BUF_Y0, CCZ4_BUF_Y1, CCZ4_BUF_Y0};
@@ -624,13 +692,22 @@ static ccz4_status restrict_levels(ccz4_grid *g, double *U, cudaStream_t s) {
   return CCZ4_OK;
 }
 
-// One RK4 stage from its derivatives; stage 3 ends the step (enforcement in
-// the algebra kernel, then the restriction on a mesh).
-static ccz4_status stage_kernel(ccz4_grid *g, const ccz4_params *P, int stage, double dt, cudaStream_t s) {
-  CUDA_TRY(launch_rk_stage(g->v, *P, stage, dt, g->der, g->buf[CCZ4_BUF_MIX], g->buf[kStageIn[stage]], ini_ptr(g),
-                           g->buf[CCZ4_BUF_U], g->buf[CCZ4_BUF_ACC], g->buf[kStageOut[stage]], s));
-  if (stage == 3 && g->v.n_levels > 1) return restrict_levels(g, g->buf[kStageOut[stage]], s);
-  return CCZ4_OK;
+// One RK4 stage, its derivatives taken from the tiles or from the stage's input, and its algebra; stage 3 ends
+// the step (enforcement in the algebra kernel, then the restriction on a mesh).
+static ccz4_status two_launch_stage(ccz4_grid *g, const ccz4_params *P, int stage, double dt, bool from_tile,
+                                    cudaStream_t s) {
+  const ccz4_status st = each_window(g, [&](const GridView &w) {
+    if (from_tile)
+      CUDA_TRY(launch_derive(w, g->buf[kStageIn[stage]], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der,
+                             all_fields(), P->precision == CCZ4_PREC_MIXED, true, false, s));
+    else
+      CUDA_TRY(derivatives(g, w, P, kStageIn[stage], s));
+    CUDA_TRY(launch_rk_stage(w, *P, stage, dt, g->der, g->buf[CCZ4_BUF_MIX], g->buf[kStageIn[stage]], ini_ptr(g),
+                             g->buf[CCZ4_BUF_U], g->buf[CCZ4_BUF_ACC], g->buf[kStageOut[stage]], s));
+    return CCZ4_OK;
+  });
+  if (st == CCZ4_OK && stage == 3 && g->v.n_levels > 1) return restrict_levels(g, g->buf[kStageOut[stage]], s);
+  return st;
 }
 
 // One RK4 stage of a step: the derivative pass and the algebra kernel as two
@@ -639,10 +716,7 @@ static ccz4_status stage_kernel(ccz4_grid *g, const ccz4_params *P, int stage, d
 // cooperative launch; the restriction after stage 3 stays a launch of its own.
 static ccz4_status step_stage(ccz4_grid *g, const ccz4_params *P, int stage, double dt, cudaStream_t s) {
   const bool pair = g->pair && !g->fused && !g->v.queue && g->v.stage_shape == 0 && P->precision != CCZ4_PREC_MIXED;
-  if (!g->fused && !pair) {
-    CUDA_TRY(derivatives(g, P, kStageIn[stage], s));
-    return stage_kernel(g, P, stage, dt, s);
-  }
+  if (!g->fused && !pair) return two_launch_stage(g, P, stage, dt, false, s);
   const auto launch = pair ? launch_pair_stage : launch_fused_stage;
   CUDA_TRY(launch(g->v, *P, stage, dt, g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der, g->buf[kStageIn[stage]],
                   ini_ptr(g), g->buf[CCZ4_BUF_U], g->buf[CCZ4_BUF_ACC], g->buf[kStageOut[stage]], s));
@@ -718,9 +792,7 @@ extern "C" ccz4_status ccz4_rk_stage(ccz4_grid *g, const ccz4_params *P, int sta
     return CCZ4_ERR_INVALID;
   }
   // the stage's input as the halo fill left it in the tile buffer
-  CUDA_TRY(launch_derive(g->v, g->buf[kStageIn[stage]], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der,
-                         all_fields(), P->precision == CCZ4_PREC_MIXED, true, false, (cudaStream_t)stream));
-  return stage_kernel(g, P, stage, dt, (cudaStream_t)stream);
+  return two_launch_stage(g, P, stage, dt, true, (cudaStream_t)stream);
 }
 
 extern "C" ccz4_status ccz4_step(ccz4_grid *g, const ccz4_params *P, double dt, int n_steps, void *stream) {
@@ -876,7 +948,7 @@ extern "C" ccz4_status ccz4_point_index(ccz4_grid *g, int n, const int *xyz, lon
 // The derivative pass of a monitor: the sums of g~, A~, phi, K and, for psi_4,
 // Gamma-hat; the tiles and mixed derivatives of every field, as the halo fill
 // of the buffer leaves them.
-static cudaError_t monitor_derivatives(ccz4_grid *g, int buf, bool gamma_hat, cudaStream_t s) {
+static cudaError_t monitor_derivatives(ccz4_grid *g, const GridView &w, int buf, bool gamma_hat, cudaStream_t s) {
   FieldList fl = all_fields();
   for (int k = 0; k < fl.n; ++k) {
     const int v = fl.f[k];
@@ -884,8 +956,7 @@ static cudaError_t monitor_derivatives(ccz4_grid *g, int buf, bool gamma_hat, cu
                       (gamma_hat && v >= GHX && v <= GHZ);
     if (!sums) fl.f[k] |= FIELD_NO_SUMS;
   }
-  return launch_derive(g->v, g->buf[buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der, fl, false, false, true,
-                       s);
+  return launch_derive(w, g->buf[buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der, fl, false, false, true, s);
 }
 
 extern "C" ccz4_status ccz4_psi4(ccz4_grid *g, int in_buf, int out_buf, const double centre[3], void *stream) {
@@ -896,9 +967,11 @@ extern "C" ccz4_status ccz4_psi4(ccz4_grid *g, int in_buf, int out_buf, const do
     return CCZ4_ERR_INVALID;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  CUDA_TRY(monitor_derivatives(g, in_buf, true, s));
-  CUDA_TRY(launch_psi4(g->v, g->der, g->buf[CCZ4_BUF_MIX], g->buf[in_buf], centre, g->buf[out_buf], s));
-  return CCZ4_OK;
+  return each_window(g, [&](const GridView &w) {
+    CUDA_TRY(monitor_derivatives(g, w, in_buf, true, s));
+    CUDA_TRY(launch_psi4(w, g->der, g->buf[CCZ4_BUF_MIX], g->buf[in_buf], centre, g->buf[out_buf], s));
+    return CCZ4_OK;
+  });
 }
 
 extern "C" ccz4_status ccz4_constraints(ccz4_grid *g, int buf, double out[5], double *dev_H, double *dev_M,
@@ -909,9 +982,13 @@ extern "C" ccz4_status ccz4_constraints(ccz4_grid *g, int buf, double out[5], do
     return CCZ4_ERR_INVALID;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  CUDA_TRY(monitor_derivatives(g, buf, false, s));
-  CUDA_TRY(launch_constraints_der(g->v, g->der, g->buf[CCZ4_BUF_MIX], g->buf[buf], dev_H, dev_M, g->red_partial,
-                                  g->red_blocks, g->red_out, s));
+  const ccz4_status st = each_window(g, [&](const GridView &w) {
+    CUDA_TRY(monitor_derivatives(g, w, buf, false, s));
+    CUDA_TRY(launch_constraints_der(w, g->der, g->buf[CCZ4_BUF_MIX], g->buf[buf], dev_H, dev_M, g->red_partial, s));
+    return CCZ4_OK;
+  });
+  if (st != CCZ4_OK) return st;
+  CUDA_TRY(launch_constraints_norms(g->v, g->red_partial, g->red_blocks, g->red_out, s));
   CUDA_TRY(cudaMemcpyAsync(g->host_out, g->red_out, sizeof(double) * 5, cudaMemcpyDeviceToHost, s));
   unsigned status = 0;
   CUDA_TRY(cudaMemcpyAsync(&status, g->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, s));

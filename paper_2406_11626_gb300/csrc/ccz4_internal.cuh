@@ -112,6 +112,9 @@ struct GridView {
   unsigned long long *queue;   // work counter of the queue launch of the stage kernel, or nullptr (flat)
   int stage_shape;             // launch shape of the flat stage kernel (CCZ4_STAGE_SHAPE_*)
   int fill_shape;              // launch shape of the halo fill (CCZ4_FILL_SHAPE_*)
+  // window of a derivative pass and the kernels that read it: patches w0 .. w0 + wn, whose sums stand at the
+  // start of a derivative buffer of wcap patches
+  int w0, wn, wcap;
 };
 
 // Level of patch n (0 on a single level).
@@ -179,6 +182,11 @@ namespace ccz4 {
 void set_error(const char *fmt, ...);
 // Gives every page of a host array that a copy is about to write its memory (ccz4_capi.cu).
 void back_host_pages(void *p, size_t bytes);
+// The patches that a derivative buffer of `slots` doubles a point shall hold: all, or equal windows of a bounded
+// number of points and at most half of the free memory (0 slots: whatever memory is free).
+int fitting_window(const GridView &v, int slots);
+// The next smaller window, 0 if there is none.
+int smaller_window(const GridView &v, int patches);
 }
 
 struct ccz4_grid {
@@ -216,7 +224,7 @@ struct ccz4_grid {
   void *alloc_ctx;
   int fused;                    // CCZ4_LAUNCH_FUSED: one cooperative launch per RK stage (p = 9)
   int pair;                     // FP64 stages in one launch, derivatives beside the algebra (pair_pays)
-  double *der;                  // derivative buffer, [DER_SLOTS][n_points] (derive.cuh), from the same allocator
+  double *der;                  // derivative buffer, [DER_SLOTS][v.wcap p^3] (derive.h), from the same allocator
 };
 
 // Kernel launchers (one translation unit each).
@@ -263,6 +271,8 @@ cudaError_t launch_restrict(const GridView &g, const int *par, const int *kid, i
 cudaError_t launch_constraints(const GridView &g, const double *tile, double *H, double *M,
                                double *partial, int blocks, double *out5, cudaStream_t s);
 cudaError_t prepare_constraints();
+// (the block sums of g's window, then the norms of all blocks')
 cudaError_t launch_constraints_der(const GridView &g, const double *der, const double *mix, const double *in, double *H,
-                                   double *M, double *partial, int blocks, double *out5, cudaStream_t s);
+                                   double *M, double *partial, cudaStream_t s);
+cudaError_t launch_constraints_norms(const GridView &g, const double *partial, int blocks, double *out5, cudaStream_t s);
 }  // namespace ccz4

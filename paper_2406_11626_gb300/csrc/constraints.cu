@@ -166,16 +166,16 @@ template <bool DER>
 __global__ void __launch_bounds__(RED_THREADS, DER ? 2 : 1) constraints_kernel(GridView g, ConsCoef LC, ConsSrc src, double *H,
                                                                      double *M, double *partial) {
   __shared__ double sh[5][RED_THREADS];
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int p = g.p, T = g.T;
+  const int p3 = p * p * p;  // 32-bit division: every state index is below 2^31
+  const long long q0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, i = (long long)g.w0 * p3 + q0;
   double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  if (i < g.n_points) {
-    const int p = g.p, T = g.T;
-    const int p3 = p * p * p;  // 32-bit division: every state index is below 2^31
+  if (q0 < (long long)g.wn * p3) {
     const int n = (int)i / p3;
     const int r = (int)i - n * p3;
     double h, m[3];
     if constexpr (DER) {
-      constraints_point(der_view<false>(g, src.der, src.mix, src.in, i), LC.C[patch_level(g, n)], h, m);
+      constraints_point(der_view<false>(g, src.der, src.mix, src.in, i, q0), LC.C[patch_level(g, n)], h, m);
     } else {
       const int z = r / (p * p), y = (r / p) % p, x = r % p;
       Nbhd N;
@@ -369,8 +369,10 @@ __global__ void __launch_bounds__(256) enforce_kernel(GridView g, double *U) {
 
 int constraint_blocks(long long n_points) { return (int)((n_points + RED_THREADS - 1) / RED_THREADS); }
 
+// The block sums of the points of g's window, at their places among all blocks' (a window starts at a
+// multiple of RED_THREADS points).
 static cudaError_t launch_constraints_from(const GridView &g, const ConsSrc &src, double *H, double *M, double *partial,
-                                           int blocks, double *out5, cudaStream_t s) {
+                                           cudaStream_t s) {
   ConsCoef LC;
   for (int l = 0; l < MAX_LEVELS; ++l) {
     const double dx = g.ldx[l];
@@ -379,19 +381,24 @@ static cudaError_t launch_constraints_from(const GridView &g, const ConsSrc &src
     LC.C[l].c3 = 1.0 / (144.0 * dx * dx);
     LC.C[l].cko = 0.0;
   }
-  if (blocks > 0) {
-    if (src.der) constraints_kernel<true><<<blocks, RED_THREADS, 0, s>>>(g, LC, src, H, M, partial);
-    else constraints_kernel<false><<<blocks, RED_THREADS, 0, s>>>(g, LC, src, H, M, partial);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+  const long long p3 = (long long)g.p * g.p * g.p;
+  const int blocks = constraint_blocks(g.wn * p3);
+  if (blocks == 0) return cudaSuccess;
+  partial += 5 * (g.w0 * p3 / RED_THREADS);
+  if (src.der) constraints_kernel<true><<<blocks, RED_THREADS, 0, s>>>(g, LC, src, H, M, partial);
+  else constraints_kernel<false><<<blocks, RED_THREADS, 0, s>>>(g, LC, src, H, M, partial);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_constraints_norms(const GridView &g, const double *partial, int blocks, double *out5, cudaStream_t s) {
   reduce_partials<<<1, RED_THREADS, 0, s>>>(partial, blocks, (double)g.n_leaf_points, out5);
   return cudaGetLastError();
 }
 
 cudaError_t launch_constraints(const GridView &g, const double *tile, double *H, double *M, double *partial,
                                int blocks, double *out5, cudaStream_t s) {
-  return launch_constraints_from(g, ConsSrc{tile, nullptr, nullptr, nullptr}, H, M, partial, blocks, out5, s);
+  const cudaError_t e = launch_constraints_from(g, ConsSrc{tile, nullptr, nullptr, nullptr}, H, M, partial, s);
+  return e == cudaSuccess ? launch_constraints_norms(g, partial, blocks, out5, s) : e;
 }
 
 // Loads the kernels of the monitors that take tiles alone (a kernel's first
@@ -404,8 +411,8 @@ cudaError_t prepare_constraints() {
 }
 
 cudaError_t launch_constraints_der(const GridView &g, const double *der, const double *mix, const double *in, double *H,
-                                   double *M, double *partial, int blocks, double *out5, cudaStream_t s) {
-  return launch_constraints_from(g, ConsSrc{nullptr, der, mix, in}, H, M, partial, blocks, out5, s);
+                                   double *M, double *partial, cudaStream_t s) {
+  return launch_constraints_from(g, ConsSrc{nullptr, der, mix, in}, H, M, partial, s);
 }
 
 cudaError_t launch_constraints_excluded(const GridView &g, const double *H, const double *M, int n_centres,

@@ -28,10 +28,10 @@ struct DerView {
   const float *f;      // FP32 slots (mixed precision)
   const double *mix;
   const float *mixf;
-  long long np;        // distance between slots
+  long long np, dnp;   // distance between slots of mix and of the derivative buffer
   __device__ __forceinline__ double at(int v, int) const { return c[v * fs]; }
-  __device__ __forceinline__ double slot(int k) const { return CCZ4_DER_LOAD(d + k * np); }
-  __device__ __forceinline__ float slotf(int k) const { return CCZ4_DER_LOAD(f + k * np); }
+  __device__ __forceinline__ double slot(int k) const { return CCZ4_DER_LOAD(d + k * dnp); }
+  __device__ __forceinline__ float slotf(int k) const { return CCZ4_DER_LOAD(f + k * dnp); }
   __device__ __forceinline__ double mixed(int k) const { return CCZ4_DER_LOAD(mix + k * np); }
   __device__ __forceinline__ float mixedf(int k) const { return CCZ4_DER_LOAD(mixf + k * np); }
   // first-derivative sum along axis k, dissipation sum (k = 3) and pure second sum of field v
@@ -105,18 +105,20 @@ __device__ __forceinline__ D fdkl(const DerView<false> &N, int v, int k, int l, 
   return N.mixed(mix_slot(v) + k + l - 1);
 }
 
-// The view of interior point i, its values from the state-shaped buffer `in`.
+// The view of interior point i, its values from the state-shaped buffer `in`, its sums at place q of the
+// derivative buffer.
 template <bool M>
 __device__ __forceinline__ DerView<M> der_view(const GridView &g, const double *der, const double *mix, const double *in,
-                                               long long i) {
+                                               long long i, long long q) {
   DerView<M> N;
   N.c = in + i;
   N.fs = g.S;
   N.st[0] = 0;
   N.st[1] = 1;
   N.st[2] = 2;
-  N.d = der + i;
-  N.f = reinterpret_cast<const float *>(der + DER_D * g.n_points) + i;
+  N.dnp = (long long)g.wcap * (g.p * g.p * g.p);
+  N.d = der + q;
+  N.f = reinterpret_cast<const float *>(der + DER_D * N.dnp) + q;
   N.mix = mix + i;
   N.mixf = reinterpret_cast<const float *>(mix) + i;
   N.np = g.n_points;

@@ -9,8 +9,8 @@ __global__ void __launch_bounds__(FILL_SHAPE_THREADS[SHAPE], (PF == 9 ? 1024 : 7
     derive_kernel(GridView g, const double *__restrict__ src, double *tile, double *__restrict__ mix,
                   double *__restrict__ der, LevelScale ls, FieldList fl, bool tile_out) {
   extern __shared__ double smem[];
-  derive_patch<SRC, MIXED, FILL_SHAPE_THREADS[SHAPE], PF, NF>(g, src, tile, mix, der, ls, fl, blockIdx.x,
-                                                                   blockIdx.y, gridDim.y, tile_out, smem);
+  derive_patch<SRC, MIXED, FILL_SHAPE_THREADS[SHAPE], PF, NF>(g, src, tile, mix, der, ls, fl, g.w0 + blockIdx.x, blockIdx.x,
+                                                              blockIdx.y, gridDim.y, tile_out, smem);
 }
 
 template <int SRC, int PF>
@@ -18,8 +18,8 @@ __global__ void __launch_bounds__(EdgeShape<PF>::threads, EdgeShape<PF>::blocks)
     derive_edge_kernel(GridView g, const double *__restrict__ src, double *tile, double *__restrict__ mix,
                        double *__restrict__ der, LevelScale ls, FieldList fl) {
   extern __shared__ double smem[];
-  derive_edge<SRC, EdgeShape<PF>::threads, PF, true>(g, src, tile, mix, der, ls, fl, blockIdx.x, blockIdx.y, gridDim.y,
-                                                     smem, threadIdx.x, 0);
+  derive_edge<SRC, EdgeShape<PF>::threads, PF, true>(g, src, tile, mix, der, ls, fl, g.w0 + blockIdx.x, blockIdx.x,
+                                                     blockIdx.y, gridDim.y, smem, threadIdx.x, 0);
 }
 
 // One field per block, 9^3 patches: small grids, whose every block is resident at once.
@@ -29,8 +29,8 @@ __global__ void __launch_bounds__(ONE_THREADS, 4)
     derive_field_kernel(GridView g, const double *__restrict__ src, double *tile, double *__restrict__ mix,
                         double *__restrict__ der, LevelScale ls, FieldList fl) {
   extern __shared__ double smem[];
-  derive_edge<SRC, ONE_THREADS, 9, true, true>(g, src, tile, mix, der, ls, fl, blockIdx.x, blockIdx.y, fl.n, smem,
-                                               threadIdx.x, 0);
+  derive_edge<SRC, ONE_THREADS, 9, true, true>(g, src, tile, mix, der, ls, fl, g.w0 + blockIdx.x, blockIdx.x, blockIdx.y,
+                                               fl.n, smem, threadIdx.x, 0);
 }
 
 // Field groups per patch. A block's set-up (the source table) is shared by
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(ONE_THREADS, 4)
 // blocks (27 patches of 9^3: one block per field).
 int field_groups(const GridView &g, const FieldList &fl) {
   const int want = 6 * 152;
-  int k = g.n_patches > 0 ? (want + g.n_patches - 1) / g.n_patches : 1;
+  int k = g.wn > 0 ? (want + g.wn - 1) / g.wn : 1;
   k = k < 1 ? 1 : k;
   return k < fl.n ? k : fl.n;
 }
@@ -47,7 +47,7 @@ int field_groups(const GridView &g, const FieldList &fl) {
 template <int SRC, bool MIXED, int SHAPE, int PF, int NF>
 cudaError_t launch_one(const GridView &g, const double *src, double *tile, double *mix, double *der,
                        const FieldList &fl, bool tile_out, cudaStream_t s) {
-  const dim3 grid(g.n_patches, field_groups(g, fl));
+  const dim3 grid(g.wn, field_groups(g, fl));
   derive_kernel<SRC, MIXED, SHAPE, PF, NF><<<grid, FILL_SHAPE_THREADS[SHAPE], derive_smem_bytes(g.p), s>>>(
       g, src, tile, mix, der, level_scale(g), fl, tile_out);
   return cudaGetLastError();
@@ -57,11 +57,11 @@ template <int SRC, int PF>
 cudaError_t launch_fixed(const GridView &g, const double *src, double *tile, double *mix, double *der,
                          const FieldList &fl, cudaStream_t s) {
   if (PF == 9 && field_groups(g, fl) == fl.n) {
-    derive_field_kernel<SRC><<<dim3(g.n_patches, fl.n), ONE_THREADS, edge_smem_bytes(9, true), s>>>(
+    derive_field_kernel<SRC><<<dim3(g.wn, fl.n), ONE_THREADS, edge_smem_bytes(9, true), s>>>(
         g, src, tile, mix, der, level_scale(g), fl);
     return cudaGetLastError();
   }
-  derive_edge_kernel<SRC, PF><<<dim3(g.n_patches, field_groups(g, fl)), EdgeShape<PF>::threads, edge_smem_bytes(PF), s>>>(
+  derive_edge_kernel<SRC, PF><<<dim3(g.wn, field_groups(g, fl)), EdgeShape<PF>::threads, edge_smem_bytes(PF), s>>>(
       g, src, tile, mix, der, level_scale(g), fl);
   return cudaGetLastError();
 }
@@ -152,7 +152,7 @@ FieldList all_fields() {
 
 cudaError_t launch_derive(const GridView &g, const double *src, double *tile, double *mix, double *der,
                           const FieldList &fl, bool mixed, bool from_tile, bool tile_out, cudaStream_t s) {
-  if (g.n_patches == 0 || fl.n == 0) return cudaSuccess;
+  if (g.wn == 0 || fl.n == 0) return cudaSuccess;
   if (from_tile)
     return mixed ? launch_shape<FROM_TILE, true>(g, src, tile, mix, der, fl, false, s)
                  : launch_shape<FROM_TILE, false>(g, src, tile, mix, der, fl, false, s);
@@ -164,7 +164,7 @@ cudaError_t launch_derive(const GridView &g, const double *src, double *tile, do
 }
 
 cudaError_t launch_derive_fo(const GridView &g, const double *src, double *der, const FieldList &fl, cudaStream_t s) {
-  if (g.n_patches == 0 || fl.n == 0) return cudaSuccess;
+  if (g.wn == 0 || fl.n == 0) return cudaSuccess;
   if (g.p == 9) return launch_one<FROM_LEVEL, false, 0, 9, 58>(g, src, nullptr, nullptr, der, fl, false, s);
   return launch_one<FROM_LEVEL, false, 0, 0, 58>(g, src, nullptr, nullptr, der, fl, false, s);
 }

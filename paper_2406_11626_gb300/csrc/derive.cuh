@@ -86,14 +86,14 @@ inline size_t derive_smem_bytes(int p) {
   return T3 * (8 + 4) + 8 * (size_t)derive_shared(p);
 }
 
-// The fields group, group + groups, ... of the list, of patch n, by one block
-// of THREADS threads. NF: fields of the formulation (25, or 58 without second
+// The fields group, group + groups, ... of the list, of patch n, into the place
+// of patch `at_patch` of the derivative buffer, by one block of THREADS threads. NF: fields of the formulation (25, or 58 without second
 // derivatives). tile: the tile buffer; interpolated halo points of a mesh pass
 // through it, tile_out (FP64) has the whole tile written to it, FROM_TILE reads it.
 template <int SRC, bool MIXED, int THREADS, int PF, int NF>
 __device__ __forceinline__ void derive_patch(const GridView &g, const double *__restrict__ src, double *tile,
                                              double *__restrict__ mix, double *__restrict__ der, const LevelScale &ls,
-                                             const FieldList &fl, int n, int group, int groups, bool tile_out,
+                                             const FieldList &fl, int n, int at_patch, int group, int groups, bool tile_out,
                                              double *smem) {
   constexpr int BATCH = PF == 9 && THREADS == 256 ? 7 : 8;  // 15^3 tile points: two rounds of 7 x 256
   const int p = PF > 0 ? PF : g.p, T = PF > 0 ? PF + 2 * HALO : g.T;
@@ -140,6 +140,7 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
   const double cmix = MESH ? ls.cmix[patch_level(g, n)] : ls.cmix[0];
   const float cmixf = MESH ? ls.cmixf[patch_level(g, n)] : ls.cmixf[0];
   const long long pbase = (long long)n * p3, np = g.n_points;
+  const long long dbase = (long long)at_patch * p3, dnp = (long long)g.wcap * p3;
   // tile offsets of this thread's points (a compile-time edge: the same for every field)
   constexpr int ROUNDS = PF > 0 ? (PF * PF * PF + THREADS - 1) / THREADS : 1;
   auto centre_at = [&](int q) {
@@ -254,10 +255,10 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
       }
     }
     if (!sums) continue;
-    double *dd = der + (MIXED ? (v == ALPHA ? 0 : 7) : 4 * v) * np + pbase;
-    double *dp = MIXED ? dd + 4 * np : der + (4 * NF + 3 * (second ? slot / 3 : 0)) * np + pbase;
-    float *fd = reinterpret_cast<float *>(der + DER_D * np) + (long long)(4 * der_f(v)) * np + pbase;
-    float *fp = reinterpret_cast<float *>(der + DER_D * np) + (long long)(DER_F + 3 * der_f2(v)) * np + pbase;
+    double *dd = der + (MIXED ? (v == ALPHA ? 0 : 7) : 4 * v) * dnp + dbase;
+    double *dp = MIXED ? dd + 4 * dnp : der + (4 * NF + 3 * (second ? slot / 3 : 0)) * dnp + dbase;
+    float *fd = reinterpret_cast<float *>(der + DER_D * dnp) + (long long)(4 * der_f(v)) * dnp + dbase;
+    float *fp = reinterpret_cast<float *>(der + DER_D * dnp) + (long long)(DER_F + 3 * der_f2(v)) * dnp + dbase;
     auto each = [&](auto is_second, auto zero) {
       using O = decltype(zero);
       constexpr bool SECOND = decltype(is_second)::value;
@@ -275,10 +276,10 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
           b = dp + q;
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) a[k * np] = o[k];
+        for (int k = 0; k < 4; ++k) a[k * dnp] = o[k];
         if (SECOND) {
 #pragma unroll
-          for (int k = 0; k < 3; ++k) b[k * np] = o[4 + k];
+          for (int k = 0; k < 3; ++k) b[k * dnp] = o[4 + k];
         }
       };
       if (PF > 0) {

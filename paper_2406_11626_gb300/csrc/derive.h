@@ -7,7 +7,8 @@
 namespace ccz4 {
 
 // ---- layout of the derivative buffer ------------------------------------------------
-// Slots of n_points values each, point index fastest. FP64 (and the
+// Slots of one value for each point of the buffer's patches (GridView::wcap; the
+// points of the pass's window in order), point index fastest. FP64 (and the
 // first-order formulation): 4 v + k for the first-derivative sum along k and
 // 4 v + 3 for the dissipation sum of field v; from 4 NV on, three pure second
 // sums for each field of the mixed-derivative buffer, in its order.

@@ -114,14 +114,14 @@ constexpr size_t edge_smem_bytes(int p, bool one = false) {
 }
 static_assert(4 * 15 * 15 * 15 <= 8 * (EDGE_EZ(9) + EDGE_EY(9)), "a source table in the place of Ez and Ey");
 
-// The fields group, group + groups, ... of the list, of patch n, by the
-// THREADS threads tid (whole warps) that share barrier bar. tile: the tile buffer;
+// The fields group, group + groups, ... of the list, of patch n, into the place
+// of patch `at_patch` of the derivative buffer, by the THREADS threads tid (whole warps) that share barrier bar. tile: the tile buffer;
 // interpolated halo points of a mesh pass through it.
 template <int SRC, int THREADS, int PF, bool CVT, bool ONE = false>
 __device__ __forceinline__ void derive_edge(const GridView &g, const double *__restrict__ src, double *tile,
                                             double *__restrict__ mix, double *__restrict__ der, const LevelScale &ls,
-                                            const FieldList &fl, int n, int group, int groups, double *smem,
-                                            int tid, int bar) {
+                                            const FieldList &fl, int n, int at_patch, int group, int groups,
+                                            double *smem, int tid, int bar) {
   constexpr int T = PF + 2 * HALO, T2 = T * T, T3 = T2 * T, P2 = PF * PF, P3 = P2 * PF, PE = PF + 4;
   constexpr int BATCH = (T3 + THREADS - 1) / THREADS <= 10 ? (T3 + THREADS - 1) / THREADS : 7;
   constexpr int ROUNDS = (P3 + THREADS - 1) / THREADS;
@@ -134,6 +134,7 @@ __device__ __forceinline__ void derive_edge(const GridView &g, const double *__r
   const int lev = MESH ? patch_level(g, n) : 0;
   const double cmix = MESH ? ls.cmix[lev] : ls.cmix[0];
   const long long pbase = (long long)n * P3, np = g.n_points;
+  const long long dbase = (long long)at_patch * P3, dnp = (long long)g.wcap * P3;
   // tile offsets of this thread's points, the same for every field (few rounds: kept)
   constexpr bool KEEP = ROUNDS <= 3;
   auto tile_at = [&](int q) { return (q / P2 + HALO) * T2 + ((q / PF) % PF + HALO) * T + (q % PF + HALO); };
@@ -180,7 +181,7 @@ __device__ __forceinline__ void derive_edge(const GridView &g, const double *__r
       }
     }
     block_sync<THREADS>(bar);
-    double *d = der + 4 * v * np + pbase, *dp = der + (4 * NV + 3 * (second ? slot / 3 : 0)) * np + pbase;
+    double *d = der + 4 * v * dnp + dbase, *dp = der + (4 * NV + 3 * (second ? slot / 3 : 0)) * dnp + dbase;
     auto take = [&](auto is_second) {
       constexpr bool SECOND = decltype(is_second)::value;
 #pragma unroll 1
@@ -191,10 +192,10 @@ __device__ __forceinline__ void derive_edge(const GridView &g, const double *__r
         double o[7];
         point_sums<SECOND, CVT>(tw + c, ex + c, T, o);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) d[k * np + q] = o[k];
+        for (int k = 0; k < 4; ++k) d[k * dnp + q] = o[k];
         if (SECOND) {
 #pragma unroll
-          for (int k = 0; k < 3; ++k) dp[k * np + q] = o[4 + k];
+          for (int k = 0; k < 3; ++k) dp[k * dnp + q] = o[4 + k];
         }
         if (SECOND) {
           const int row = q / PF;

@@ -29,9 +29,10 @@ namespace {
 // first derivatives, written into the state `out`.
 __global__ void __launch_bounds__(128) fo_reconstruct_kernel(GridView g, const double *__restrict__ der,
                                                              double *__restrict__ out, double c1) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.n_points) return;
-  const FoView N = fo_view(g, der, out, i);
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x, p3 = g.p * g.p * g.p;
+  if (q >= g.wn * p3) return;
+  const long long i = g.w0 * p3 + q;
+  const FoView N = fo_view(g, der, out, i, q);
   const long long S = g.S;
   auto put = [&](int v, double val) { out[v * S + i] = val; };
   fo_reconstruct_point(N, c1, put);
@@ -66,7 +67,8 @@ struct ccz4_fo {
   ccz4_grid *g;
   int variant;
   double *buf[6];  // U, Y0, Y1, ACC, RHS, INI: [58][S]
-  double *der;     // derivative buffer, [4 x 58][n_points]
+  GridView v;      // the grid's, with the windows of this derivative buffer
+  double *der;     // derivative buffer, [4 x 58][v.wcap p^3]
 };
 
 static const int kFoIn[4] = {CCZ4_BUF_U, CCZ4_BUF_Y0, CCZ4_BUF_Y1, CCZ4_BUF_Y0};
@@ -88,20 +90,44 @@ static void fo_release(ccz4_fo *f) {
   free(f);
 }
 
-// The derivative pass over fields [v0, v0 + nv).
-static cudaError_t fo_derive(const ccz4_fo *f, const double *src, int v0, int nv, cudaStream_t s) {
+// f on the view of each window of the formulation's derivative buffer.
+template <class F>
+static cudaError_t fo_windows(const ccz4_fo *f, F call) {
+  GridView w = f->v;
+  cudaError_t e = cudaSuccess;
+  for (w.w0 = 0; w.w0 < w.n_patches && e == cudaSuccess; w.w0 += w.wcap) {
+    w.wn = w.n_patches - w.w0 < w.wcap ? w.n_patches - w.w0 : w.wcap;
+    e = call(w);
+  }
+  return e;
+}
+
+// The derivative pass over fields [v0, v0 + nv) of a window.
+static cudaError_t fo_derive(const ccz4_fo *f, const GridView &w, const double *src, int v0, int nv, cudaStream_t s) {
   FieldList fl;
   fl.n = nv;
   for (int k = 0; k < nv; ++k) fl.f[k] = (unsigned char)(v0 + k);
-  return launch_derive_fo(f->g->v, src, f->der, fl, s);
+  return launch_derive_fo(w, src, f->der, fl, s);
 }
 
 static cudaError_t fo_reconstruct_into(const ccz4_fo *f, double *state, cudaStream_t s) {
-  const GridView &v = f->g->v;
-  cudaError_t e = fo_derive(f, state, 0, NV, s);
-  if (e != cudaSuccess || v.n_points == 0) return e;
-  fo_reconstruct_kernel<<<(unsigned)((v.n_points + 127) / 128), 128, 0, s>>>(v, f->der, state, 1.0 / (12.0 * v.dx));
-  return cudaGetLastError();
+  return fo_windows(f, [&](const GridView &w) {
+    const cudaError_t e = fo_derive(f, w, state, 0, NV, s);
+    if (e != cudaSuccess) return e;
+    const long long points = (long long)w.wn * w.p * w.p * w.p;
+    fo_reconstruct_kernel<<<(unsigned)((points + 127) / 128), 128, 0, s>>>(w, f->der, state, 1.0 / (12.0 * w.dx));
+    return cudaGetLastError();
+  });
+}
+
+// The right-hand side or a stage (launch_fo) of every window, from the derivatives of fields [v0, 58) and
+// those that the buffer holds already.
+static cudaError_t fo_stage_windows(const ccz4_fo *f, int stage, const ccz4_params &P, bool first, const double *in,
+                                    int v0, const double *ini, const FoStageArgs &a, cudaStream_t s) {
+  return fo_windows(f, [&](const GridView &w) {
+    const cudaError_t e = fo_derive(f, w, in, v0, NVF - v0, s);
+    return e == cudaSuccess ? launch_fo(stage, w, P, first, f->der, in, ini, a, s) : e;
+  });
 }
 
 static const double *fo_ini(const ccz4_fo *f) {
@@ -147,10 +173,15 @@ extern "C" ccz4_status ccz4_fo_alloc(ccz4_grid *g, int variant, ccz4_fo **out) {
       return CCZ4_ERR_NOMEM;
     }
   }
-  const size_t der = sizeof(double) * 4 * (size_t)NVF * (size_t)v.n_points;
-  if (der && cudaMalloc(&f->der, der) != cudaSuccess) {
-    set_error("fo_alloc: cudaMalloc of the %zu-byte derivative buffer failed: %s", der,
-              cudaGetErrorString(cudaGetLastError()));
+  f->v = v;
+  for (f->v.wcap = fitting_window(v, 4 * NVF); v.n_points > 0;) {
+    const size_t der = sizeof(double) * 4 * (size_t)NVF * (size_t)f->v.wcap * (size_t)(v.p * v.p * v.p);
+    if (cudaMalloc(&f->der, der) == cudaSuccess) break;
+    f->der = nullptr;
+    const cudaError_t e = cudaGetLastError();
+    f->v.wcap = smaller_window(v, f->v.wcap);
+    if (f->v.wcap > 0) continue;
+    set_error("fo_alloc: cudaMalloc of the %zu-byte derivative buffer failed: %s", der, cudaGetErrorString(e));
     fo_release(f);
     return CCZ4_ERR_NOMEM;
   }
@@ -226,9 +257,8 @@ extern "C" ccz4_status ccz4_fo_rhs(ccz4_fo *f, const ccz4_params *P, int in_buf,
   }
   cudaStream_t s = (cudaStream_t)stream;
   const double *in = f->buf[in_buf];
-  FO_TRY(fo_derive(f, in, 0, NVF, s));
   FoStageArgs a{nullptr, nullptr, f->buf[out_buf], 0.0};
-  FO_TRY(launch_fo(-1, f->g->v, *P, f->variant == CCZ4_FO_FIRST_ORDER, f->der, in, fo_ini(f), a, s));
+  FO_TRY(fo_stage_windows(f, -1, *P, f->variant == CCZ4_FO_FIRST_ORDER, in, 0, fo_ini(f), a, s));
   return CCZ4_OK;
 }
 
@@ -239,14 +269,11 @@ extern "C" ccz4_status ccz4_fo_rhs(ccz4_fo *f, const ccz4_params *P, int in_buf,
 static ccz4_status fo_stage(ccz4_fo *f, const ccz4_params *P, int stage, double dt, cudaStream_t s) {
   double *in = f->buf[kFoIn[stage]];
   const bool first = f->variant == CCZ4_FO_FIRST_ORDER;
-  if (first) {
-    FO_TRY(fo_derive(f, in, 0, NVF, s));
-  } else {
-    FO_TRY(fo_reconstruct_into(f, in, s));
-    FO_TRY(fo_derive(f, in, NV, NVF - NV, s));
-  }
+  if (!first) FO_TRY(fo_reconstruct_into(f, in, s));
+  // (one window: the reconstruction has left the primaries' derivatives in the buffer)
+  const int v0 = !first && f->v.wcap >= f->v.n_patches ? NV : 0;
   FoStageArgs a{f->buf[CCZ4_BUF_U], f->buf[CCZ4_BUF_ACC], f->buf[kFoOut[stage]], dt};
-  FO_TRY(launch_fo(stage, f->g->v, *P, first, f->der, in, fo_ini(f), a, s));
+  FO_TRY(fo_stage_windows(f, stage, *P, first, in, v0, fo_ini(f), a, s));
   if (stage == 3 && !first) FO_TRY(fo_reconstruct_into(f, f->buf[CCZ4_BUF_U], s));
   return CCZ4_OK;
 }

@@ -63,7 +63,7 @@ struct FoSink {
 struct FoView {
   const double *c;   // field 0 of the state at the point
   const double *d;   // slot 0 at the point
-  long long S, np;
+  long long S, np;   // distance between fields of the state, between slots of the buffer
   int st[3];
 };
 template <class D>
@@ -77,8 +77,9 @@ __device__ __forceinline__ D d1u(const FoView &N, int v, int axis) { return __ld
 template <class D>
 __device__ __forceinline__ D ko_sum(const FoView &N, int v) { return __ldcs(N.d + (4 * v + 3) * N.np); }
 
-__device__ __forceinline__ FoView fo_view(const GridView &g, const double *der, const double *in, long long i) {
-  return FoView{in + i, der + i, g.S, g.n_points, {0, 1, 2}};
+__device__ __forceinline__ FoView fo_view(const GridView &g, const double *der, const double *in, long long i,
+                                          long long q) {
+  return FoView{in + i, der + q, g.S, (long long)g.wcap * (g.p * g.p * g.p), {0, 1, 2}};
 }
 
 // All variables of one Sommerfeld ghost cell: the radiative condition (Eq.
@@ -110,7 +111,7 @@ __device__ __forceinline__ void fo_ghost_cell(const GridView &g, const ccz4_para
 }
 
 // The first ghost_blocks blocks: one thread per ghost cell. The others: one
-// thread per interior point, the 58-variable right-hand side (RED: with the
+// thread per interior point of the window, the 58-variable right-hand side (RED: with the
 // red terms; AUX: the auxiliary variables' equations too) from the derivative
 // buffer and the stage update of what it evolves.
 // The FP64 pipe holds it (ncu: 86 % busy; 3, 4 and 5 blocks within 1 %), so what
@@ -127,9 +128,10 @@ __global__ void __launch_bounds__(128, CCZ4_FO_MIN_BLOCKS)
     if (id < g.n_ghost) fo_ghost_cell<MODE>(g, P, in, ini, a, id);
     return;
   }
-  const long long i = (long long)(blockIdx.x - ghost_blocks) * blockDim.x + threadIdx.x;
-  if (i >= g.n_points) return;
-  const FoView N = fo_view(g, der, in, i);
+  const long long q = (long long)(blockIdx.x - ghost_blocks) * blockDim.x + threadIdx.x, p3 = g.p * g.p * g.p;
+  if (q >= g.wn * p3) return;
+  const long long i = g.w0 * p3 + q;
+  const FoView N = fo_view(g, der, in, i, q);
   FoSink<MODE> sink{g.S, i, a};
   fo_rhs_point<RED, AUX>(F, N, C, sink);
   sink.finish();
@@ -144,13 +146,15 @@ inline StencilCoef<double> fo_coefs(double dx, double eps) {
   return C;
 }
 
-// Launches the stage kernel of one (MODE, RED, AUX) on every ghost cell and interior point.
+// Launches the stage kernel of one (MODE, RED, AUX) on the interior points of the window and, with the first
+// one, every ghost cell.
 template <int MODE, bool RED, bool AUX>
 cudaError_t launch_fo_interior(const GridView &g, const ccz4_params &P, const double *der, const double *in,
                                const double *ini, const FoStageArgs &a, cudaStream_t s) {
   const FoPhys F{make_phys<double>(P), P.mu};
-  const int t = g.n_points < 16LL * 152 * 128 ? 32 : 128;  // a small grid spreads over the SMs in shares of 32 points
-  const long long gb = (g.n_ghost + t - 1) / t, nb = (g.n_points + t - 1) / t;
+  const long long points = (long long)g.wn * g.p * g.p * g.p, ghosts = g.w0 == 0 ? g.n_ghost : 0;
+  const int t = points < 16LL * 152 * 128 ? 32 : 128;  // a small grid spreads over the SMs in shares of 32 points
+  const long long gb = (ghosts + t - 1) / t, nb = (points + t - 1) / t;
   if (gb + nb == 0) return cudaSuccess;
   fo_interior_kernel<MODE, RED, AUX><<<(unsigned)(gb + nb), t, 0, s>>>(g, F, fo_coefs(g.dx, P.ko_eps), P, der, in, ini, a,
                                                                        (int)gb);

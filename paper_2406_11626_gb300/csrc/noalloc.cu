@@ -87,6 +87,7 @@ extern "C" ccz4_status ccz4_constraints_noalloc(const double *tiles, int p, int 
   v.T = p + 2 * HALO;
   v.n_patches = n_patches;
   v.n_points = n_points;
+  v.wn = n_patches;
   v.T3 = (long long)v.T * v.T * v.T;
   v.dx = dx;
   v.n_levels = 1;

@@ -312,9 +312,10 @@ __device__ __forceinline__ void psi4_point(const DerView<false> &N, const Stenci
 __global__ void __launch_bounds__(128, 3) psi4_kernel(GridView g, Psi4Coef PC, const double *__restrict__ der,
                                                       const double *__restrict__ mix, const double *__restrict__ in,
                                                       double cx, double cy, double cz, double *__restrict__ out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.n_points) return;
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int p = g.p, p3 = p * p * p;
+  if (q >= (long long)g.wn * p3) return;
+  const long long i = (long long)g.w0 * p3 + q;
   const int n = (int)i / p3;
   const int r = (int)i - n * p3;
   const int z = r / (p * p), y = (r / p) % p, x = r % p;
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(128, 3) psi4_kernel(GridView g, Psi4Coef PC, c
                        g.origin[1] + (__ldg(g.ijk + 3 * n + 1) * p + y + 0.5) * h - cy,
                        g.origin[2] + (__ldg(g.ijk + 3 * n + 2) * p + z + 0.5) * h - cz};
   double v[2];
-  psi4_point(der_view<false>(g, der, mix, in, i), PC.C[lev], X, v);
+  psi4_point(der_view<false>(g, der, mix, in, i, q), PC.C[lev], X, v);
   out[i] = v[0];
   out[g.S + i] = v[1];
 }
@@ -333,7 +334,8 @@ __global__ void __launch_bounds__(128, 3) psi4_kernel(GridView g, Psi4Coef PC, c
 
 cudaError_t launch_psi4(const GridView &g, const double *der, const double *mix, const double *in,
                         const double centre[3], double *out, cudaStream_t s) {
-  if (g.n_points == 0) return cudaSuccess;
+  const long long points = (long long)g.wn * g.p * g.p * g.p;
+  if (points == 0) return cudaSuccess;
   Psi4Coef PC;
   for (int l = 0; l < MAX_LEVELS; ++l) {
     const double dx = g.ldx[l];
@@ -342,7 +344,7 @@ cudaError_t launch_psi4(const GridView &g, const double *der, const double *mix,
     PC.C[l].c3 = 1.0 / (144.0 * dx * dx);
     PC.C[l].cko = 0.0;
   }
-  psi4_kernel<<<(unsigned)((g.n_points + 127) / 128), 128, 0, s>>>(g, PC, der, mix, in, centre[0], centre[1], centre[2],
+  psi4_kernel<<<(unsigned)((points + 127) / 128), 128, 0, s>>>(g, PC, der, mix, in, centre[0], centre[1], centre[2],
                                                                     out);
   return cudaGetLastError();
 }

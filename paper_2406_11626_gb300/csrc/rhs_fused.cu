@@ -27,26 +27,34 @@ __global__ void __launch_bounds__(FUSED_THREADS, (StageBlocks<R, 0>::value))
                        double *tile, double *mix, double *der, const double *__restrict__ in,
                        const double *__restrict__ ini, StageArgs a) {
   extern __shared__ double smem[];
-  for (int n = blockIdx.x; n < g.n_patches; n += gridDim.x) {
-    constexpr int SRC = MESH ? FROM_MESH : FROM_LEVEL;
-    if constexpr (std::is_same<R, float>::value)
-      derive_patch<SRC, true, FUSED_THREADS, FUSED_PF, NV>(g, in, tile, mix, der, ls, fl, n, 0, 1, false, smem);
-    else
-      derive_edge<SRC, FUSED_THREADS, FUSED_PF, true>(g, in, tile, mix, der, ls, fl, n, 0, 1, smem, threadIdx.x, 0);
-    __syncthreads();  // the next patch's source table overwrites this one's shared memory
-  }
-  cooperative_groups::this_grid().sync();
   const StageBufs b{der, mix, in, ini};
   const int lane = threadIdx.x & 31;
-  const long long warps = (long long)gridDim.x * (FUSED_THREADS / 32), gi = (g.n_ghost + 31) / 32;
-  for (long long item = (long long)blockIdx.x * (FUSED_THREADS / 32) + threadIdx.x / 32; (item - gi) * 32 < g.n_points;
-       item += warps) {
-    if (item < gi) {
-      const long long id = item * 32 + lane;
-      if (id < g.n_ghost) ghost_cell<MODE>(g, Pg, b, a, id);
-    } else {
-      const long long i = (item - gi) * 32 + lane;
-      if (i < g.n_points) stage_point<MODE, R, MESH>(g, P, LC, b, a, i);
+  const long long warps = (long long)gridDim.x * (FUSED_THREADS / 32);
+  constexpr int P3 = FUSED_PF * FUSED_PF * FUSED_PF;
+#pragma unroll 1
+  for (int w0 = 0; w0 < g.n_patches; w0 += g.wcap) {  // (the derivative buffer holds wcap patches)
+    const int wn = g.n_patches - w0 < g.wcap ? g.n_patches - w0 : g.wcap;
+    if (w0 > 0) cooperative_groups::this_grid().sync();  // the sums of the window before are read
+    for (int k = blockIdx.x; k < wn; k += gridDim.x) {
+      constexpr int SRC = MESH ? FROM_MESH : FROM_LEVEL;
+      const int n = w0 + k;
+      if constexpr (std::is_same<R, float>::value)
+        derive_patch<SRC, true, FUSED_THREADS, FUSED_PF, NV>(g, in, tile, mix, der, ls, fl, n, k, 0, 1, false, smem);
+      else
+        derive_edge<SRC, FUSED_THREADS, FUSED_PF, true>(g, in, tile, mix, der, ls, fl, n, k, 0, 1, smem, threadIdx.x, 0);
+      __syncthreads();  // the next patch's source table overwrites this one's shared memory
+    }
+    cooperative_groups::this_grid().sync();
+    const long long gi = w0 == 0 ? (g.n_ghost + 31) / 32 : 0, points = (long long)wn * P3;
+    for (long long item = (long long)blockIdx.x * (FUSED_THREADS / 32) + threadIdx.x / 32; (item - gi) * 32 < points;
+         item += warps) {
+      if (item < gi) {
+        const long long id = item * 32 + lane;
+        if (id < g.n_ghost) ghost_cell<MODE>(g, Pg, b, a, id);
+      } else {
+        const long long q = (item - gi) * 32 + lane;
+        if (q < points) stage_point<MODE, R, MESH>(g, P, LC, b, a, (long long)w0 * P3 + q, q);
+      }
     }
   }
 }

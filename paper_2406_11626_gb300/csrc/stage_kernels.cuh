@@ -160,17 +160,17 @@ struct StageBlocks {
   static constexpr int value = SHAPE == 1 ? base + 1 : SHAPE == 2 ? (base > 1 ? base - 1 : 1) : base;
 };
 
-// One interior point of the stage.
+// One interior point of the stage, its sums at place q of the derivative buffer.
 template <int MODE, class R, bool MESH>
 __device__ __forceinline__ void stage_point(const GridView &g, const Phys<R> &P, const LevelCoef<R> &LC,
-                                            const StageBufs &b, const StageArgs &a, long long i) {
+                                            const StageBufs &b, const StageArgs &a, long long i, long long q) {
   constexpr bool MIXED = std::is_same<R, float>::value;
   // the patch (32-bit division: every state index is below 2^31) only where its level matters;
   // a run-time index into the parameter array makes ptxas keep a local copy of the array
   const int lev = MESH ? patch_level(g, (int)i / (g.p * g.p * g.p)) : 0;
   const StencilCoef<double> C = MESH ? LC.C[lev] : LC.C[0];
   const StencilCoef<R> CR = MESH ? LC.CR[lev] : LC.CR[0];
-  const DerView<MIXED> N = der_view<MIXED>(g, b.der, b.mix, b.in, i);
+  const DerView<MIXED> N = der_view<MIXED>(g, b.der, b.mix, b.in, i, q);
   StageSink<MODE> sink{g, i, a};
   ccz4_rhs_point<double, R>(P, N, C, CR, sink);
   sink.finish();
@@ -223,7 +223,12 @@ __device__ __forceinline__ long long next_item(const GridView &g, int lane) {
   return (long long)__shfl_sync(0xffffffffu, q, 0);
 }
 
-// Every ghost cell and every interior point of every level.
+// First point of the window and the number of its points.
+__device__ __forceinline__ long long window_begin(const GridView &g) { return (long long)g.w0 * (g.p * g.p * g.p); }
+__device__ __forceinline__ long long window_points(const GridView &g) { return (long long)g.wn * (g.p * g.p * g.p); }
+
+// Every interior point of the window, of every level, and with the first
+// window every ghost cell.
 // Flat launch (QUEUE false): the first ghost_blocks blocks take the ghost
 // cells, the others one interior point per thread.
 // Queue launch (QUEUE, the grid sized to the resident blocks): each warp
@@ -238,22 +243,26 @@ __global__ void __launch_bounds__(128, (StageBlocks<R, SHAPE>::value))
       if (id < g.n_ghost) ghost_cell<MODE>(g, Pg, b, a, id);
       return;
     }
-    const long long i = (long long)(blockIdx.x - ghost_blocks) * blockDim.x + threadIdx.x;
-    if (i < g.n_points) stage_point<MODE, R, MESH>(g, P, LC, b, a, i);
+    const long long q = (long long)(blockIdx.x - ghost_blocks) * blockDim.x + threadIdx.x;
+    if (q < window_points(g)) stage_point<MODE, R, MESH>(g, P, LC, b, a, window_begin(g) + q, q);
     return;
   }
   const int lane = threadIdx.x & 31;
-  const long long gi = (g.n_ghost + 31) / 32;  // items of ghost cells
-  for (long long item = next_item(g, lane); (item - gi) * 32 < g.n_points; item = next_item(g, lane)) {
+  const long long gi = g.w0 == 0 ? (g.n_ghost + 31) / 32 : 0;  // items of ghost cells
+  for (long long item = next_item(g, lane); (item - gi) * 32 < window_points(g); item = next_item(g, lane)) {
     if (item < gi) {
       const long long id = item * 32 + lane;
       if (id < g.n_ghost) ghost_cell<MODE>(g, Pg, b, a, id);
     } else {
-      const long long i = (item - gi) * 32 + lane;
-      if (i < g.n_points) stage_point<MODE, R, MESH>(g, P, LC, b, a, i);
+      const long long q = (item - gi) * 32 + lane;
+      if (q < window_points(g)) stage_point<MODE, R, MESH>(g, P, LC, b, a, window_begin(g) + q, q);
     }
   }
 }
+
+// Points of the window, and the ghost cells that go with it.
+inline long long launch_points(const GridView &g) { return (long long)g.wn * g.p * g.p * g.p; }
+inline long long launch_ghosts(const GridView &g) { return g.w0 == 0 ? g.n_ghost : 0; }
 
 StencilCoef<double> coefs(double dx, const ccz4_params &P) {
   StencilCoef<double> C;
@@ -293,8 +302,8 @@ inline int stage_threads(long long points) { return points < 16LL * 152 * 128 ? 
 template <int MODE, class R, bool MESH, int SHAPE>
 cudaError_t launch_flat(const GridView &g, const ccz4_params &P, const StageBufs &b, const StageArgs &a,
                         cudaStream_t s) {
-  const int t = stage_threads(g.n_points);
-  const long long gb = (g.n_ghost + t - 1) / t, nb = (g.n_points + t - 1) / t;
+  const int t = stage_threads(launch_points(g));
+  const long long gb = (launch_ghosts(g) + t - 1) / t, nb = (launch_points(g) + t - 1) / t;
   if (gb + nb == 0) return cudaSuccess;
   algebra_kernel<MODE, R, MESH, false, SHAPE><<<(unsigned)(gb + nb), t, 0, s>>>(g, make_phys<R>(P), level_coefs<R>(g, P),
                                                                                 P, b, a, (int)gb);
@@ -305,7 +314,7 @@ template <int MODE, class R, bool MESH>
 cudaError_t launch_mode(const GridView &g, const ccz4_params &P, const StageBufs &b, const StageArgs &a,
                         cudaStream_t s) {
   if (g.queue) {
-    const long long items = (g.n_points + 31) / 32 + (g.n_ghost + 31) / 32, qb = queue_blocks<MODE, R, MESH>();
+    const long long items = (launch_points(g) + 31) / 32 + (launch_ghosts(g) + 31) / 32, qb = queue_blocks<MODE, R, MESH>();
     if (qb <= 0) return cudaErrorInvalidConfiguration;
     if (items == 0) return cudaSuccess;
     const long long blocks = qb < (items + 3) / 4 ? qb : (items + 3) / 4;

@@ -8,7 +8,8 @@
 // threads takes the derivatives of its next patch while the other
 // evaluates the points of the one before. The parts meet at a barrier per
 // patch; nothing waits on another block, and a block reads no derivatives but
-// its own. Streams do not do it: the same overlap by two streams and chunks
+// its own: it keeps those of two patches, in places of its own of the derivative
+// buffer. Streams do not do it: the same overlap by two streams and chunks
 // of patches took 37.8 ms (4 chunks) and 46.0 ms (16) as a graph, the blocks of
 // one kernel filling the SMs before the other's.
 //
@@ -45,6 +46,10 @@ cudaError_t launch_pair_mesh(const GridView &g, const ccz4_params &P, int stage,
 
 namespace {
 
+// The place that block `block` of `blocks` gives the derivatives of patch n: one of two, which take turns.
+// A patch's are overwritten two rounds later, when the barrier of the round between has shown them read.
+__device__ __forceinline__ int pair_place(int n, int block, int blocks) { return block + (n / blocks % 2) * blocks; }
+
 template <bool MESH>
 struct Split {
   // threads of the derivatives and of the algebra, and the registers each of them gets
@@ -69,8 +74,9 @@ __global__ void __launch_bounds__(Split<MESH>::threads, 1)
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(X::derive_regs));
 #pragma unroll 1
     for (int n = blockIdx.x; n < g.n_patches; n += gridDim.x) {
-      derive_edge<MESH ? FROM_MESH : FROM_LEVEL, X::derive, PF, false>(g, in, tile, mix, der, ls, fl, n, 0, 1, smem,
-                                                                            threadIdx.x, 1);
+      derive_edge<MESH ? FROM_MESH : FROM_LEVEL, X::derive, PF, false>(g, in, tile, mix, der, ls, fl, n,
+                                                                       pair_place(n, blockIdx.x, gridDim.x), 0, 1, smem,
+                                                                       threadIdx.x, 1);
       block_sync<X::threads>(2);
     }
   } else {
@@ -87,7 +93,8 @@ __global__ void __launch_bounds__(Split<MESH>::threads, 1)
       block_sync<X::threads>(2);  // patch n's derivatives are written
 #pragma unroll 1
       for (int q = tid; q < P3; q += X::algebra)
-        stage_point<MODE, double, MESH>(g, P, LC, b, a, (long long)n * P3 + q);
+        stage_point<MODE, double, MESH>(g, P, LC, b, a, (long long)n * P3 + q,
+                                        (long long)pair_place(n, blockIdx.x, gridDim.x) * P3 + q);
     }
   }
 }
