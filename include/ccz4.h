@@ -97,7 +97,7 @@ enum { CCZ4_PREC_FP64 = 0, CCZ4_PREC_MIXED = 1 };
    ACC: RK accumulator. RHS: output of ccz4_rhs. INI: Q_ini of the
    Sommerfeld condition (ghost part only is used). TILE: halo tiles. The
    state-shaped buffers (U, Y0, Y1, ACC, RHS, INI) share one layout.
-   ccz4_rhs and the step calls use TILE and MIX as scratch.
+   The step calls use TILE and MIX as scratch.
    MIX: [33][n_points] mixed second derivatives written by ccz4_fill_halos
    with the tiles: for g~_xx..g~_zz (slots 0..17), alpha (18..20),
    beta^x..beta^z (21..29) and phi (30..32), three slots each in the order
@@ -211,8 +211,8 @@ ccz4_status ccz4_fill_halos_for(ccz4_grid *g, int buf, const ccz4_params *P, voi
    by the listed relations and Eq. NR_foccz4_modified_ricci) plus the
    Kreiss-Oliger term of Eq. exa_fd4_ko summed over x, y, z, at every
    interior point, and the Sommerfeld right-hand side at every ghost cell.
-   Fills the halos of `in_buf` first (the TILE buffer is overwritten) and
-   writes `out_buf`. in_buf and out_buf must differ. */
+   Leaves the halos of `in_buf` in TILE and its mixed derivatives in MIX (as
+   ccz4_fill_halos_for) and writes `out_buf`. in_buf and out_buf must differ. */
 ccz4_status ccz4_rhs(ccz4_grid *g, const ccz4_params *P, int in_buf, int out_buf, void *stream);
 
 /* One stage s = 0..3 of classic RK4 (weights 1/6, 1/3, 1/3, 1/6; nodes

@@ -675,11 +675,16 @@ extern "C" ccz4_status ccz4_rhs(ccz4_grid *g, const ccz4_params *P, int in_buf, 
     return CCZ4_ERR_INVALID;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  return each_window(g, [&](const GridView &w) {
+  const ccz4_status st = each_window(g, [&](const GridView &w) {
     CUDA_TRY(derivatives(g, w, P, in_buf, s));
     CUDA_TRY(launch_rhs(w, *P, g->der, g->buf[CCZ4_BUF_MIX], g->buf[in_buf], ini_ptr(g), g->buf[out_buf], s));
     return CCZ4_OK;
   });
+  if (st != CCZ4_OK) return st;
+  // the halo tiles that a caller finds after this call (on a mesh the pass has left values of its own in them)
+  CUDA_TRY(launch_fill_halos(g->v, g->buf[in_buf], g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], s,
+                             P->precision == CCZ4_PREC_MIXED));
+  return CCZ4_OK;
 }
 
 static const int kStageIn[4] = {CCZ4_BUF_U, CCZ4_BUF_Y0, CCZ4_BUF_Y1, CCZ4_BUF_Y0};
