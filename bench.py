@@ -467,14 +467,6 @@ def time_first_order(C, I, cfg, K, W, stream):
     return out
 
 
-def stage_launches(g, precision):
-    """Kernel launches of one RK stage: the derivative pass and the algebra, one launch on large FP64 grids of 9^3
-    patches (pair_pays in csrc/ccz4_capi.cu)."""
-    n, rounds = g.n_patches, (g.n_patches + 151) // 152
-    pays = 117 * n >= (100 * rounds + 105) * 152 if g.n_levels > 1 else 13 * n >= (10 * rounds + 6) * 152
-    return 1 if precision == "fp64" and g.p == 9 and pays else 2
-
-
 def max_over_ranks(x, dist, device):
     """The largest value of x over the ranks (the slowest rank sets the job time)."""
     import torch
@@ -599,7 +591,7 @@ def run_gb300(args):
                 "fp64_flops_per_point_stage": fl["fp64"], "fp32_flops_per_point_stage": fl["fp32"],
                 "fp32_tflops": f32 / t_stage / 1e12,
                 "note": "frac = max(F64/P64, F32/P32) / kernel time", "peak_measured": peaks}
-    launches_per_stage = stage_launches(g, args.precision)
+    launches_per_stage = g.stage_launches(P)
     restrict_per_step = g.n_levels - 1
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": args.warmup,

@@ -242,6 +242,13 @@ ccz4_status ccz4_stage_buffers(int stage, int *in_buf, int *out_buf);
    between. */
 ccz4_status ccz4_step(ccz4_grid *g, const ccz4_params *P, double dt, int n_steps, void *stream);
 
+/* Kernel launches of one RK stage of ccz4_step and ccz4_step_graph with
+   parameters P on this grid as it is set (ccz4_set_launch,
+   ccz4_set_tuning), the restriction of a mesh apart: 2, derivatives and
+   algebra, for each window of the derivative buffer; 1 where both run in
+   one launch (CCZ4_LAUNCH_FUSED; FP64 on large grids of 9^3 patches). */
+ccz4_status ccz4_stage_launches(const ccz4_grid *g, const ccz4_params *P, int *launches);
+
 /* n_steps RK4 steps on U, like ccz4_step, replayed from a CUDA graph of one
    step. The graph is captured on a private stream the first time, and again
    whenever the parameters or dt differ from the captured ones; capturing

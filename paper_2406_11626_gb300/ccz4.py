@@ -82,6 +82,7 @@ def lib():
         "ccz4_step_graph": [vp, ctypes.POINTER(Params), ctypes.c_double, ctypes.c_int, vp],
         "ccz4_evolve_host": [vp, ctypes.POINTER(Params), ctypes.c_double, ctypes.c_int,
                              _dbl_p, _dbl_p, _dbl_p, _dbl_p, vp],
+        "ccz4_stage_launches": [vp, ctypes.POINTER(Params), ctypes.POINTER(ctypes.c_int)],
         "ccz4_enforce": [vp, ctypes.c_int, vp],
         "ccz4_constraints": [vp, ctypes.c_int, _dbl_p, _dbl_p, _dbl_p, vp],
         "ccz4_alloc_mesh": [ctypes.POINTER(MeshDesc), ctypes.POINTER(vp)],
@@ -392,6 +393,12 @@ class Grid:
 
     def step(self, P, dt, n_steps=1, stream=None):
         _check(lib().ccz4_step(self._h, ctypes.byref(P), float(dt), int(n_steps), _stream(stream)))
+
+    def stage_launches(self, P):
+        """Kernel launches of one RK stage of step and step_graph (ccz4_stage_launches)."""
+        n = ctypes.c_int()
+        _check(lib().ccz4_stage_launches(self._h, ctypes.byref(P), ctypes.byref(n)))
+        return n.value
 
     def step_graph(self, P, dt, n_steps=1, stream=None):
         _check(lib().ccz4_step_graph(self._h, ctypes.byref(P), float(dt), int(n_steps), _stream(stream)))

@@ -439,7 +439,10 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
   prepare_derive();
   prepare_constraints();
   if (v.p == 9) prepare_fused();
-  g->pair = v.p == 9 && pair_fits(v) && pair_pays(v.n_patches, mesh != nullptr) && prepare_pair(mesh != nullptr) == cudaSuccess;
+  if (v.p == 9 && pair_fits(v) && pair_pays(v.n_patches, mesh != nullptr)) {
+    g->pair = prepare_pair(mesh != nullptr) == cudaSuccess;
+    if (!g->pair) cudaGetLastError();  // two launches do as well (ccz4_stage_launches tells); no later call reports it
+  }
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     set_error("grid set-up failed: %s", cudaGetErrorString(e));
@@ -719,13 +722,31 @@ static ccz4_status two_launch_stage(ccz4_grid *g, const ccz4_params *P, int stag
 // launches, on large FP64 grids in the default launch mode and shape as one
 // (stage_pair.cuh, the same arithmetic), or (CCZ4_LAUNCH_FUSED) both in one
 // cooperative launch; the restriction after stage 3 stays a launch of its own.
+static bool one_launch(const ccz4_grid *g, const ccz4_params *P) {
+  return g->pair && !g->fused && !g->v.queue && g->v.stage_shape == 0 && P->precision != CCZ4_PREC_MIXED;
+}
 static ccz4_status step_stage(ccz4_grid *g, const ccz4_params *P, int stage, double dt, cudaStream_t s) {
-  const bool pair = g->pair && !g->fused && !g->v.queue && g->v.stage_shape == 0 && P->precision != CCZ4_PREC_MIXED;
+  const bool pair = one_launch(g, P);
   if (!g->fused && !pair) return two_launch_stage(g, P, stage, dt, false, s);
   const auto launch = pair ? launch_pair_stage : launch_fused_stage;
   CUDA_TRY(launch(g->v, *P, stage, dt, g->buf[CCZ4_BUF_TILE], g->buf[CCZ4_BUF_MIX], g->der, g->buf[kStageIn[stage]],
                   ini_ptr(g), g->buf[CCZ4_BUF_U], g->buf[CCZ4_BUF_ACC], g->buf[kStageOut[stage]], s));
   if (stage == 3 && g->v.n_levels > 1) return restrict_levels(g, g->buf[kStageOut[stage]], s);
+  return CCZ4_OK;
+}
+
+extern "C" ccz4_status ccz4_stage_launches(const ccz4_grid *g, const ccz4_params *P, int *launches) {
+  if (!g) {
+    set_error("grid is NULL");
+    return CCZ4_ERR_INVALID;
+  }
+  if (check_params(P)) return CCZ4_ERR_INVALID;
+  if (!launches) {
+    set_error("stage_launches: NULL launches");
+    return CCZ4_ERR_INVALID;
+  }
+  const int windows = g->v.wcap > 0 ? (g->v.n_patches + g->v.wcap - 1) / g->v.wcap : 0;
+  *launches = g->fused || one_launch(g, P) ? 1 : 2 * windows;
   return CCZ4_OK;
 }
 
