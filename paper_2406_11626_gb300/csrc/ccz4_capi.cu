@@ -103,9 +103,9 @@ extern "C" ccz4_status ccz4_set_allocator(ccz4_alloc_fn alloc, ccz4_dealloc_fn d
 // longer derivatives (interpolated halo points): 1.17 times and 1.05 of a round,
 // taken with equal parts (432 patches 4.33 ms in two launches, 4.77 in one; 2240
 // 19.8 and 18.9, 17.7 with the parts that meshes have now).
-static bool pair_pays(int patches, bool mesh) {
-  const long long rounds = (patches + 151) / 152;
-  return mesh ? 117LL * patches >= (100 * rounds + 105) * 152 : 13LL * patches >= (10 * rounds + 6) * 152;
+static bool pair_pays(int patches, int sms, bool mesh) {
+  const long long rounds = (patches + sms - 1) / sms;
+  return mesh ? 117LL * patches >= (100 * rounds + 105) * sms : 13LL * patches >= (10 * rounds + 6) * sms;
 }
 
 // Points of a derivative buffer: WINDOW_CAP at most (8.9 GB of 133 doubles a point, beside the 299 doubles that
@@ -149,12 +149,7 @@ int ccz4::fitting_window(const GridView &v, int slots) {
 }
 
 // Whether the buffer holds the two patches of each block that the one-launch stages keep (stage_pair.cuh).
-static bool pair_fits(const GridView &v) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return v.wcap >= v.n_patches || v.wcap >= 2 * sms;
-}
+static bool pair_fits(const GridView &v) { return v.wcap >= v.n_patches || v.wcap >= 2 * v.sms; }
 
 static size_t der_bytes(const GridView &v) {
   return sizeof(double) * (size_t)DER_SLOTS * (size_t)v.wcap * (size_t)(v.p * v.p * v.p);
@@ -368,6 +363,10 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
     return CCZ4_ERR_INVALID;
   }
   cudaGetDevice(&g->device);
+  if (cudaDeviceGetAttribute(&v.sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess) {
+    cudaGetLastError();
+    v.sms = 1;  // no device: the first allocation says so
+  }
   const long long state_len = (long long)NV * v.S;
   const long long lens[8] = {state_len, state_len, state_len, state_len, state_len,
                              d->bc == CCZ4_BC_SOMMERFELD ? state_len : 0,
@@ -439,7 +438,7 @@ static ccz4_status create_grid(const ccz4_grid_desc *d, const std::vector<int> &
   prepare_derive();
   prepare_constraints();
   if (v.p == 9) prepare_fused();
-  if (v.p == 9 && pair_fits(v) && pair_pays(v.n_patches, mesh != nullptr)) {
+  if (v.p == 9 && pair_fits(v) && pair_pays(v.n_patches, v.sms, mesh != nullptr)) {
     g->pair = prepare_pair(mesh != nullptr) == cudaSuccess;
     if (!g->pair) cudaGetLastError();  // two launches do as well (ccz4_stage_launches tells); no later call reports it
   }

@@ -115,6 +115,7 @@ struct GridView {
   // window of a derivative pass and the kernels that read it: patches w0 .. w0 + wn, whose sums stand at the
   // start of a derivative buffer of wcap patches
   int w0, wn, wcap;
+  int sms;                     // multiprocessors of the grid's device
 };
 
 // Level of patch n (0 on a single level).

@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(ONE_THREADS, 4)
 // a grid of few patches splits them until there are about two waves of
 // blocks (27 patches of 9^3: one block per field).
 int field_groups(const GridView &g, const FieldList &fl) {
-  const int want = 6 * 152;
+  const int want = 6 * g.sms;
   int k = g.wn > 0 ? (want + g.wn - 1) / g.wn : 1;
   k = k < 1 ? 1 : k;
   return k < fl.n ? k : fl.n;

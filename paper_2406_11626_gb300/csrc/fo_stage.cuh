@@ -153,7 +153,7 @@ cudaError_t launch_fo_interior(const GridView &g, const ccz4_params &P, const do
                                const double *ini, const FoStageArgs &a, cudaStream_t s) {
   const FoPhys F{make_phys<double>(P), P.mu};
   const long long points = (long long)g.wn * g.p * g.p * g.p, ghosts = g.w0 == 0 ? g.n_ghost : 0;
-  const int t = points < 16LL * 152 * 128 ? 32 : 128;  // a small grid spreads over the SMs in shares of 32 points
+  const int t = points < 16LL * g.sms * 128 ? 32 : 128;  // a small grid spreads over the SMs in shares of 32 points
   const long long gb = (ghosts + t - 1) / t, nb = (points + t - 1) / t;
   if (gb + nb == 0) return cudaSuccess;
   fo_interior_kernel<MODE, RED, AUX><<<(unsigned)(gb + nb), t, 0, s>>>(g, F, fo_coefs(g.dx, P.ko_eps), P, der, in, ini, a,

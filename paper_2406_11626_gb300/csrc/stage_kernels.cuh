@@ -297,12 +297,12 @@ long long queue_blocks() {
 // Threads of a block: 128, or on a small grid one warp, so that the points
 // spread over the SMs in shares of 32 (the FP64 pipe of the fullest SM sets
 // the time: 27^3 points are 154 blocks of 128, two of them on some SM).
-inline int stage_threads(long long points) { return points < 16LL * 152 * 128 ? 32 : 128; }
+inline int stage_threads(long long points, int sms) { return points < 16LL * sms * 128 ? 32 : 128; }
 
 template <int MODE, class R, bool MESH, int SHAPE>
 cudaError_t launch_flat(const GridView &g, const ccz4_params &P, const StageBufs &b, const StageArgs &a,
                         cudaStream_t s) {
-  const int t = stage_threads(launch_points(g));
+  const int t = stage_threads(launch_points(g), g.sms);
   const long long gb = (launch_ghosts(g) + t - 1) / t, nb = (launch_points(g) + t - 1) / t;
   if (gb + nb == 0) return cudaSuccess;
   algebra_kernel<MODE, R, MESH, false, SHAPE><<<(unsigned)(gb + nb), t, 0, s>>>(g, make_phys<R>(P), level_coefs<R>(g, P),

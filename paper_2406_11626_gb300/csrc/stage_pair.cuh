@@ -112,11 +112,7 @@ cudaError_t prepare_pair_one() {
 template <int MODE, bool MESH, int PF>
 cudaError_t launch_pair_one(const GridView &g, const ccz4_params &P, double *tile, double *mix, double *der,
                             const double *in, const double *ini, const StageArgs &a, cudaStream_t s) {
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  pair_kernel<MODE, MESH, PF><<<g.n_patches < sms ? g.n_patches : sms, Split<MESH>::threads, edge_smem_bytes(PF), s>>>(
+  pair_kernel<MODE, MESH, PF><<<g.n_patches < g.sms ? g.n_patches : g.sms, Split<MESH>::threads, edge_smem_bytes(PF), s>>>(
       g, make_phys<double>(P), level_coefs<double>(g, P), level_scale(g), P, all_fields(), tile, mix, der, in, ini, a);
   return cudaGetLastError();
 }
