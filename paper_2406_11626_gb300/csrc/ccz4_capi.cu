@@ -95,17 +95,16 @@ extern "C" ccz4_status ccz4_set_allocator(ccz4_alloc_fn alloc, ccz4_dealloc_fn d
   return CCZ4_OK;
 }
 
-// Whether FP64 stages with derivatives beside the algebra pay. In one launch
-// every 152 patches cost a round of 260 us a stage and the first patch's
-// derivatives another 0.6 of one; in two launches 152 patches cost 1.3 times as
-// much as a round (a step of 539 patches 4.97 ms in two launches, 4.73 in one; of
-// 1000 8.88 and 7.85; of 1728 15.0 and 13.0). Patches of a refined mesh have
-// longer derivatives (interpolated halo points): 1.17 times and 1.05 of a round,
-// taken with equal parts (432 patches 4.33 ms in two launches, 4.77 in one; 2240
-// 19.8 and 18.9, 17.7 with the parts that meshes have now).
+// Whether FP64 stages with derivatives beside the algebra pay. In one launch every round of patches, one a
+// multiprocessor, costs the same (152 patches: 256 us a stage on a level, 269 on a mesh) and the first patch's
+// derivatives 0.63 of a round, on a mesh, whose interpolated halo points make them longer, about one; in two
+// launches a round's patches cost 1.36 and 1.34 rounds. One RK4 step, two launches against one, smooth data: a
+// level of 294 patches 2.80 / 2.67 ms, 343 3.18 / 3.69, 504 4.63 / 4.74, 512 4.76 / 4.74, 576 5.29 / 4.76,
+// 648 5.94 / 5.77; a mesh of 432 4.39 / 4.41, 667 6.41 / 6.48, 702 6.82 / 6.63, 829 7.92 / 7.72, 945 9.22 /
+// 8.77, 1241 11.74 / 10.87, 2240 20.2 / 17.9.
 static bool pair_pays(int patches, int sms, bool mesh) {
   const long long rounds = (patches + sms - 1) / sms;
-  return mesh ? 117LL * patches >= (100 * rounds + 105) * sms : 13LL * patches >= (10 * rounds + 6) * sms;
+  return mesh ? 134LL * patches >= (100 * rounds + 100) * sms : 136LL * patches >= (100 * rounds + 63) * sms;
 }
 
 // Points of a derivative buffer: WINDOW_CAP at most (8.9 GB of 133 doubles a point, beside the 299 doubles that

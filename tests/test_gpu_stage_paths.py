@@ -43,6 +43,23 @@ def test_large_fp64_meshes_take_one_launch():
     g.close()
 
 
+@pytest.mark.parametrize("side,box,launches", [(6, (2, 2, 3), 2), (6, (2, 3, 3), 1), (8, (3, 3, 3), 1)])
+def test_the_line_between_the_launches_of_meshes(side, box, launches):
+    from paper_2406_11626_gb300 import ccz4 as C
+    lo = [(side - b) // 2 for b in box]
+    level, ijk = I.refined_mesh((side,) * 3, [(tuple(lo), tuple(a + b for a, b in zip(lo, box)))])
+    g = C.Grid(9, (side,) * 3, ijk, (-3.0,) * 3, 0.11, "periodic", level=level)
+    assert g.stage_launches(_params()) == launches
+    g.close()
+
+
+@pytest.mark.parametrize("npv,launches", [((7, 7, 6), 1), ((7, 7, 7), 2), ((8, 8, 8), 2), ((9, 8, 8), 1)])
+def test_the_line_between_the_launches_of_levels(npv, launches):
+    g = _level(9, npv)
+    assert g.stage_launches(_params()) == launches
+    g.close()
+
+
 @pytest.mark.parametrize("p,npv", [(9, (3, 3, 3)), (8, (8, 8, 8)), (12, (4, 4, 4)), (6, (8, 8, 8))])
 def test_other_grids_take_two(p, npv):
     g = _level(p, npv)
