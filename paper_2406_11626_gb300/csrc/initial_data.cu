@@ -19,6 +19,7 @@
 #include "../../include/ccz4_id.h"
 #include "ccz4_algebra.cuh"
 #include "fixed_stencil.cuh"
+#include "quotient.cuh"
 #include "ccz4_internal.cuh"
 
 struct ccz4_idsolver {
@@ -40,6 +41,7 @@ struct ccz4_idsolver {
 namespace {
 
 using ccz4::fx_laplacian;
+using ccz4::quotient;
 
 constexpr int ID_THREADS = 256;
 
@@ -69,21 +71,6 @@ __device__ __forceinline__ double recip(double d) {
   double r = ccz4::f2d_bits(__frcp_rn(ccz4::d2f_bits(d)));
   r = fma(r, fma(-d, r, 1.0), r);
   return fma(r, fma(-d, r, 1.0), r);
-}
-
-// num / den for normal den: the reciprocal of den's mantissa in FP32 with the
-// exponent put back by integer operations, then two steps q <- q + r (num -
-// den q), each in two FMAs: five FP64 operations, the result within an ulp,
-// over the whole range of exponents.
-__device__ __forceinline__ double quotient(double num, double den) {
-  const unsigned hi = (unsigned)__double2hiint(den), lo = (unsigned)__double2loint(den);
-  const unsigned e = (hi >> 20) & 0x7FFu;
-  const float m = __uint_as_float(0x3F800000u | ((hi & 0xFFFFFu) << 3) | (lo >> 29));  // [1, 2)
-  const unsigned f = __float_as_uint(__frcp_rn(m));                                    // (1/2, 1]
-  const double r = __hiloint2double((int)((hi & 0x80000000u) | ((f >> 3) + ((1919u - e) << 20))), (int)(f << 29));
-  double q = num * r;
-  q = fma(r, fma(-den, q, num), q);
-  return fma(r, fma(-den, q, num), q);
 }
 
 __global__ void __launch_bounds__(ID_THREADS) setup_kernel(int n, double L, double h, PunctureSet B,
