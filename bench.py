@@ -32,8 +32,9 @@ UNIT = "point-stages/s"
 # maximum SM clock (the nominal 1.25 TFLOP/s FP64 rate).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
-KERNEL_SOURCES = ("paper_2406_11626_gb300/csrc/stage_kernels.cuh", "paper_2406_11626_gb300/csrc/ccz4_algebra.cuh",
-                  "paper_2406_11626_gb300/csrc/ccz4_internal.cuh")
+KERNEL_SOURCES = tuple("paper_2406_11626_gb300/csrc/" + f for f in (
+    "stage_kernels.cuh", "stage_pair.cuh", "ccz4_algebra.cuh", "der_view.cuh", "derive.cuh", "derive_edge.cuh",
+    "fixed_stencil.cuh"))
 
 
 def measure_fma_peaks():
@@ -323,8 +324,8 @@ def _has_children(cfg, n):
 # GB300 arm
 # ----------------------------------------------------------------------------
 def load_traffic(n_points, precision="fp64", mesh=False):
-    """DRAM bytes of one stage-kernel launch over n_points, from the ncu
-    capture of the single-level instance of that precision recorded in
+    """DRAM bytes of one RK stage (all its launches) over n_points, from the
+    ncu capture of a single level in that precision recorded in
     profiles/traffic.json, scaled by points; None for a refined mesh, for a
     precision without a record, or once the kernel sources have changed."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
@@ -376,28 +377,12 @@ def init_state(C, I, cfg, g):
 
 
 def time_path(C, I, cfg, precision, K, W, stream, dist, clocks_index=None):
-    """Builds a grid, times the stage kernels of rk_stage over a few steps,
-    starts again, runs W warm-up and K timed RK4 steps; returns the grid,
-    the time of the K steps and the per-stage kernel times (ms)."""
+    """Builds a grid, runs W warm-up and K timed RK4 steps; returns the grid,
+    the parameters, the time of the K steps (ms) and the clocks."""
     import torch
     g = C.Grid.from_config(cfg)
     init_state(C, I, cfg, g)
     P = C.make_params(**cfg.params, precision=precision)
-    bufs = [C.stage_buffers(s) for s in range(4)]
-    n = min(K, 3)
-    kev = [[[torch.cuda.Event(enable_timing=True) for _ in range(2)] for _ in range(4)] for _ in range(n)]
-    for k in range(-1, n):  # one untimed step first
-        for s in range(4):
-            g.fill_halos(bufs[s][0], stream, P)
-            if k >= 0:
-                kev[k][s][0].record(stream)
-            g.rk_stage(P, s, cfg.dt, stream, fill=False)
-            if k >= 0:
-                kev[k][s][1].record(stream)
-    torch.cuda.synchronize()
-    stage_ms = [kev[k][s][0].elapsed_time(kev[k][s][1]) for k in range(n) for s in range(4)]
-
-    init_state(C, I, cfg, g)
     g.step(P, cfg.dt, W, stream)
     torch.cuda.synchronize()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -416,7 +401,7 @@ def time_path(C, I, cfg, precision, K, W, stream, dist, clocks_index=None):
         dist.barrier()
     clocks = clk.stop() if clk else None
     ms = e0.elapsed_time(e1)
-    return g, P, ms, stage_ms, clocks
+    return g, P, ms, clocks
 
 
 def time_graph(g, P, dt, K, W, stream, dist):
@@ -498,7 +483,7 @@ def run_gb300(args):
     cfg = bench_config(args)
     stream = torch.cuda.current_stream()
     K = args.steps
-    g, P, ms, stage_ms, clocks = time_path(C, I, cfg, args.precision, K, args.warmup, stream, dist, local)
+    g, P, ms, clocks = time_path(C, I, cfg, args.precision, K, args.warmup, stream, dist, local)
     ms = max_over_ranks(ms, dist, "cuda")
     value = job_rate(world, cfg.n_points, 4 * K, ms * 1e-3)
     out = g.constraints("U", raise_nonfinite=False)
@@ -526,8 +511,8 @@ def run_gb300(args):
     if not args.no_mixed and args.precision == "fp64":
         # the mixed path on the same workload, same steps; its state is
         # compared with the FP64 state after the same W + K steps
-        g64, _, _, _, _ = time_path(C, I, cfg, "fp64", K, args.warmup, stream, None)
-        gmx, _, ms_mx, stage_mx, _ = time_path(C, I, cfg, "mixed", K, args.warmup, stream, None)
+        g64, _, _, _ = time_path(C, I, cfg, "fp64", K, args.warmup, stream, None)
+        gmx, _, ms_mx, _ = time_path(C, I, cfg, "mixed", K, args.warmup, stream, None)
         a, _ = g64.download("U")
         b, _ = gmx.download("U")
         a = a.reshape(I.NV, -1)
@@ -539,7 +524,7 @@ def run_gb300(args):
         c64 = g64.constraints("U", raise_nonfinite=False)
         cmx = gmx.constraints("U", raise_nonfinite=False)
         flm = C.flops_per_point_stage("mixed")
-        t_stage_mx = sum(stage_mx) / len(stage_mx) * 1e-3
+        t_stage_mx = ms_mx / (4 * K) * 1e-3
         t_roof_mx = max(flm["fp64"] * cfg.n_points / (FP64_PEAK_TFLOPS * 1e12),
                         flm["fp32"] * cfg.n_points / (FP32_PEAK_TFLOPS * 1e12))
         mixed = {"value": world * cfg.n_points * 4 * K / (ms_mx * 1e-3), "unit": UNIT,
@@ -573,14 +558,15 @@ def run_gb300(args):
             dist.destroy_process_group()
         return 0
     fl = C.flops_per_point_stage(args.precision)
-    t_stage = sum(stage_ms) / len(stage_ms) * 1e-3
+    t_stage = ms / (4 * K) * 1e-3
     f64 = fl["fp64"] * cfg.n_points
     f32 = fl["fp32"] * cfg.n_points
     if args.precision == "fp64" or f32 == 0:
         roof = {"bound": "alu", "achieved": f64 / t_stage / 1e12, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": f64 / t_stage / 1e12 / FP64_PEAK_TFLOPS, "traffic": load_traffic(cfg.n_points, args.precision, g.n_levels > 1),
-                "kernel": "derivative pass and algebra_kernel (RHS + RK stage, ghost cells) of ccz4_rk_stage; stencil sums "
-                          "in integers count as the FP64 operations they replace",
+                "kernel": "a quarter of the timed step: derivatives, RHS + RK stage and ghost cells (pair_kernel, or the "
+                          "derivative pass and algebra_kernel), a mesh's restriction included; stencil sums in "
+                          "integers count as the FP64 operations they replace",
                 "flops_per_point_stage": fl["fp64"], "units_per_launch": cfg.n_points,
                 "peak_source": "FP64 pipe: 152 SMs x 2 FMA/clk x 2 flop x 2070 MHz",
                 "peak_measured": peaks}
@@ -590,7 +576,7 @@ def run_gb300(args):
                 "frac": t_roof / t_stage, "traffic": load_traffic(cfg.n_points, args.precision, g.n_levels > 1),
                 "fp64_flops_per_point_stage": fl["fp64"], "fp32_flops_per_point_stage": fl["fp32"],
                 "fp32_tflops": f32 / t_stage / 1e12,
-                "note": "frac = max(F64/P64, F32/P32) / kernel time", "peak_measured": peaks}
+                "note": "frac = max(F64/P64, F32/P32) / a quarter of the timed step", "peak_measured": peaks}
     launches_per_stage = g.stage_launches(P)
     restrict_per_step = g.n_levels - 1
     line = {
@@ -600,7 +586,7 @@ def run_gb300(args):
         "data": ("synthetic (Bowen-York binary data from the initial-data solve)" if args.workload == "binary"
                  else "synthetic (Brill-Lindquist puncture data generated in closed form)"),
         "config": workload_config(g, args.precision, K, args.workload),
-        "stage_kernel_ms": sum(stage_ms) / len(stage_ms),
+        "stage_kernel_ms": t_stage * 1e3,
         "roofline": roof,
         "clocks": clocks,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": 8 * I.NV * n_state,
@@ -611,7 +597,7 @@ def run_gb300(args):
                   "ms_per_step": ms_graph / K, "gpu_launches": (launches_per_stage * 4 + restrict_per_step) * K,
                   "how": "ccz4_step_graph: each RK4 step one replay of a captured CUDA graph (the derivative "
                          "passes, algebra kernels and restriction of the step), the same K steps after the "
-                         "launch-path run; value and the kernel times above come from the launch path"},
+                         "launch-path run; value and the stage times above come from the launch path"},
         "constraints_after": {"L2_H": out[0], "L2_M": out[1], "max_H": out[2], "nonfinite": out[4]},
     }
     if mixed is not None:

@@ -559,14 +559,16 @@ ccz4_status ccz4_tracers_free(ccz4_tracers *t);
 
 /* Launch shapes (a tuning choice; results are identical): the flat algebra
    kernel asks the default number of resident 128-thread blocks per SM
-   (CCZ4_STAGE_SHAPE_DEFAULT), one more (MORE_BLOCKS, fewer registers per
-   thread) or one fewer (FEWER_BLOCKS, more registers); SPLIT takes the
-   derivatives of all points before the algebra in a launch of its own, also on
-   the large FP64 grids of 9^3 patches where the default runs the two side by
-   side; the halo fill and the derivative pass (the pass: mixed precision, 9^3
-   patches) run 256 threads per patch (DEFAULT), 512 (WIDE) or 128 (NARROW), the fill with 8 independent loads per thread in its
-   gather or 16 (DEEP). Drops a captured step graph. CCZ4_ERR_INVALID for an
-   unknown shape. */
+   (CCZ4_STAGE_SHAPE_DEFAULT and SPLIT), one more (MORE_BLOCKS, fewer
+   registers per thread) or one fewer (FEWER_BLOCKS, more registers); every
+   shape but DEFAULT takes the derivatives of all points before the algebra
+   in a launch of its own, also on the large FP64 grids of 9^3 patches where
+   DEFAULT runs the two side by side (ccz4_stage_launches). The halo fill
+   runs 256 threads per patch (DEFAULT), 512 (WIDE) or 128 (NARROW) with 8
+   independent loads per thread in its gather, or 256 with 16 (DEEP); of a
+   step, whose derivative pass takes the place of the fill, these reach the
+   mixed precision on 9^3 patches only (the threads, not the loads). Drops a
+   captured step graph. CCZ4_ERR_INVALID for an unknown shape. */
 enum { CCZ4_STAGE_SHAPE_DEFAULT = 0, CCZ4_STAGE_SHAPE_MORE_BLOCKS = 1, CCZ4_STAGE_SHAPE_FEWER_BLOCKS = 2,
        CCZ4_STAGE_SHAPE_SPLIT = 3 };
 enum { CCZ4_FILL_SHAPE_DEFAULT = 0, CCZ4_FILL_SHAPE_WIDE = 1, CCZ4_FILL_SHAPE_DEEP = 2, CCZ4_FILL_SHAPE_NARROW = 3 };

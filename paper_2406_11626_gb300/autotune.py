@@ -11,9 +11,12 @@ The cost of a step depends on
   per RK stage;
 - the algebra kernel's launch shape: the default number of resident
   128-thread blocks per SM, one more (fewer registers per thread, more
-  warps to hide latency, more register spills) or one fewer (shape 3 is the
-  default again);
-- the derivative pass's launch shape: threads per patch block.
+  warps to hide latency, more register spills), one fewer, or the default
+  with the derivatives in a launch of their own (any shape but the default
+  takes that: on the large FP64 grids of 9^3 patches the default runs the
+  derivatives beside the algebra);
+- the derivative pass's launch shape: threads per patch block (mixed
+  precision and 9^3 patches; elsewhere the shapes run the same code).
 The tuner times one RK4 step (replays of the step captured as a CUDA graph,
 the way a production loop runs it, CUDA events) of each candidate on the
 workload itself and descends one coordinate at a time: first p and the
@@ -40,8 +43,8 @@ DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "ccz4_gb300", "a
 # the patch edges of the paper's patch-size study, plus the largest edge the fill kernel takes
 CANDIDATES = (6, 9, 12, 17, 18)
 LAUNCHES = ("flat", "queue", "fused")
-STAGE_SHAPES = (0, 1, 2, 3)   # default, one resident block more, one fewer, default
-FILL_SHAPES = (0, 1, 2, 3)    # 256 threads, 512, 256, 128
+STAGE_SHAPES = (0, 1, 2, 3)   # default, one resident block more, one fewer, derivatives in their own launch
+FILL_SHAPES = (0, 1, 2, 3)    # 256 threads, 512, 256, 128 (mixed precision, 9^3 patches)
 WORKLOADS = ("puncture144", "puncture3level", "binary")
 
 

@@ -313,10 +313,13 @@ class Grid:
         _check(lib().ccz4_set_launch(self._h, m))
 
     def set_tuning(self, stage_shape=0, fill_shape=0):
-        """Launch shapes of the flat algebra kernel (0 and 3 default, 1 one
-        resident block more, 2 one fewer) and of the derivative pass and the
-        halo fill (0 default, 1 512 threads, 2 16 loads per thread in the fill,
-        3 128 threads); results are identical."""
+        """Launch shapes of the flat algebra kernel (0 default, 1 one resident
+        block more, 2 one fewer, 3 default) and of the halo fill and, in the
+        mixed precision with 9^3 patches, the derivative pass (0 default, 1 512
+        threads, 2 16 loads per thread in the fill, 3 128 threads); results are
+        identical. Stage shapes 1 to 3 take the derivatives in a launch of their
+        own also on the large FP64 grids where the default runs them beside the
+        algebra (stage_launches)."""
         _check(lib().ccz4_set_tuning(self._h, int(stage_shape), int(fill_shape)))
 
     def restrict(self, buf="U", stream=None):

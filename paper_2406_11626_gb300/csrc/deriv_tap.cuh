@@ -1,10 +1,12 @@
-// Two-phase evaluation of the mixed-precision right-hand side from tiles (a host check of its templates).
+// Two-phase evaluation of the mixed-precision right-hand side from tiles. No kernel evaluates it this way (the
+// derivative pass has taken that place); tests/host_rhs.cu does, on the host, to check the stencil values that the
+// templates ask for against those of one phase.
 //
 // DerivTap stands in for the neighbourhood (Nbhd) of ccz4_rhs_point. In
 // the recording phase (TAP_RECORD) every stencil value the right-hand side
 // asks for -- first derivatives, pure second derivatives with their
 // Kreiss-Oliger sum, Kreiss-Oliger sums -- is computed from the tile as
-// before and also stored in this thread's slots in shared memory; run with
+// before and also stored in this point's slots; run with
 // a sink that discards the right-hand side, the algebra is dead code and
 // only the differencing remains. In the replay phase (TAP_REPLAY) the same
 // requests, made in the same order, read the slots back: the algebra runs

@@ -22,7 +22,8 @@ __global__ void __launch_bounds__(EdgeShape<PF>::threads, EdgeShape<PF>::blocks)
                                                      blockIdx.y, gridDim.y, smem, threadIdx.x, 0);
 }
 
-// One field per block, 9^3 patches: small grids, whose every block is resident at once.
+// One field per block, 9^3 patches: small grids. Four blocks of 54 KB fit an SM, so 24 patches are one wave of
+// 600 blocks (27 are 675, a wave and a tenth).
 constexpr int ONE_THREADS = 256;
 template <int SRC>
 __global__ void __launch_bounds__(ONE_THREADS, 4)
@@ -35,8 +36,9 @@ __global__ void __launch_bounds__(ONE_THREADS, 4)
 
 // Field groups per patch. A block's set-up (the source table) is shared by
 // the fields it takes, so a grid of many patches gives each block all fields;
-// a grid of few patches splits them until there are about two waves of
-// blocks (27 patches of 9^3: one block per field).
+// a grid of few patches splits them into about six blocks an SM, whatever number
+// of them is resident (9^3: three or four, 12^3: one, so that 140 patches of 12^3
+// in seven groups are 6.4 waves).
 int field_groups(const GridView &g, const FieldList &fl) {
   const int want = 6 * g.sms;
   int k = g.wn > 0 ? (want + g.wn - 1) / g.wn : 1;

@@ -7,14 +7,14 @@
 // the mixed derivatives are integer sums too.
 //
 // What bounds it: instruction issue and the latency of its phases (three
-// barriers a field). Per point 17 k thread instructions against 20 k of the
-// general pass and 91 FP64 operations (conversions and the scale of the mixed
-// derivatives; 33 without the conversions) against 300, so that it can run
-// beside the algebra, which needs all of the FP64 pipe (stage_pair.cuh). As a
-// launch of its own it takes, against the general pass with a fixed edge, one
-// RK4 step of 140 patches of 12^3 from 3.51 to 3.36 ms, of 1000 patches of 6^3
-// from 3.56 to 3.09 ms; with 9^3 patches, where the general pass has a fixed
-// edge too, the two are within 3 % of one another either way.
+// barriers a field; ncu, 1000 patches of 9^3: 0.78 ms, issue slots 52 % busy, the
+// integer pipe 66 %). 22.4 k thread instructions a point, 192 on the FP64 pipe
+// (143 without the conversions; the general pass has 286 for the sums of 14 fields
+// and all mixed derivatives), so that it can run beside the algebra, which needs
+// all of that pipe (stage_pair.cuh). As a launch of its own it took, against the
+// general pass, one RK4 step of 140 patches of 12^3 from 3.51 to 3.36 ms, of 1000
+// patches of 6^3 from 3.56 to 3.09 ms; with 9^3 patches, where the general pass
+// has a fixed edge too, the two were within 3 % of one another either way.
 #pragma once
 
 #include "derive.cuh"
@@ -115,8 +115,8 @@ constexpr size_t edge_smem_bytes(int p, bool one = false) {
 static_assert(4 * 15 * 15 * 15 <= 8 * (EDGE_EZ(9) + EDGE_EY(9)), "a source table in the place of Ez and Ey");
 
 // The fields group, group + groups, ... of the list, of patch n, into the place
-// of patch `at_patch` of the derivative buffer, by the THREADS threads tid (whole warps) that share barrier bar. tile: the tile buffer;
-// interpolated halo points of a mesh pass through it.
+// of patch `at_patch` of the derivative buffer, by the THREADS threads tid (whole
+// warps) that share barrier bar. tile: the tile buffer; interpolated halo points of a mesh pass through it.
 template <int SRC, int THREADS, int PF, bool CVT, bool ONE = false>
 __device__ __forceinline__ void derive_edge(const GridView &g, const double *__restrict__ src, double *tile,
                                             double *__restrict__ mix, double *__restrict__ der, const LevelScale &ls,

@@ -2,8 +2,10 @@
 // blocks first take the derivatives of all patches (one patch per block at
 // a time, the pass of derive.cuh), wait for one another at a grid-wide barrier,
 // then evolve the Sommerfeld ghost cells and the interior points (items of 32
-// per warp, strided over the grid). This is the paper's enclave
-// batching taken to a whole stage: every patch of every level in one task.
+// per warp, strided over the grid); on a grid with more patches than its
+// derivative buffer holds, window after window, with a barrier between. This is
+// the paper's enclave batching taken to a whole stage: every patch of every level
+// in one task.
 // Compiled for 9^3 patches (the derivative pass's instance for that edge) and
 // the RK stages; the restriction after a step stays its own launch.
 //
