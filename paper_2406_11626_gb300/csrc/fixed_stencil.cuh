@@ -6,18 +6,16 @@
 // an FP64 evaluation of the same stencil rounds every partial sum.
 //
 // The unit of a sum is 2^-56 of (the power of two of) the largest value that
-// the sum itself has: the centre and the four neighbours of its axis for a
-// first and a pure second derivative, all 19 values for the dissipation. Values
+// the sum itself has: the four neighbours of its axis for a first derivative,
+// the centre too for a second, all 19 values for the dissipation. Values
 // within a factor of sixteen of the largest are held exactly; of a smaller one
 // the bits below the unit are dropped, toward zero, so that the sums keep the
 // symmetries of FP64's: f -> -f and a reflection change the sign of a result and
 // no bit, and zeros, of either sign, add nothing. A dropped bit costs up to 8
 // (first derivative) or 16 (second) units; the rounding of an FP64 difference at
-// the scale of the largest value costs as much as 8 of them. Where a
-// derivative's centre exceeds its four neighbours by more than two binades (an
-// isolated point), which would spend the guard bits, where the largest value's
-// biased exponent is FX_TOP or more (infinities and NaN too), or below FX_FLOOR,
-// the point is evaluated in FP64.
+// the scale of the largest value costs as much as 8 of them. Where the largest
+// value's biased exponent is FX_TOP or more (infinities and NaN too), or that of a
+// sum not all of zeros is below FX_FLOOR, the point is evaluated in FP64.
 //
 // Against extended precision, field by field on the puncture and gauge-wave
 // data, the root-mean-square error of the second derivatives and of the
@@ -199,8 +197,6 @@ __host__ __device__ __forceinline__ double fx_return(int64_t v, unsigned unit) {
 #endif
   return fx_out<K, true>(v, unit);
 }
-// The binades by which a derivative's centre may exceed its neighbours.
-constexpr unsigned FX_SPIKE = 2;
 
 // A zero that the compiler cannot move or foresee: what depends on it is not evaluated ahead of the
 // branch it stands in.
@@ -237,7 +233,9 @@ __host__ __device__ __forceinline__ void fx_point_fp64(const int64_t *w, const E
 }
 
 // The stencil sums of the point at w, ex (neighbours at multiples of st[k] along axis k): out[0..2]
-// first derivatives, out[3] dissipation, out[4..6] pure second derivatives.
+// first derivatives, out[3] dissipation, out[4..6] pure second derivatives. The neighbours of an axis are
+// brought to the unit of their own largest; their part of a second derivative and of the dissipation is
+// truncated to the unit of that sum where that is larger.
 // Magnitudes in units: 18 x 2^57 for a first, 64 x (2^57 - 1) for a second derivative; the dissipation
 // 3 x + s3 - 60 c = 4 (x - 15 c) + (s3 - x), x the sum of 5 t1 - 2 t2 over the axes, whose parts stay below
 // 57 x 2^57 and 48 x 2^57, is formed as it is or, where that is too large, as its quarter with the two bits
@@ -245,7 +243,7 @@ __host__ __device__ __forceinline__ void fx_point_fp64(const int64_t *w, const E
 template <bool SECOND, bool CVT, class E>
 __host__ __device__ __forceinline__ void fx_point(const int64_t *w, const E *ex, const int (&st)[3], double *out) {
   const unsigned e0 = ex[0];
-  unsigned ep[3][3], em[3][3], u[3], top = e0, least = ~0u, low = ~0u;  // least: smallest of the axes' neighbours
+  unsigned ep[3][3], em[3][3], u[3], top = e0, low = e0 - 1u;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
 #pragma unroll
@@ -253,18 +251,17 @@ __host__ __device__ __forceinline__ void fx_point(const int64_t *w, const E *ex,
       ep[k][j] = ex[(j + 1) * st[k]];
       em[k][j] = ex[-(j + 1) * st[k]];
     }
-    const unsigned a = fx_max(fx_max(ep[k][0], em[k][0]), fx_max(ep[k][1], em[k][1]));
-    u[k] = fx_max(a, e0);
-    least = a < least ? a : least;
-    low = u[k] < low ? u[k] : low;
+    u[k] = fx_max(fx_max(ep[k][0], em[k][0]), fx_max(ep[k][1], em[k][1]));
+    low = u[k] - 1u < low ? u[k] - 1u : low;  // (zeros do not count)
     top = fx_max(top, fx_max(u[k], fx_max(ep[k][2], em[k][2])));
+    u[k] = fx_max(u[k], FX_FIRST);  // shifts zeros out
   }
   if (top == 0) {
 #pragma unroll
     for (int q = 0; q < (SECOND ? 7 : 4); ++q) out[q] = 0.0;
     return;
   }
-  if (top > FX_LAST || low < FX_FIRST || e0 > least + FX_SPIKE) {
+  if (top > FX_LAST || top < FX_FIRST || low < FX_FIRST - 1u) {
     fx_point_fp64<SECOND>(w, ex, st, out);
     return;
   }
@@ -272,16 +269,16 @@ __host__ __device__ __forceinline__ void fx_point(const int64_t *w, const E *ex,
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const int s = st[k];
-    const unsigned unit = (u[k] << 21) | FX_LOW;
     const int64_t p1 = fx_shifted(w[s], u[k] - ep[k][0]), m1 = fx_shifted(w[-s], u[k] - em[k][0]);
     const int64_t p2 = fx_shifted(w[2 * s], u[k] - ep[k][1]), m2 = fx_shifted(w[-2 * s], u[k] - em[k][1]);
     const int64_t t1 = p1 + m1, t2 = p2 + m2;
     x += fx_div2(t1 * 5 - t2 * 2, top - u[k]);
     if (SECOND) {
-      const int64_t q = 2 * fx_shifted(w[0], u[k] - e0);
-      out[4 + k] = fx_return<5, CVT>((t1 - q) * 16 - (t2 - q), unit);
+      const unsigned v = fx_max(u[k], e0);
+      const int64_t q = 2 * fx_shifted(w[0], v - e0);
+      out[4 + k] = fx_return<5, CVT>(fx_div2(t1 * 16 - t2, v - u[k]) - q * 15, (v << 21) | FX_LOW);
     }
-    out[k] = fx_out<5>((p1 - m1) * 8 - (p2 - m2), unit);
+    out[k] = fx_out<5>((p1 - m1) * 8 - (p2 - m2), (u[k] << 21) | FX_LOW);
     s3 += fx_shifted(w[3 * s], top - ep[k][2]) + fx_shifted(w[-3 * s], top - em[k][2]);
   }
   const int64_t y = x - 15 * fx_shifted(w[0], top - e0), r = s3 - x, v = y + (r >> 2);
@@ -292,9 +289,9 @@ __host__ __device__ __forceinline__ void fx_point(const int64_t *w, const E *ex,
 // The first-derivative sum along stride s alone, as fx_point takes it.
 template <class E>
 __host__ __device__ __forceinline__ double fx_first_sum(const int64_t *w, const E *ex, int s) {
-  const unsigned a = ex[s], b = ex[-s], c = ex[2 * s], d = ex[-2 * s], e0 = ex[0];
-  const unsigned n = fx_max(fx_max(a, b), fx_max(c, d)), u = fx_max(n, e0);
-  if (u > FX_LAST || u < FX_FIRST || e0 > n + FX_SPIKE) {
+  const unsigned a = ex[s], b = ex[-s], c = ex[2 * s], d = ex[-2 * s];
+  const unsigned u = fx_max(fx_max(a, b), fx_max(c, d));
+  if (u > FX_LAST || u < FX_FIRST) {
     const int z = here_zero();
     w += z;
     ex += z;
