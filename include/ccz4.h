@@ -137,7 +137,7 @@ typedef struct ccz4_grid ccz4_grid;
    "Spatial Discretisation": p^3 patches with K = 3 halo layers). The
    descriptor and its ijk array are copied. Buffers start zeroed. Besides
    the CCZ4_BUF_* buffers a grid holds a derivative buffer of 133 doubles a
-   point for all its points, for a part of them on a grid of more than 2^23
+   point for all its points, for a part of them on a grid of more than 2^24
    points (or than the environment variable CCZ4_DERIVE_POINTS says) and
    where memory is short; results do not depend on it. On error *out is set
    to NULL. */

@@ -107,13 +107,14 @@ static bool pair_pays(int patches, int sms, bool mesh) {
   return mesh ? 134LL * patches >= (100 * rounds + 100) * sms : 136LL * patches >= (100 * rounds + 63) * sms;
 }
 
-// Points of a derivative buffer: WINDOW_CAP at most (8.9 GB of 133 doubles a point, beside the 299 doubles that
+// Points of a derivative buffer: WINDOW_CAP at most (17.9 GB of 133 doubles a point, beside the 299 doubles that
 // a point of a grid of 9^3 patches takes otherwise), less where memory is short, so that the buffer does not bound
 // the size of a grid. A larger grid takes its derivatives and what reads them in equal windows, each of which
 // costs a launch's ramp and last wave twice a stage: a mixed step of 144^3 15.0 ms in one window, 15.7 in two,
-// 16.3 in three; of three levels of 5.5 M points 28.6, 29.2 in two, 30.4 in four. FP64 stages in one launch need
-// two patches a block of the buffer and no windows. CCZ4_DERIVE_POINTS sets another bound.
-constexpr long long WINDOW_CAP = 1ll << 23;
+// 16.3 in three; of three levels of 5.5 M points 28.6, 29.2 in two, 30.4 in four; of the four-level binary's
+// 14.8 M 75.7, 77.1 in two. FP64 stages in one launch need two patches a block of the buffer and no windows.
+// CCZ4_DERIVE_POINTS sets another bound.
+constexpr long long WINDOW_CAP = 1ll << 24;
 
 // Windows of k * unit patches, unit the least number whose points fill whole blocks of the monitors' sums.
 static int window_unit(const GridView &v) {
