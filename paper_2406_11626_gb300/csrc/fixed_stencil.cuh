@@ -117,20 +117,34 @@ __device__ __forceinline__ double fx_out_cvt(long long v, unsigned unit) {
 }
 #endif
 
-// A value that the compiler may not evaluate ahead of the branch this stands in.
-__host__ __device__ __forceinline__ double fx_here(double u) {
+// A zero that the compiler cannot move or foresee: what depends on it is not evaluated ahead of the
+// branch it stands in.
+__host__ __device__ __forceinline__ int here_zero() {
+  int z = 0;
 #ifdef __CUDA_ARCH__
-  asm volatile("" : "+d"(u));
+  asm volatile("mov.u32 %0, 0;" : "=r"(z));
 #endif
-  return u;
+  return z;
 }
 
-// 8 (a1 - b1) - (a2 - b2): the first-derivative stencil of the values at +1, -1, +2, -2
-__host__ __device__ __forceinline__ double fx_first(double a1, double b1, double a2, double b2) {
-  const unsigned u = fx_unit(fx_max(fx_max(fx_key(a1), fx_key(b1)), fx_max(fx_key(a2), fx_key(b2))));
-  if (fx_outside(u)) return fma(8.0, fx_here(a1) - b1, -(fx_here(a2) - b2));
+// 8 (a1 - b1) - (a2 - b2): the first-derivative stencil of the values at +1, -1, +2, -2, all of them
+// zero or within the integer range (not fx_wild).
+__host__ __device__ __forceinline__ double fx_first_in(double a1, double b1, double a2, double b2) {
+  const unsigned key = fx_max(fx_max(fx_key(a1), fx_key(b1)), fx_max(fx_key(a2), fx_key(b2)));
+  const unsigned u = fx_unit(fx_max(key, FX_FLOOR << 21));  // shifts zeros out
   const int64_t d1 = fx_in(a1, u) - fx_in(b1, u), d2 = fx_in(a2, u) - fx_in(b2, u);
   return fx_out<4>(d1 * 8 - d2, u);
+}
+__host__ __device__ __forceinline__ bool fx_wild(double u) {
+  const uint64_t b = fx_bits(u);
+  const unsigned hi = (unsigned)(b >> 32) & 0x7FFFFFFFu;
+  return hi - (FX_FLOOR << 20) >= (FX_TOP - FX_FLOOR) << 20 && (hi | (unsigned)b) != 0;
+}
+// The same of any values. (The compiler predicates the FP64 side: its operations take their slots of the
+// FP64 pipe whether or not a thread needs them.)
+__host__ __device__ __forceinline__ double fx_first(double a1, double b1, double a2, double b2) {
+  const unsigned u = fx_unit(fx_max(fx_max(fx_key(a1), fx_key(b1)), fx_max(fx_key(a2), fx_key(b2))));
+  return fx_outside(u) ? fma(8.0, a1 - b1, -(a2 - b2)) : fx_first_in(a1, b1, a2, b2);
 }
 
 // The FP64 side of fx_laplacian: out of line, or the compiler evaluates it ahead of the branch.
@@ -196,16 +210,6 @@ __host__ __device__ __forceinline__ double fx_return(int64_t v, unsigned unit) {
   if constexpr (CVT) return fx_out_cvt<K>(v, unit);
 #endif
   return fx_out<K, true>(v, unit);
-}
-
-// A zero that the compiler cannot move or foresee: what depends on it is not evaluated ahead of the
-// branch it stands in.
-__host__ __device__ __forceinline__ int here_zero() {
-  int z = 0;
-#ifdef __CUDA_ARCH__
-  asm volatile("mov.u32 %0, 0;" : "=r"(z));
-#endif
-  return z;
 }
 
 // The stencil sums of fx_point in FP64. Inline: a call's registers would be its callee's choice.
