@@ -96,15 +96,15 @@ extern "C" ccz4_status ccz4_set_allocator(ccz4_alloc_fn alloc, ccz4_dealloc_fn d
 }
 
 // Whether FP64 stages with derivatives beside the algebra pay. In one launch every round of patches, one a
-// multiprocessor, costs the same (152 patches: 256 us a stage on a level, 269 on a mesh) and the first patch's
-// derivatives 0.63 of a round, on a mesh, whose interpolated halo points make them longer, about one; in two
-// launches a round's patches cost 1.36 and 1.34 rounds. One RK4 step, two launches against one, smooth data: a
-// level of 294 patches 2.80 / 2.67 ms, 343 3.18 / 3.69, 504 4.63 / 4.74, 512 4.76 / 4.74, 576 5.29 / 4.76,
-// 648 5.94 / 5.77; a mesh of 432 4.39 / 4.41, 667 6.41 / 6.48, 702 6.82 / 6.63, 829 7.92 / 7.72, 945 9.22 /
-// 8.77, 1241 11.74 / 10.87, 2240 20.2 / 17.9.
+// multiprocessor, costs the same (152 patches: 237 us a stage on a level, 258 on a mesh) and the first patch's
+// derivatives 0.70 of a round, on a mesh, whose interpolated halo points make them longer, 1.07; in two launches a
+// round's patches cost 1.44 rounds and 0.15 beside them, on a mesh 1.36 and 0.3. One RK4 step, two launches
+// against one: a level of 252 patches 2.44 / 2.57 ms, 294 2.81 / 2.59, 343 3.19 / 3.51, 384 3.60 / 3.52, 504 4.66
+// / 4.46, 648 5.98 / 5.41, 1000 9.13 / 7.32; a mesh of 280 2.97 / 3.27, 341 3.48 / 4.15, 432 4.34 / 4.16, 667
+// 6.32 / 6.08, 945 9.12 / 8.14, 2240 20.0 / 16.6.
 static bool pair_pays(int patches, int sms, bool mesh) {
   const long long rounds = (patches + sms - 1) / sms;
-  return mesh ? 134LL * patches >= (100 * rounds + 100) * sms : 136LL * patches >= (100 * rounds + 63) * sms;
+  return mesh ? 136LL * patches >= (100 * rounds + 77) * sms : 144LL * patches >= (100 * rounds + 55) * sms;
 }
 
 // Points of a derivative buffer: WINDOW_CAP at most (17.9 GB of 133 doubles a point, beside the 299 doubles that

@@ -19,12 +19,14 @@
 // 31.7, two blocks of 256 + 128 (56, 128) 33.3, 384 + 384 (48, 112) 31.6: the
 // algebra wants 12 warps to cover its latency, the derivatives 12 to keep up. With
 // their conversions to FP64 in integers (CVT false) 30.4; with an algebra of 100
-// operations less 28.5; with stencil sums in units of their own (fixed_stencil.cuh)
-// 28.65, and (40, 120) 29.3, (56, 104) 28.8. On a mesh the derivatives are the
-// longer part (interpolated halo points): two levels of 2240 patches 18.9 ms with
-// 384 + 384, 18.7 with 512 + 384, 17.7 with 512 + 256 (48, 144), 17.8 with 640 +
-// 256; now 18.1, and (56, 128) 18.7. What bounds it: the FP64 pipe (1215 operations
-// a point are 23.1 ms) and the stalls that the algebra's warps leave open.
+// operations less 28.5; with no FP64 operation of theirs issued in vain 26.46, and
+// 26.27 with (40, 120), 26.5 with (56, 104), 38.8 with 256 + 384 (56, 120). On a mesh
+// the derivatives are the longer part (interpolated halo points): two levels of 2240
+// patches 18.9 ms with 384 + 384, 18.7 with 512 + 384, 17.7 with 512 + 256 (48, 144),
+// 17.8 with 640 + 256; of late 16.7, and (40, 160) 16.8, (56, 128) 17.1, 384 + 384 (48,
+// 112) 17.5. What bounds it: the FP64 pipe (1187
+// operations a point, 22.5 of the 26.2 ms) and the stalls that the algebra's warps
+// leave open.
 //
 // Mixed precision keeps two launches: there the derivative pass is the longer
 // part and wants the whole SM (15.0 ms against 15.2 at best).
@@ -54,7 +56,7 @@ template <bool MESH>
 struct Split {
   // threads of the derivatives and of the algebra, and the registers each of them gets
   static constexpr int derive = MESH ? 512 : 384, algebra = MESH ? 256 : 384, threads = derive + algebra;
-  static constexpr int derive_regs = 48, algebra_regs = MESH ? 144 : 112;
+  static constexpr int derive_regs = MESH ? 48 : 40, algebra_regs = MESH ? 144 : 120;
   // Registers a thread of the launch (what 65536 leave for its threads, in steps
   // of 8). The parts may not ask for more in sum: they would wait for ever.
   static constexpr int regs = 65536 / threads / 8 * 8;

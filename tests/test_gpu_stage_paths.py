@@ -43,7 +43,7 @@ def test_large_fp64_meshes_take_one_launch():
     g.close()
 
 
-@pytest.mark.parametrize("side,box,launches", [(6, (2, 2, 3), 2), (6, (2, 3, 3), 1), (8, (3, 3, 3), 1)])
+@pytest.mark.parametrize("side,box,launches", [(5, (2, 2, 2), 2), (6, (2, 2, 2), 1), (8, (3, 3, 3), 1)])
 def test_the_line_between_the_launches_of_meshes(side, box, launches):
     from paper_2406_11626_gb300 import ccz4 as C
     lo = [(side - b) // 2 for b in box]
@@ -53,7 +53,7 @@ def test_the_line_between_the_launches_of_meshes(side, box, launches):
     g.close()
 
 
-@pytest.mark.parametrize("npv,launches", [((7, 7, 6), 1), ((7, 7, 7), 2), ((8, 8, 8), 2), ((9, 8, 8), 1)])
+@pytest.mark.parametrize("npv,launches", [((6, 6, 7), 2), ((7, 7, 6), 1), ((7, 7, 7), 2), ((6, 8, 8), 1)])
 def test_the_line_between_the_launches_of_levels(npv, launches):
     g = _level(9, npv)
     assert g.stage_launches(_params()) == launches
