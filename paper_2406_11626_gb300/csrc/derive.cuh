@@ -27,11 +27,11 @@ namespace ccz4 {
 namespace {
 
 // The stencil sums of the point at w, ex in a tile of edge T: out[0..2] first
-// derivatives, out[3] dissipation, out[4..6] pure second derivatives. CVT: as fx_return.
-template <bool SECOND, bool CVT = true, class E>
+// derivatives, out[3] dissipation, out[4..6] pure second derivatives. CVT, FIRST_CVT: as fx_point.
+template <bool SECOND, bool CVT = true, bool FIRST_CVT = false, class E>
 __device__ __forceinline__ void point_sums(const int64_t *w, const E *ex, int T, double *out) {
   const int st[3] = {1, T, T * T};
-  fx_point<SECOND, CVT>(w, ex, st, out);
+  fx_point<SECOND, CVT, FIRST_CVT>(w, ex, st, out);
 }
 
 // The same in FP32 from split pairs (mixed precision), whose FP32 pipe is
@@ -266,7 +266,9 @@ __device__ __forceinline__ void derive_patch(const GridView &g, const double *__
         O o[7];
         if constexpr (std::is_same<O, float>::value)
           point_sums<SECOND>(reinterpret_cast<const float2 *>(ts) + c0, ex, T, o);
-        else point_sums<SECOND>(reinterpret_cast<const int64_t *>(ts) + c0, ex + c0, T, o);
+        // the 58 fields leave the FP64 pipe to 3 %: 25 steps at 54^3 106.4 ms with their first derivatives returned in
+        // integers, 104.5 by the conversion instruction; the 25 do not (monitors 5.84 against 5.88)
+        else point_sums<SECOND, true, NF != NV>(reinterpret_cast<const int64_t *>(ts) + c0, ex + c0, T, o);
         O *a, *b;
         if constexpr (std::is_same<O, float>::value) {
           a = fd + q;

@@ -8,10 +8,10 @@
 //
 // What bounds it: instruction issue and the latency of its phases (three
 // barriers a field; ncu, 1000 patches of 9^3: 0.78 ms, issue slots 52 % busy, the
-// integer pipe 66 %). 22.4 k thread instructions a point, 192 on the FP64 pipe
-// (143 without the conversions; the general pass has 286 for the sums of 14 fields
-// and all mixed derivatives), so that it can run beside the algebra, which needs
-// all of that pipe (stage_pair.cuh). As a launch of its own it took, against the
+// integer pipe 65 %). 22 k thread instructions a point, 91 on the FP64 pipe (33
+// without the conversions; the general pass has 286 for the sums of 14 fields and
+// all mixed derivatives), so that it can run beside the algebra, which needs all of
+// that pipe (stage_pair.cuh). As a launch of its own it took, against the
 // general pass, one RK4 step of 140 patches of 12^3 from 3.51 to 3.36 ms, of 1000
 // patches of 6^3 from 3.56 to 3.09 ms; with 9^3 patches, where the general pass
 // has a fixed edge too, the two were within 3 % of one another either way.

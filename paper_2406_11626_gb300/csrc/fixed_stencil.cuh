@@ -239,12 +239,13 @@ __host__ __device__ __forceinline__ void fx_point_fp64(const int64_t *w, const E
 // The stencil sums of the point at w, ex (neighbours at multiples of st[k] along axis k): out[0..2]
 // first derivatives, out[3] dissipation, out[4..6] pure second derivatives. The neighbours of an axis are
 // brought to the unit of their own largest; their part of a second derivative and of the dissipation is
-// truncated to the unit of that sum where that is larger.
+// truncated to the unit of that sum where that is larger. FIRST_CVT: first derivatives return as the others do,
+// with CVT (for a pass that leaves the FP64 pipe idle).
 // Magnitudes in units: 18 x 2^57 for a first, 64 x (2^57 - 1) for a second derivative; the dissipation
 // 3 x + s3 - 60 c = 4 (x - 15 c) + (s3 - x), x the sum of 5 t1 - 2 t2 over the axes, whose parts stay below
 // 57 x 2^57 and 48 x 2^57, is formed as it is or, where that is too large, as its quarter with the two bits
 // below kept as one (they can only tell which side of a tie it is).
-template <bool SECOND, bool CVT, class E>
+template <bool SECOND, bool CVT, bool FIRST_CVT = false, class E>
 __host__ __device__ __forceinline__ void fx_point(const int64_t *w, const E *ex, const int (&st)[3], double *out) {
   const unsigned e0 = ex[0];
   unsigned ep[3][3], em[3][3], u[3], top = e0, low = e0 - 1u;
@@ -282,7 +283,9 @@ __host__ __device__ __forceinline__ void fx_point(const int64_t *w, const E *ex,
       const int64_t q = 2 * fx_shifted(w[0], v - e0);
       out[4 + k] = fx_return<5, CVT>(fx_div2(t1 * 16 - t2, v - u[k]) - q * 15, (v << 21) | FX_LOW);
     }
-    out[k] = fx_out<5>((p1 - m1) * 8 - (p2 - m2), (u[k] << 21) | FX_LOW);
+    const int64_t f = (p1 - m1) * 8 - (p2 - m2);
+    const unsigned unit = (u[k] << 21) | FX_LOW;
+    out[k] = FIRST_CVT ? fx_return<5, true>(f, unit) : fx_out<5>(f, unit);
     s3 += fx_shifted(w[3 * s], top - ep[k][2]) + fx_shifted(w[-3 * s], top - em[k][2]);
   }
   const int64_t y = x - 15 * fx_shifted(w[0], top - e0), r = s3 - x, v = y + (r >> 2);
