@@ -323,11 +323,12 @@ def _has_children(cfg, n):
 # ----------------------------------------------------------------------------
 # GB300 arm
 # ----------------------------------------------------------------------------
-def load_traffic(n_points, precision="fp64", mesh=False):
-    """DRAM bytes of one RK stage (all its launches) over n_points, from the
-    ncu capture of a single level in that precision recorded in
-    profiles/traffic.json, scaled by points; None for a refined mesh, for a
-    precision without a record, or once the kernel sources have changed."""
+def load_counters(precision="fp64", mesh=False):
+    """Counters of one RK stage (all its launches) per point, from the ncu
+    capture of a single level in that precision recorded in
+    profiles/traffic.json: DRAM bytes and FP64-pipe instructions; None for a
+    refined mesh, for a precision without a record, or once the kernel
+    sources have changed."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         d = json.load(open(path))
@@ -338,7 +339,16 @@ def load_traffic(n_points, precision="fp64", mesh=False):
     cap = d.get(precision, {})
     if not cap.get("points"):
         return None
-    return (cap["dram_bytes_read"] + cap["dram_bytes_write"]) * n_points / cap["points"]
+    out = {"bytes": (cap["dram_bytes_read"] + cap["dram_bytes_write"]) / cap["points"]}
+    if "fp64_pipe_instructions" in cap:
+        out["fp64_ops"] = cap["fp64_pipe_instructions"] * 32.0 / cap["points"]
+    return out
+
+
+def load_traffic(n_points, precision="fp64", mesh=False):
+    """DRAM bytes of one RK stage over n_points (load_counters), or None."""
+    c = load_counters(precision, mesh)
+    return c and c["bytes"] * n_points
 
 
 def bench_config(args):
@@ -562,11 +572,17 @@ def run_gb300(args):
     f64 = fl["fp64"] * cfg.n_points
     f32 = fl["fp32"] * cfg.n_points
     if args.precision == "fp64" or f32 == 0:
-        roof = {"bound": "alu", "achieved": f64 / t_stage / 1e12, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": f64 / t_stage / 1e12 / FP64_PEAK_TFLOPS, "traffic": load_traffic(cfg.n_points, args.precision, g.n_levels > 1),
+        # the FP64 pipe's own instructions (a slot counted as an FMA's two flops); without a record of them the
+        # operations of the formulas, stencil sums in integers counted as the FP64 operations they replace
+        counted = (load_counters("fp64", g.n_levels > 1) or {}).get("fp64_ops")
+        flops = 2.0 * counted * cfg.n_points if counted else f64
+        roof = {"bound": "alu", "achieved": flops / t_stage / 1e12, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
+                "frac": flops / t_stage / 1e12 / FP64_PEAK_TFLOPS,
+                "traffic": load_traffic(cfg.n_points, args.precision, g.n_levels > 1),
                 "kernel": "a quarter of the timed step: derivatives, RHS + RK stage and ghost cells (pair_kernel, or the "
-                          "derivative pass and algebra_kernel), a mesh's restriction included; stencil sums in "
-                          "integers count as the FP64 operations they replace",
+                          "derivative pass and algebra_kernel), a mesh's restriction included",
+                "counted": "FP64-pipe instructions (ncu), two flops each" if counted else
+                           "operations of the formulas, stencil sums in integers as the FP64 operations they replace",
                 "flops_per_point_stage": fl["fp64"], "units_per_launch": cfg.n_points,
                 "peak_source": "FP64 pipe: 152 SMs x 2 FMA/clk x 2 flop x 2070 MHz",
                 "peak_measured": peaks}

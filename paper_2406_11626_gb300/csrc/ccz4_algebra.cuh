@@ -557,7 +557,7 @@ __host__ __device__ __forceinline__ T sym_inverse(const T g[6], T ig[6]) {
 // use, which keeps the number of live values (and so register spills) low.
 // NB: the point's view of the derivative pass (DerView), or of a halo'd tile
 // (Nbhd and, on the host, its recording DerivTap).
-// What counts is its FP64 operations, about 1180 a point in the FP64 path: the
+// What counts is its FP64 operations, about 1135 a point in the FP64 path: the
 // pipe is 91 % busy with them (the last 100 saved took one RK4 step at 144^3 from
 // 30.4 to 28.5 ms).
 template <class D, class R, class Sink, class NB>
