@@ -136,8 +136,8 @@ _TORCH_ALLOCATOR = None   # the callbacks handed to the library, kept alive whil
 
 
 def use_torch_allocator(enable=True):
-    """Grids created from now on take their large buffers (state buffers,
-    halo tiles, mixed derivatives) from PyTorch's caching allocator on the
+    """Grids created from now on take their large buffers (state buffers, halo
+    tiles, mixed and other derivatives) from PyTorch's caching allocator on the
     current device (ccz4_set_allocator); enable=False restores cudaMalloc.
     Grids keep the allocator they were created with."""
     global _TORCH_ALLOCATOR
